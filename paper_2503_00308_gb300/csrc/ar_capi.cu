@@ -1543,7 +1543,8 @@ int ar_render_concrete(ar_scene *s, const ar_intrinsics *in, const ar_nominal_po
         RK(bin_pairs(ws, ws.boxes.as<PixBox>(), ws.keys.as<double>(), n, n, 1, ne, nent, TS, ntx, n_tiles, st, bo,
                      launches));
         if (launch_concrete_render(ws.recs.as<double>(), ws.boxes.as<PixBox>(), ws.segs.as<uint32_t>(),
-                                   ws.sege.as<uint32_t>(), bo.ent_ev, bo.ev_val, bo.ev_key, W, H, ntx, n_tiles, o, st))
+                                   ws.sege.as<uint32_t>(), bo.ent_ev, bo.ev_val, bo.ev_key, ws.cells.p, W, H, ntx, n_tiles,
+                                   o, st))
             return fail(AR_EDEVICE, "concrete render launch: %s", cudaGetErrorString(cudaGetLastError()));
     }
     return AR_OK;

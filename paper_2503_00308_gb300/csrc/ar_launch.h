@@ -91,8 +91,8 @@ int launch_concrete_prep(const float *uw, const double *Mw, const double *tau, c
                          const CallConst &cc, const void *pose, int TS, double *recs, PixBox *boxes, double *keys,
                          unsigned long long *counters, cudaStream_t st);
 int launch_concrete_render(const double *recs, const PixBox *boxes, const uint32_t *seg_start, const uint32_t *seg_end,
-                           const uint32_t *ent_ev, const uint32_t *ev_val, const uint64_t *ev_key, int W, int H,
-                           int ntx, int n_tiles, float *out, cudaStream_t st);
+                           const uint32_t *ent_ev, const uint32_t *ev_val, const uint64_t *ev_key, const void *pose,
+                           int W, int H, int ntx, int n_tiles, float *out, cudaStream_t st);
 int launch_scene_prep(const float *logscale, const float *quat, const float *opacity, int64_t n, double *Mw,
                       double *tau, cudaStream_t st);
 int launch_pose_prep(const float *uw_lo, const float *uw_hi, const double *Mw, int64_t n, const CallConst &cc,
