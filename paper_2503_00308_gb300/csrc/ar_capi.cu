@@ -66,9 +66,12 @@ int rec_width_m6();
 int rec_scalar_offset_m1();
 int rec_scalar_offset_m4();
 int rec_scalar_offset_m6();
-int launch_cell_prep_m1(const double *, const double *, const CallConst &, void *, cudaStream_t);
-int launch_cell_prep_m4(const double *, const double *, const CallConst &, void *, cudaStream_t);
-int launch_cell_prep_m6(const double *, const double *, const CallConst &, void *, cudaStream_t);
+int launch_call_prep_m1(const double *, const double *, const CallConst &, void *, const float *, const float *,
+                        const double *, double *, cudaStream_t);
+int launch_call_prep_m4(const double *, const double *, const CallConst &, void *, const float *, const float *,
+                        const double *, double *, cudaStream_t);
+int launch_call_prep_m6(const double *, const double *, const CallConst &, void *, const float *, const float *,
+                        const double *, double *, cudaStream_t);
 int launch_record_prep_m1(const double *, const void *, const CallConst &, const void *, int, float *, PixBox *,
                           double *, unsigned long long *, cudaStream_t, uint32_t *, uint32_t *);
 int launch_record_prep_m4(const double *, const void *, const CallConst &, const void *, int, float *, PixBox *,
@@ -120,10 +123,12 @@ static int rec_scalar_offset(int M)
 {
     return M == 1 ? rec_scalar_offset_m1() : (M == 4 ? rec_scalar_offset_m4() : rec_scalar_offset_m6());
 }
-int launch_cell_prep(int M, const double *lo, const double *hi, const CallConst &cc, void *cells, cudaStream_t st)
+int launch_call_prep(int M, const double *lo, const double *hi, const CallConst &cc, void *cells, const float *uw_lo,
+                     const float *uw_hi, const double *Mw, double *vN, cudaStream_t st)
 {
-    return M == 1 ? launch_cell_prep_m1(lo, hi, cc, cells, st)
-                  : (M == 4 ? launch_cell_prep_m4(lo, hi, cc, cells, st) : launch_cell_prep_m6(lo, hi, cc, cells, st));
+    if (M == 1) return launch_call_prep_m1(lo, hi, cc, cells, uw_lo, uw_hi, Mw, vN, st);
+    if (M == 4) return launch_call_prep_m4(lo, hi, cc, cells, uw_lo, uw_hi, Mw, vN, st);
+    return launch_call_prep_m6(lo, hi, cc, cells, uw_lo, uw_hi, Mw, vN, st);
 }
 int launch_record_prep(int M, const double *vN, const void *gp,
                        const CallConst &cc, const void *cells, int TS, float *recs, PixBox *boxes, double *keys,
@@ -680,7 +685,9 @@ static int render_batch(ar_scene *s, Workspace &ws, const CallConst &cc, int M, 
     const bool cull = !plain && (s->cull_force >= 0 ? s->cull_force == 1 : ws.cull_on);
     if (cull) RK(ws.clist.ensure(sizeof(uint32_t) * (n_pairs + 1)));
     NvtxRange prep_range("ar.prep: cells and (Gaussian, cell) decisions");
-    if (launch_cell_prep(M, d_lo, d_hi, cc, ws.cells.p, st)) return fail(AR_EDEVICE, "cell_prep launch");
+    if (launch_call_prep(M, d_lo, d_hi, cc, ws.cells.p, s->uw_lo, s->uw_hi, s->Mw,
+                         batch == 0 ? ws.vN.as<double>() : nullptr, st))
+        return fail(AR_EDEVICE, "call_prep launch");
     const int rp = plain ? launch_record_prep64(M, ws.vN.as<double>(), s->gp, cc, ws.cells.p, TS,
                                                 ws.recs.as<double>(), ws.boxes.as<PixBox>(), ws.keys.as<double>(),
                                                 ws.counters.as<unsigned long long>(), st)
@@ -1142,8 +1149,6 @@ int render_core(ar_scene *s, Workspace &ws, const ar_intrinsics *in, const ar_no
     CK(cudaMemsetAsync(ws.counters.as<unsigned long long>() + 8, 0, sizeof(unsigned long long) * kCountersPerBatch * max_batches, st));
     int launches = 0;
     NvtxRange call_range(plain ? "ar.render_abstract_plain_fp64" : "ar.render_abstract");
-    if (launch_pose_prep(s->uw_lo, s->uw_hi, s->Mw, s->n, cc, ws.vN.as<double>(), st)) return fail(AR_EDEVICE, "pose_prep launch");
-    ++launches;
     std::vector<std::pair<int, int>> batches;  // (first cell, cells)
     for (int c0 = 0; c0 < n_cells; c0 += (int)per_batch)
         batches.push_back({c0, (int)(c0 + per_batch <= n_cells ? per_batch : n_cells - c0)});
@@ -1574,8 +1579,7 @@ int ar_debug_records(ar_scene *s, const ar_intrinsics *in, const ar_nominal_pose
     CK(cudaMemcpy(ws.cells_lohi.p, lohi, sizeof lohi, cudaMemcpyHostToDevice));
     CK(cudaMemset(ws.counters.p, 0, sizeof(unsigned long long) * 8));
     const double *d_lo = ws.cells_lohi.as<double>(), *d_hi = d_lo + MAXV;
-    if (launch_pose_prep(s->uw_lo, s->uw_hi, s->Mw, s->n, cc, ws.vN.as<double>(), st) ||
-        launch_cell_prep(M, d_lo, d_hi, cc, ws.cells.p, st) ||
+    if (launch_call_prep(M, d_lo, d_hi, cc, ws.cells.p, s->uw_lo, s->uw_hi, s->Mw, ws.vN.as<double>(), st) ||
         (s->cull_force != 0 && ws.clist.ensure(sizeof(uint32_t) * (cc.n_gauss + 1)) != AR_OK) ||
         launch_record_prep(M, ws.vN.as<double>(), s->gp, cc, ws.cells.p, 16, ws.recs.as<float>(),
                            ws.boxes.as<PixBox>(), ws.keys.as<double>(), ws.counters.as<unsigned long long>(), st,

@@ -53,7 +53,9 @@ struct RenderLaunch {
 
 size_t cell_data_bytes(int M);
 int rec_width(int M);
-int launch_cell_prep(int M, const double *lo, const double *hi, const CallConst &cc, void *cells, cudaStream_t st);
+// the cells' forms, and (vN non-null) the Gaussians' v and N
+int launch_call_prep(int M, const double *lo, const double *hi, const CallConst &cc, void *cells, const float *uw_lo,
+                     const float *uw_hi, const double *Mw, double *vN, cudaStream_t st);
 // list, count (optional): cull the certain drops first and run the FP64
 // decision chain over the list of the other pairs (cull_kernel)
 int launch_record_prep(int M, const double *vN, const void *gp,
@@ -95,8 +97,6 @@ int launch_concrete_render(const double *recs, const PixBox *boxes, const uint32
                            int W, int H, int ntx, int n_tiles, float *out, cudaStream_t st);
 int launch_scene_prep(const float *logscale, const float *quat, const float *opacity, int64_t n, double *Mw,
                       double *tau, cudaStream_t st);
-int launch_pose_prep(const float *uw_lo, const float *uw_hi, const double *Mw, int64_t n, const CallConst &cc,
-                     double *vN, cudaStream_t st);
 int launch_gparam(const float *o_lo, const float *o_hi, const float *c_lo, const float *c_hi, int64_t n, void *gp,
                   cudaStream_t st);
 

@@ -3,9 +3,8 @@
 //
 //   scene_prep    : Mw = R(q) diag(exp(s)) and tau = 2 ln(255 o) per Gaussian
 //                   (the Gaussian tuple <uw, Mw, o, c> of Sec. 2.2).
-//   pose_prep     : v = R_wc (uw - t) and N = R_wc Mw per Gaussian for the
-//                   nominal camera of the call.
-//   cell_prep<M>  : linear forms of R_delta(theta) (first-order Taylor at the
+//   call_prep<M>  : v = R_wc (uw - t) and N = R_wc Mw per Gaussian for the
+//                   nominal camera of the call, and linear forms of R_delta(theta) (first-order Taylor at the
 //                   cell centre, remainder (1/2)(sum h_theta)^2) and of
 //                   s = R_wc delta_t, per cell.
 //   record_prep<M>: Algorithm 1 lines 2-8 with set-valued variables (Sec. 3.3)
@@ -64,82 +63,80 @@ __device__ __forceinline__ void rot3(int axis, double a, double R[9], double D[9
     }
 }
 
-// One thread per cell.
-template <int M>
-__global__ void cell_prep_kernel(const double *__restrict__ cells_lo, const double *__restrict__ cells_hi,
-                                 CallConst cc, CellData<M> *__restrict__ out)
-{
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= cc.n_cells) return;
-    CellData<M> &cd = out[c];
+// A cell's forms with the 32 lanes of a warp: every value is the one a single
+// thread computes (the same operations in the same order), each by a lane of its
+// own.  One thread took 57 us at six pose variables, a chain of a few thousand
+// FP64 operations that every render waited for.
+template <int M> struct CellScratch {
+    CellData<M> cd;
     double ctr[MAXV], h[MAXV];
-    for (int k = 0; k < MAXV; ++k) {
-        double lo = cells_lo[MAXV * c + k], hi = cells_hi[MAXV * c + k];
-        ctr[k] = dmul(0.5, dadd(lo, hi));
-        h[k] = dmul(0.5, dsub(hi, lo));
+    double rot[6][9];  // X, Y, Z, then their derivatives
+    double prod[3][9]; // X Y, dX Y, X dY
+    double R[4][9];    // R_delta = Rx Ry Rz at the centre and its partial derivatives
+};
+template <int M>
+__device__ __forceinline__ void cell_prep_warp(const double *__restrict__ lo6, const double *__restrict__ hi6,
+                                               const CallConst &cc, CellData<M> *__restrict__ out, CellScratch<M> &w,
+                                               int ln)
+{
+    CellData<M> &cd = w.cd;
+    if (ln < MAXV) {
+        const double lo = lo6[ln], hi = hi6[ln];
+        w.ctr[ln] = dmul(0.5, dadd(lo, hi));
+        w.h[ln] = dmul(0.5, dsub(hi, lo));
     }
-    // R_delta = Rx Ry Rz at the centre and its partial derivatives
-    double X[9], dX[9], Y[9], dY[9], Z[9], dZ[9], T[9], R[9], dR[3][9];
-    rot3(0, ctr[3], X, dX);
-    rot3(1, ctr[4], Y, dY);
-    rot3(2, ctr[5], Z, dZ);
-    mat3(X, Y, T); mat3(T, Z, R);
-    mat3(dX, Y, T); mat3(T, Z, dR[0]);
-    mat3(X, dY, T); mat3(T, Z, dR[1]);
-    mat3(X, Y, T); mat3(T, dZ, dR[2]);
-    double hs = dadd(dadd(h[3], h[4]), h[5]);
-    double rem = dmul(0.5, dmul(hs, hs));
-    for (int e = 0; e < 9; ++e) {
+    __syncwarp();
+    if (ln < 3) rot3(ln, w.ctr[3 + ln], w.rot[ln], w.rot[3 + ln]);
+    __syncwarp();
+    auto entry = [](const double *A, const double *B, int e) {  // of A B
+        const int i = e / 3, j = e - 3 * i;
+        double s = 0;
+        for (int k = 0; k < 3; ++k) s = dadd(s, dmul(A[3 * i + k], B[3 * k + j]));
+        return s;
+    };
+    if (ln < 27) {
+        const int p = ln / 9, e = ln - 9 * p;
+        w.prod[p][e] = entry(w.rot[p == 1 ? 3 : 0], w.rot[p == 2 ? 4 : 1], e);
+    }
+    __syncwarp();
+    for (int i = ln; i < 36; i += 32) {  // R, then dR[0..2]
+        const int p = i / 9, e = i - 9 * p;
+        w.R[p][e] = entry(w.prod[p < 3 ? p : 0], w.rot[p < 3 ? 2 : 5], e);
+    }
+    __syncwarp();
+    const double hs = dadd(dadd(w.h[3], w.h[4]), w.h[5]);
+    const double rem = dmul(0.5, dmul(hs, hs));
+    if (ln < 9) {
+        const int e = ln;
         for (int j = 0; j <= M; ++j) { cd.rd_lo[e][j] = 0; cd.rd_hi[e][j] = 0; }
         for (int k = 0; k < 3; ++k) {
-            int sl = cc.m_slot[3 + k];
-            if (sl >= 0) { double v = dmul(dR[k][e], h[3 + k]); cd.rd_lo[e][sl] = v; cd.rd_hi[e][sl] = v; }
+            const int sl = cc.m_slot[3 + k];
+            if (sl >= 0) { const double v = dmul(w.R[1 + k][e], w.h[3 + k]); cd.rd_lo[e][sl] = v; cd.rd_hi[e][sl] = v; }
         }
-        cd.rd_lo[e][M] = dsub(R[e], rem);
-        cd.rd_hi[e][M] = dadd(R[e], rem);
-    }
-    for (int a = 0; a < 3; ++a) {
+        cd.rd_lo[e][M] = dsub(w.R[0][e], rem);
+        cd.rd_hi[e][M] = dadd(w.R[0][e], rem);
+    } else if (ln < 12) {
+        const int a = ln - 9;
         for (int j = 0; j <= M; ++j) cd.s[a][j] = 0;
         double kk = 0;
         for (int k = 0; k < 3; ++k) {
-            int sl = cc.m_slot[k];
-            if (sl >= 0) cd.s[a][sl] = dmul(cc.R0[3 * a + k], h[k]);
-            kk = dadd(kk, dmul(cc.R0[3 * a + k], ctr[k]));
+            const int sl = cc.m_slot[k];
+            if (sl >= 0) cd.s[a][sl] = dmul(cc.R0[3 * a + k], w.h[k]);
+            kk = dadd(kk, dmul(cc.R0[3 * a + k], w.ctr[k]));
         }
         cd.s[a][M] = kk;
-    }
-    for (int j = 0; j < M; ++j) cd.g[j] = 0;
-    for (int k = 0; k < 3; ++k) {
-        double s = 0;
-        for (int b = 0; b < 3; ++b) s = dadd(s, dmul(R[3 * b + 2], cc.R0[3 * b + k]));
-        int sl = cc.m_slot[k];
-        if (sl >= 0) cd.g[sl] = dmul(-s, h[k]);
-    }
-    for (int e = 0; e < 9; ++e) {
-        DF<M> lo, hi;
-        for (int j = 0; j < M; ++j) { lo.c[j] = cd.rd_lo[e][j]; hi.c[j] = cd.rd_hi[e][j]; }
-        lo.k = cd.rd_lo[e][M]; hi.k = cd.rd_hi[e][M];
-        cd.rd_int[e][0] = df_min(lo);
-        cd.rd_int[e][1] = df_max(hi);
-    }
-    for (int a = 0; a < 3; ++a) {
-        DF<M> f;
-        for (int j = 0; j < M; ++j) f.c[j] = cd.s[a][j];
-        f.k = cd.s[a][M];
-        cd.s_int[a][0] = df_min(f);
-        cd.s_int[a][1] = df_max(f);
-    }
-    for (int e = 0; e < 9; ++e)
-        for (int t = 0; t < 2; ++t) {
-            cd.rd_int32[e][t][0] = __double2float_rd(cd.rd_int[e][t]);
-            cd.rd_int32[e][t][1] = __double2float_ru(cd.rd_int[e][t]);
-        }
-    for (int a = 0; a < 3; ++a)
-        for (int t = 0; t < 2; ++t) {
-            cd.s_int32[a][t][0] = __double2float_rd(cd.s_int[a][t]);
-            cd.s_int32[a][t][1] = __double2float_ru(cd.s_int[a][t]);
-        }
-    {
+    } else if (ln < 12 + M) {
+        // the depth-key offset of the slot's translation (0 on the others)
+        const int j = ln - 12;
+        double g = 0;
+        for (int k = 0; k < 3; ++k)
+            if (cc.m_slot[k] == j) {
+                double s = 0;
+                for (int b = 0; b < 3; ++b) s = dadd(s, dmul(w.R[0][3 * b + 2], cc.R0[3 * b + k]));
+                g = dmul(-s, w.h[k]);
+            }
+        cd.g[j] = g;
+    } else if (ln == 31) {
         const double gx = dmul(GUARD, (double)cc.W), gy = dmul(GUARD, (double)cc.H);
         const double gc[4] = {dadd((double)cc.cx, gx), dsub((double)cc.cx, gx), dadd((double)cc.cy, gy),
                               dsub((double)cc.cy, gy)};
@@ -149,12 +146,6 @@ __global__ void cell_prep_kernel(const double *__restrict__ cells_lo, const doub
         }
         cd.slack32[0] = __double2float_rd(BOX_SLACK);
         cd.slack32[1] = __double2float_ru(BOX_SLACK);
-    }
-    // per-cell parts of the depth chain (see record_decide): R_delta[b][2]
-    // has coefficients on the rotation slots only and s_b on the translation
-    // slots only, so the products xm * (-s_b) and their sums over b are the
-    // same for every Gaussian of the cell
-    {
         int nt = 0, na = 0;
         for (int k = 0; k < MAXV; ++k) {
             if (cc.m_slot[k] < 0) continue;
@@ -163,42 +154,38 @@ __global__ void cell_prep_kernel(const double *__restrict__ cells_lo, const doub
         }
         cd.n_t = nt;
         cd.n_a = na;
-        for (int j = 0; j < M; ++j) cd.dd_t[j] = 0.0;
-        for (int b = 0; b < 3; ++b) {
-            const int e = 3 * b + 2;
-            DF<M> lo, hi;
-            for (int j = 0; j < M; ++j) { lo.c[j] = cd.rd_lo[e][j]; hi.c[j] = cd.rd_hi[e][j]; }
-            lo.k = cd.rd_lo[e][M]; hi.k = cd.rd_hi[e][M];
-            const double xl = df_min(lo), xh = df_max(hi);
-            const double xm = dmul(0.5, dadd(xl, xh));
-            cd.dx[b][0] = xl; cd.dx[b][1] = xh; cd.dx[b][2] = xm;
-            for (int j = 0; j < nt; ++j) {
-                const double t = dmul(xm, dsub(0.0, cd.s[b][j]));
-                cd.dd_t[j] = b == 0 ? t : dadd(cd.dd_t[j], t);
-            }
-        }
-        for (int j = 0; j < M; ++j) cd.kd_t[j] = dsub(cd.dd_t[j], cd.g[j]);
-        auto enc = [](double x, float *o) {
-            o[0] = __double2float_rd(x);
-            o[1] = __double2float_ru(x);
-        };
-        for (int b = 0; b < 3; ++b) {
-            for (int k = 0; k < 3; ++k) enc(cd.dx[b][k], cd.dx32[b][k]);
-            for (int j = 0; j <= M; ++j) {
-                enc(cd.s[b][j], cd.s32[b][j]);
-                enc(cd.rd_lo[3 * b + 2][j], cd.rdd32[b][0][j]);
-                enc(cd.rd_hi[3 * b + 2][j], cd.rdd32[b][1][j]);
-            }
-        }
-        for (int j = 0; j < M; ++j) enc(cd.dd_t[j], cd.ddt32[j]);
     }
-    // FP64 value-chain copies, widened to cover the rounding of sin, cos and
-    // the Taylor terms (a relative 1e-14 is far above their few-ulp error);
-    // the lower and upper forms share their coefficients
-    for (int e = 0; e < 12; ++e) {
-        const double *lo = e < 9 ? cd.rd_lo[e] : cd.s[e - 9];
-        const double *hi = e < 9 ? cd.rd_hi[e] : cd.s[e - 9];
-        SB<M, double> &b = e < 9 ? cd.rd64[e] : cd.s64[e - 9];
+    __syncwarp();
+    auto enc = [](double x, float *o) {
+        o[0] = __double2float_rd(x);
+        o[1] = __double2float_ru(x);
+    };
+    if (ln < 12) {
+        // the concretised forms and their FP32 enclosures; then the FP64
+        // value-chain copies, widened to cover the rounding of sin, cos and
+        // the Taylor terms (a relative 1e-14 is far above their few-ulp error);
+        // the lower and upper forms share their coefficients
+        const double *lo = ln < 9 ? cd.rd_lo[ln] : cd.s[ln - 9];
+        const double *hi = ln < 9 ? cd.rd_hi[ln] : cd.s[ln - 9];
+        DF<M> fl, fh;
+        for (int j = 0; j < M; ++j) { fl.c[j] = lo[j]; fh.c[j] = hi[j]; }
+        fl.k = lo[M];
+        fh.k = hi[M];
+        const double xl = df_min(fl), xh = df_max(fh);
+        double *oi = ln < 9 ? cd.rd_int[ln] : cd.s_int[ln - 9];
+        float(*o32)[2] = ln < 9 ? cd.rd_int32[ln] : cd.s_int32[ln - 9];
+        oi[0] = xl;
+        oi[1] = xh;
+        enc(xl, o32[0]);
+        enc(xh, o32[1]);
+        if (ln < 9 && ln % 3 == 2) {  // R_delta[b][2], of the depth chain
+            const int b = ln / 3;
+            cd.dx[b][0] = xl;
+            cd.dx[b][1] = xh;
+            cd.dx[b][2] = dmul(0.5, dadd(xl, xh));
+            for (int k = 0; k < 3; ++k) enc(cd.dx[b][k], cd.dx32[b][k]);
+        }
+        SB<M, double> &b = ln < 9 ? cd.rd64[ln] : cd.s64[ln - 9];
         double mag = 1.0;
         for (int j = 0; j <= M; ++j) mag = __dadd_ru(mag, fmax(fabs(lo[j]), fabs(hi[j])));
         const double pad = __dmul_ru(1e-14, mag);
@@ -207,6 +194,96 @@ __global__ void cell_prep_kernel(const double *__restrict__ cells_lo, const doub
         b.khi = __dadd_ru(hi[M], pad);
         sb_finish(b);
     }
+    for (int i = ln; i < 3 * (M + 1); i += 32) {
+        const int b = i / (M + 1), j = i - b * (M + 1);
+        enc(cd.s[b][j], cd.s32[b][j]);
+        enc(cd.rd_lo[3 * b + 2][j], cd.rdd32[b][0][j]);
+        enc(cd.rd_hi[3 * b + 2][j], cd.rdd32[b][1][j]);
+    }
+    __syncwarp();
+    // per-cell parts of the depth chain (see record_decide): R_delta[b][2]
+    // has coefficients on the rotation slots only and s_b on the translation
+    // slots only, so the products xm * (-s_b) and their sums over b are the
+    // same for every Gaussian of the cell
+    if (ln < M) {
+        double t = 0.0;
+        if (ln < cd.n_t)
+            for (int b = 0; b < 3; ++b) {
+                const double u = dmul(cd.dx[b][2], dsub(0.0, cd.s[b][ln]));
+                t = b == 0 ? u : dadd(t, u);
+            }
+        cd.dd_t[ln] = t;
+        cd.kd_t[ln] = dsub(t, cd.g[ln]);
+        enc(t, cd.ddt32[ln]);
+    }
+    __syncwarp();
+    static_assert(sizeof(CellData<M>) % sizeof(double) == 0, "copied by doubles");
+    const double *src = reinterpret_cast<const double *>(&cd);
+    double *dst = reinterpret_cast<double *>(out);
+    for (int i = ln; i < (int)(sizeof(CellData<M>) / sizeof(double)); i += 32) dst[i] = src[i];
+}
+
+// v = R_wc (uw - t) as an interval over the mean's box [uw_lo, uw_hi] (each
+// product at the end of the box its sign selects; lo = hi without a box),
+// and N = R_wc Mw, for the call's nominal camera: VN_STRIDE doubles each.
+__device__ __forceinline__ void pose_prep_one(const float *__restrict__ uw_lo, const float *__restrict__ uw_hi,
+                                              const double *__restrict__ Mw, int64_t i, const CallConst &cc, double *o)
+{
+    for (int a = 0; a < 3; ++a) {
+        double sl = 0, sh = 0;
+        for (int b = 0; b < 3; ++b) {
+            const double r = cc.R0[3 * a + b];
+            const double dl = dsub((double)uw_lo[3 * i + b], cc.t0[b]);
+            if (uw_lo == uw_hi) {  // no box: both ends are the same sum
+                sl = dadd(sl, dmul(r, dl));
+                continue;
+            }
+            const double dh = dsub((double)uw_hi[3 * i + b], cc.t0[b]);
+            sl = dadd(sl, dmul(r, r >= 0 ? dl : dh));
+            sh = dadd(sh, dmul(r, r >= 0 ? dh : dl));
+        }
+        o[a] = sl;
+        o[3 + a] = uw_lo == uw_hi ? sl : sh;
+    }
+    mat3(cc.R0, Mw + 9 * i, o + 6);
+    float *enc = reinterpret_cast<float *>(o + VN_ENC);
+    for (int k = 0; k < VN_ENC; ++k) {
+        enc[2 * k] = __double2float_rd(o[k]);
+        enc[2 * k + 1] = __double2float_ru(o[k]);
+    }
+}
+
+// What a render computes before its records: the first cell_blocks blocks take
+// a cell per warp, the others 64 Gaussians each.  One launch, so that the
+// cells' short serial chains run beside the Gaussians.  The Gaussians' rows go
+// through shared memory (31 doubles apart: no two lanes on one bank) and out in
+// order; one thread per row wrote 240 bytes apart.  A whole render went from
+// 381 to 344 us (64 Gaussians, 1 cell), 1011 to 959 (10k) and 2133 to 2052
+// (300k at 1280 x 720).
+constexpr int CALL_PREP_T = 64;
+template <int M>
+__global__ void __launch_bounds__(CALL_PREP_T) call_prep_kernel(
+    const double *__restrict__ cells_lo, const double *__restrict__ cells_hi, CallConst cc,
+    CellData<M> *__restrict__ cells, unsigned cell_blocks, const float *__restrict__ uw_lo,
+    const float *__restrict__ uw_hi, const double *__restrict__ Mw, double *__restrict__ vN)
+{
+    constexpr int ROW = VN_STRIDE + 1;
+    __shared__ union {
+        CellScratch<M> cell[CALL_PREP_T / 32];
+        double row[CALL_PREP_T * ROW];
+    } sm;
+    if (blockIdx.x < cell_blocks) {
+        const int w = threadIdx.x >> 5, c = (int)blockIdx.x * (CALL_PREP_T / 32) + w;
+        if (c < cc.n_cells)
+            cell_prep_warp<M>(cells_lo + MAXV * c, cells_hi + MAXV * c, cc, cells + c, sm.cell[w], threadIdx.x & 31);
+        return;
+    }
+    const int64_t g0 = (int64_t)(blockIdx.x - cell_blocks) * CALL_PREP_T;
+    const int n = (int)min((int64_t)CALL_PREP_T, cc.n_gauss - g0);
+    if ((int)threadIdx.x < n) pose_prep_one(uw_lo, uw_hi, Mw, g0 + threadIdx.x, cc, sm.row + threadIdx.x * ROW);
+    __syncthreads();
+    double *dst = vN + g0 * VN_STRIDE;
+    for (int i = threadIdx.x; i < n * VN_STRIDE; i += CALL_PREP_T) dst[i] = sm.row[i + i / VN_STRIDE];
 }
 
 // FP32 form -> FP64 (exact); an FP64 form passes through

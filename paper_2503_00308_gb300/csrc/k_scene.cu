@@ -1,4 +1,4 @@
-// k_scene.cu -- per-scene and per-call preprocessing of the Gaussians.
+// k_scene.cu -- per-scene preprocessing of the Gaussians.
 #include "ar_launch.h"
 #include "k_prep.cuh"
 
@@ -19,34 +19,6 @@ __global__ void scene_prep_kernel(const float *__restrict__ logscale, const floa
         for (int b = 0; b < 3; ++b) Mw[9 * i + 3 * a + b] = dmul(R[3 * a + b], e[b]);
     double o = opacity[i];
     tau[i] = (o > 0) ? dmul(2.0, log(dmul(255.0, o))) : -INFINITY;
-}
-
-// v = R_wc (uw - t) as an interval over the mean's box [uw_lo, uw_hi] (each
-// product at the end of the box its sign selects; lo = hi without a box),
-// and N = R_wc Mw, for the call's nominal camera: VN_STRIDE doubles each.
-__global__ void pose_prep_kernel(const float *__restrict__ uw_lo, const float *__restrict__ uw_hi,
-                                 const double *__restrict__ Mw, int64_t n, CallConst cc, double *__restrict__ vN)
-{
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double *o = vN + VN_STRIDE * i;
-    for (int a = 0; a < 3; ++a) {
-        double sl = 0, sh = 0;
-        for (int b = 0; b < 3; ++b) {
-            const double r = cc.R0[3 * a + b];
-            const double dl = dsub((double)uw_lo[3 * i + b], cc.t0[b]), dh = dsub((double)uw_hi[3 * i + b], cc.t0[b]);
-            sl = dadd(sl, dmul(r, r >= 0 ? dl : dh));
-            sh = dadd(sh, dmul(r, r >= 0 ? dh : dl));
-        }
-        o[a] = sl;
-        o[3 + a] = sh;
-    }
-    mat3(cc.R0, Mw + 9 * i, o + 6);
-    float *enc = reinterpret_cast<float *>(o + VN_ENC);
-    for (int k = 0; k < VN_ENC; ++k) {
-        enc[2 * k] = __double2float_rd(o[k]);
-        enc[2 * k + 1] = __double2float_ru(o[k]);
-    }
 }
 
 // The GParam of every Gaussian from its opacity and colour boxes.
@@ -75,15 +47,6 @@ int launch_scene_prep(const float *logscale, const float *quat, const float *opa
     if (n <= 0) return 0;
     const int T = 128;
     scene_prep_kernel<<<(unsigned)((n + T - 1) / T), T, 0, st>>>(logscale, quat, opacity, n, Mw, tau);
-    return cudaGetLastError() == cudaSuccess ? 0 : 1;
-}
-
-int launch_pose_prep(const float *uw_lo, const float *uw_hi, const double *Mw, int64_t n, const CallConst &cc,
-                     double *vN, cudaStream_t st)
-{
-    if (n <= 0) return 0;
-    const int T = 128;
-    pose_prep_kernel<<<(unsigned)((n + T - 1) / T), T, 0, st>>>(uw_lo, uw_hi, Mw, n, cc, vN);
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
 
