@@ -81,8 +81,8 @@ struct TunedTile {
 // demand -> build -> render per round, windows w0, 8192, then unlimited.
 // state [n_pairs] (zeroed here), wlist [n_pairs], act0/act1 [n_seg], words [8];
 // build_counters: [0] fallbacks, [1] records built, [2] splits (optional);
-// split_list [n_pairs]: pairs whose MatrixInv needs input splitting, which a
-// second kernel finishes with a warp each; precise_list [n_seg]: segments that
+// split_list [n_pairs]: pairs whose MatrixInv needs input splitting or a high
+// order, which a last kernel finishes; precise_list [n_seg]: segments that
 // meet an opacity evaluation needing FP64, swept again by the FP64-capable
 // render instance in the same round, and precise_mask [n_seg * TS * TS / 32]
 // the pixels of each that do.

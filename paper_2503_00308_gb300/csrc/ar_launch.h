@@ -79,8 +79,8 @@ int launch_width_partials(const float *lo, const float *hi, int n_cells, size_t 
                           cudaStream_t st);
 // value parts of the records listed in work[0, *count); counters: [0] fallbacks, [1] built, [2] split.
 // split_list (list_cap >= *count entries), split_count and khigh_count (zeroed by the caller): pairs whose
-// MatrixInv fails on the cell are split by a warp each in a second kernel, pairs whose Taylor order exceeds
-// the default are finished in a third (listed from the back of split_list).
+// MatrixInv fails on the cell, and from the back pairs whose Taylor order exceeds the default, which a last
+// kernel finishes.
 int launch_record_build(int M, const double *vN, const CallConst &cc, const void *cells, int64_t n_gauss,
                         const uint32_t *work, const uint32_t *count, float *recs, unsigned long long *counters,
                         uint32_t *split_list, uint32_t *split_count, uint32_t list_cap, uint32_t *khigh_count,

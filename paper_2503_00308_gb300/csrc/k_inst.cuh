@@ -124,23 +124,33 @@ int AR_CAT(launch_record_build_m, AR_M)(const double *vN, const CallConst &cc, c
                                         unsigned long long *counters, uint32_t *split_list, uint32_t *split_count,
                                         uint32_t list_cap, uint32_t *khigh_count, cudaStream_t st)
 {
-    auto kern = record_build_kernel<AR_M>;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const CellData<AR_M> *cd = (const CellData<AR_M> *)cells;
+    // the list's length is on the device: a short list is the group builder's,
+    // a long one the one-thread builder's
+    auto coop = record_build_coop_kernel<AR_M>;
+    const int coop_smem = (int)sizeof(double) * (COOP_T / 4) * Coop<AR_M>::STRIDE;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, coop, COOP_T, coop_smem) != cudaSuccess || per_sm < 1)
+        per_sm = 1;
+    const int coop_most = (int)(COOP_MAX / (COOP_T / 4));
+    coop<<<sms * per_sm < coop_most ? sms * per_sm : coop_most, COOP_T, coop_smem, st>>>(
+        vN, cc.fx, cc.fy, cc.cx, cc.cy, cd, n_gauss, work, count, recs, counters, split_list, split_count);
+    if (cudaGetLastError() != cudaSuccess) return 1;
+    auto kern = record_build_kernel<AR_M>;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 128, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
-    kern<<<sms * per_sm, 128, 0, st>>>(vN, cc.fx, cc.fy, cc.cx, cc.cy, (const CellData<AR_M> *)cells, n_gauss, work,
-                                       count, recs, counters, split_list, split_count, list_cap, khigh_count);
+    kern<<<sms * per_sm, 128, 0, st>>>(vN, cc.fx, cc.fy, cc.cx, cc.cy, cd, n_gauss, work, count, recs, counters,
+                                       split_list, split_count, list_cap, khigh_count);
     if (cudaGetLastError() != cudaSuccess) return 1;
-    // the deferred pairs (the counts stay on the device): splits one warp
-    // each, high orders one thread each, grid-stride
-    split_build_kernel<AR_M><<<sms, 128, 0, st>>>(vN, cc.fx, cc.fy, cc.cx, cc.cy, (const CellData<AR_M> *)cells,
-                                                 n_gauss, split_list, split_count, recs, counters);
-    if (cudaGetLastError() != cudaSuccess) return 1;
-    auto kh = khigh_build_kernel<AR_M>;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kh, 128, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
-    kh<<<sms * per_sm, 128, 0, st>>>(vN, cc.fx, cc.fy, cc.cx, cc.cy, (const CellData<AR_M> *)cells, n_gauss,
-                                     split_list, list_cap, khigh_count, recs, counters);
+    // the deferred pairs (the counts stay on the device)
+    auto fin = finish_build_kernel<AR_M>;
+    const int fin_smem = (int)sizeof(double) * FINISH_GROUPS * Coop<AR_M>::STRIDE;
+    if (cudaFuncSetAttribute(fin, cudaFuncAttributeMaxDynamicSharedMemorySize, fin_smem) != cudaSuccess) return 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fin, FINISH_T, fin_smem) != cudaSuccess || per_sm < 1)
+        per_sm = 1;
+    fin<<<sms * per_sm, FINISH_T, fin_smem, st>>>(vN, cc.fx, cc.fy, cc.cx, cc.cy, cd, n_gauss, split_list, split_count,
+                                                  list_cap, khigh_count, recs, counters);
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
 

@@ -941,9 +941,9 @@ __device__ __noinline__ int matinv_split(const SB<M, double> X[4], SB<M, double>
 }
 
 // Split modes of record_value (see there).
-enum { SPLIT_INLINE = 0, SPLIT_DEFER = 1, SPLIT_WARP = 2 };
+enum { SPLIT_INLINE = 0, SPLIT_DEFER = 1 };
 
-// A piece of the pose cell for matinv_split_warp, packed in 64 bits: for each
+// A piece of the pose cell (finish_build_kernel), packed in 64 bits: for each
 // slot j, bits 9j..9j+2 hold its bisection depth d_j and bits 9j+3..9j+8 its
 // index i_j, the piece being ctr_j = (2 i_j + 1) 2^-d_j - 1, h_j = 2^-d_j
 // (exact dyadic numbers, the same as repeated halving gives).
@@ -965,85 +965,6 @@ __device__ __forceinline__ void piece_box(uint64_t pc, double *ctr, double *h)
     }
 }
 
-// matinv_split with the 32 lanes of a warp, for a pair on whose cell
-// MatrixInv failed: the same pieces (each failing piece bisected along its
-// own split_var, down to SPLIT_DEPTH), tried level by level with one piece
-// per lane; the hull and the outcome do not depend on the order.  Every lane
-// passes the same X and gets the same result; list is the warp's 2 x 64
-// shared-memory piece lists.  Returns the number of pieces, or 0 if a piece
-// at the depth limit still fails.
-template <int M, class RS>
-__device__ __noinline__ int matinv_split_warp(const SB<M, double> X[4], SB<M, double> conic[4], uint64_t *list)
-{
-    const int lane = threadIdx.x & 31;
-    const unsigned full = 0xffffffffu;
-    double lo[4], hi[4];
-    for (int e = 0; e < 4; ++e) {
-        lo[e] = Num<double>::BIG;
-        hi[e] = -Num<double>::BIG;
-    }
-    int pieces = 0;
-    bool failed = false;
-    {
-        const int js = split_var<M>(X);
-        if (lane == 0) {
-            list[0] = piece_child(0, js, 0);
-            list[1] = piece_child(0, js, 1);
-        }
-    }
-    __syncwarp();
-    int cnt = 2, cur = 0;
-    for (int depth = 1; depth <= SPLIT_DEPTH && cnt > 0; ++depth) {
-        int next = 0;
-        for (int base = 0; base < cnt; base += 32) {
-            const int i = base + lane;
-            bool need = false;
-            uint64_t pc = 0;
-            int js = 0;
-            if (i < cnt) {
-                pc = list[cur * 64 + i];
-                double ctr[M], h[M];
-                piece_box<M>(pc, ctr, h);
-                SB<M, double> Xr[4];
-                for (int e = 0; e < 4; ++e) Xr[e] = sb_restrict<M>(X[e], ctr, h);
-                SB<M, double> C[4];
-                if (matinv_box<M, RS>(Xr, C) == MI_OK) {
-                    for (int e = 0; e < 4; ++e) {
-                        lo[e] = fmin(lo[e], C[e].vlo);
-                        hi[e] = fmax(hi[e], C[e].vhi);
-                    }
-                    ++pieces;
-                } else if (depth < SPLIT_DEPTH) {
-                    need = true;
-                    js = split_var<M>(Xr);
-                } else {
-                    failed = true;
-                }
-            }
-            const unsigned m = __ballot_sync(full, need);
-            if (need) {
-                const int at = next + 2 * __popc(m & ((1u << lane) - 1u));
-                list[(cur ^ 1) * 64 + at] = piece_child(pc, js, 0);
-                list[(cur ^ 1) * 64 + at + 1] = piece_child(pc, js, 1);
-            }
-            next += 2 * __popc(m);
-        }
-        __syncwarp();
-        if (__any_sync(full, failed)) return 0;
-        cnt = next;
-        cur ^= 1;
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-        pieces += __shfl_xor_sync(full, pieces, off);
-        for (int e = 0; e < 4; ++e) {
-            lo[e] = fmin(lo[e], __shfl_xor_sync(full, lo[e], off));
-            hi[e] = fmax(hi[e], __shfl_xor_sync(full, hi[e], off));
-        }
-    }
-    for (int e = 0; e < 4; ++e) conic[e] = sb_cst<M, double>(lo[e], hi[e]);
-    return pieces;
-}
-
 // The value part of one (Gaussian, cell) pair: the forms the per-pixel stage
 // reads, S = d^2 and R = mu S - P (Algorithm 1 lines 2-8 with set-valued
 // variables), MatrixInv (Algorithm 3) and W = Conic Mp.  v points at the
@@ -1053,13 +974,10 @@ __device__ __noinline__ int matinv_split_warp(const SB<M, double> X[4], SB<M, do
 // finite) and returns that word.  SPLIT: where MatrixInv fails on the cell,
 // SPLIT_INLINE splits it in this thread (matinv_split), SPLIT_DEFER returns
 // the flags with F_SPLIT_PENDING before writing W and the flags (and with
-// F_KHIGH_PENDING where the cell's Taylor order would exceed KTAYLOR), and
-// SPLIT_WARP (all 32 lanes of a warp call it for one deferred pair, with the
-// warp's split_list) splits it with the warp (matinv_split_warp).
+// F_KHIGH_PENDING where the cell's Taylor order would exceed KTAYLOR).
 template <int M, class RO = float, int SPLIT = SPLIT_INLINE>
 __device__ __forceinline__ uint32_t record_value(const double *__restrict__ v, float fx, float fy, float cx, float cy,
-                                                 const CellData<M> &cd, RO mux, RO muy, uint32_t flags, RO *rec,
-                                                 uint64_t *split_list = nullptr)
+                                                 const CellData<M> &cd, RO mux, RO muy, uint32_t flags, RO *rec)
 {
     using RL = Rec<M>;
     using NO = Num<RO>;
@@ -1155,20 +1073,14 @@ __device__ __forceinline__ uint32_t record_value(const double *__restrict__ v, f
             p.init(0.0, 0.0); p.mul(Mp64[0], Mp64[3]); p.mul(Mp64[1], Mp64[4]); p.mul(Mp64[2], Mp64[5]); X[1] = p.result();
             X[2] = X[1];
         }
-        if (SPLIT == SPLIT_WARP) {
-            // a deferred pair (MatrixInv failed on its cell): the warp splits it
-            if (matinv_split_warp<M, RO>(X, conic, split_list) > 0) flags |= F_SPLIT;
+        // deferring: a pair whose order would exceed the default goes to a
+        // pass of its own, so that warps do not wait on a few long series
+        const int mi = matinv_box<M, RO, SPLIT == SPLIT_DEFER ? KTAYLOR : KMAX>(X, conic);
+        if (SPLIT == SPLIT_DEFER && mi == MI_KHIGH) return flags | F_KHIGH_PENDING;
+        if (mi == MI_FAIL) {
+            if (SPLIT == SPLIT_DEFER) return flags | F_SPLIT_PENDING;
+            if (matinv_split<M, RO>(X, conic) > 0) flags |= F_SPLIT;
             else fallback = true;
-        } else {
-            // deferring: a pair whose order would exceed the default goes to a
-            // pass of its own, so that warps do not wait on a few long series
-            const int mi = matinv_box<M, RO, SPLIT == SPLIT_DEFER ? KTAYLOR : KMAX>(X, conic);
-            if (SPLIT == SPLIT_DEFER && mi == MI_KHIGH) return flags | F_KHIGH_PENDING;
-            if (mi == MI_FAIL) {
-                if (SPLIT == SPLIT_DEFER) return flags | F_SPLIT_PENDING;
-                if (matinv_split<M, RO>(X, conic) > 0) flags |= F_SPLIT;
-                else fallback = true;
-            }
         }
         if (!fallback)
             for (int e = 0; e < 4; ++e)
@@ -1326,16 +1238,355 @@ __global__ void __launch_bounds__(128, 5) record_prep_list_kernel(
     }
 }
 
+// ------------------------------------------------- records by groups of lanes
+// The value chain of record_value with four lanes to a record.  One thread's
+// chain is a few thousand FP64 operations over a code of many kilobytes: with
+// few records (a small call, a pair that MatrixInv splits) the device waits on
+// that one chain and on the fetching of its code.  Four lanes compute one
+// entry each (of uc, Mc, Mp, X, E, the series, Conic and W), every entry by the
+// operations record_value gives it, so the record is the same bit for bit, in a
+// third of the time and of the code; but per record it takes twice the FP64
+// issue slots (9 entries of Mc on 4 lanes, 3 of X), so lists longer than
+// COOP_MAX go to the one-thread builder.  Both over the same lists (the build
+// stage, in us, groups / threads): 64 records 78 / 115, 1000 180 / 244, 3946
+// 198 / 259, 18291 377 / 398, 27693 459 / 404, 76970 941 / 683.
+constexpr uint32_t COOP_MAX = 20480;
+
+// Forms of a group in shared memory, COOP_FORM<M> doubles each: c[M], klo, khi,
+// r, vlo, vhi.  (v - s takes the slots of X, Conic those of J.)
+template <int M> struct Coop {
+    static constexpr int FORM = M + 5;
+    static constexpr int UC = 0, MC = 3, MP = 12, J = 18, X = 22, FORMS = 25;
+    static constexpr int STRIDE = (FORMS * FORM) | 1;  // doubles per group
+};
+template <int M> __device__ __forceinline__ SB<M, double> ld_form(const double *s, int slot)
+{
+    SB<M, double> b;
+    s += slot * Coop<M>::FORM;
+#pragma unroll
+    for (int j = 0; j < M; ++j) b.c[j] = s[j];
+    b.klo = s[M];
+    b.khi = s[M + 1];
+    b.r = s[M + 2];
+    b.vlo = s[M + 3];
+    b.vhi = s[M + 4];
+    return b;
+}
+template <int M> __device__ __forceinline__ void st_form(double *s, int slot, const SB<M, double> &b)
+{
+    s += slot * Coop<M>::FORM;
+#pragma unroll
+    for (int j = 0; j < M; ++j) s[j] = b.c[j];
+    s[M] = b.klo;
+    s[M + 1] = b.khi;
+    s[M + 2] = b.r;
+    s[M + 3] = b.vlo;
+    s[M + 4] = b.vhi;
+}
+
+// record_value up to X (kept in s with Mp), lane q of the group; stores the S
+// and R entries of rec (store).  Returns whether this lane's entry is finite.
+// Every lane of the warp calls it.
+template <int M>
+__device__ __forceinline__ bool coop_chain(double *s, int q, const double *__restrict__ v, float fx, float fy, float cx,
+                                           float cy, const CellData<M> &cd, float mux, float muy, float *rec, bool store)
+{
+    using RL = Rec<M>;
+    using G = Coop<M>;
+    typedef SB<M, double> BD;
+    typedef SAcc<M, double> AD;
+    const double *N = v + 6;
+    AD p;
+    {
+        double vabs = 1.0;
+        for (int b = 0; b < 3; ++b) vabs += fmax(fabs(v[b]), fabs(v[3 + b]));
+        const double ev = __dmul_ru(1e-14, vabs);
+        if (q < 3) {
+            p.init(__dsub_rd(v[q], ev), __dadd_ru(v[3 + q], ev));
+            p.term(-1.0, cd.s64[q]);
+            st_form<M>(s, G::X + q, p.result());
+        }
+    }
+    __syncwarp();
+    if (q < 3) {
+        p.init(0.0, 0.0);
+#pragma unroll 1
+        for (int b = 0; b < 3; ++b) p.mul(cd.rd64[3 * b + q], ld_form<M>(s, G::X + b));
+        st_form<M>(s, G::UC + q, p.result());
+    }
+    __syncwarp();
+    bool fin = true;
+    {
+        // lanes 0, 1: R_x, R_y = mu S - P; lane 2: S (see record_value)
+        const BD d64 = ld_form<M>(s, G::UC + 2);
+        const BD S = sb_sqr<M, double>(d64);
+        const int a = q & 1;
+        p.init(0.0, 0.0);
+        p.term((double)(a ? fy : fx), ld_form<M>(s, G::UC + a));
+        p.term((double)(a ? cy : cx), d64);
+        const BD P = sb_mul<M, double>(d64, p.result());
+        p.init(0.0, 0.0);
+        p.term_same_side((double)(a ? muy : mux), S);
+        p.term(-1.0, P);
+        const BD R = p.result();
+        BD F = S;
+        if (q < 2) F = R;
+        SB<M, float> f32;
+        const double gap = sb_to_f32<M>(F, f32);
+        fin = sb_finite(f32);
+        if (store && q < 3) store_sb<M>(rec + (q == 0 ? RL::RX : q == 1 ? RL::RY : RL::S), f32);
+        if (store && q == 2) rec_up(gap, rec[RL::GAP_S]);
+    }
+#pragma unroll 1
+    for (int i = q; i < 9; i += 4) {
+        const int a = i / 3, c = i - 3 * a;
+        p.init(0.0, 0.0);
+        p.term(N[c], cd.rd64[a]);
+        p.term(N[3 + c], cd.rd64[3 + a]);
+        p.term(N[6 + c], cd.rd64[6 + a]);
+        st_form<M>(s, G::MC + i, p.result());
+    }
+    // J00, J02, J11, J12
+    p.init(0.0, 0.0);
+    p.term((q & 1) ? -(double)(q < 2 ? fx : fy) : (double)(q < 2 ? fx : fy), ld_form<M>(s, G::UC + ((q & 1) ? q >> 1 : 2)));
+    st_form<M>(s, G::J + q, p.result());
+    __syncwarp();
+#pragma unroll 1
+    for (int i = q; i < 6; i += 4) {
+        const int r = i / 3, c = i - 3 * r;
+        p.init(0.0, 0.0);
+        p.mul(ld_form<M>(s, G::J + 2 * r), ld_form<M>(s, G::MC + 3 * r + c));
+        p.mul(ld_form<M>(s, G::J + 2 * r + 1), ld_form<M>(s, G::MC + 6 + c));
+        st_form<M>(s, G::MP + i, p.result());
+    }
+    __syncwarp();
+    // X00, X01, X11
+    p.init(0.0, 0.0);
+    if (q == 1) {
+#pragma unroll 1
+        for (int c = 0; c < 3; ++c) p.mul(ld_form<M>(s, G::MP + c), ld_form<M>(s, G::MP + 3 + c));
+    } else if (q != 3) {
+#pragma unroll 1
+        for (int c = 0; c < 3; ++c) p.sqr(ld_form<M>(s, G::MP + (q ? 3 : 0) + c));
+    }
+    if (q < 3) st_form<M>(s, G::X + q, p.result());
+    __syncwarp();
+    return fin;
+}
+
+// a form of another lane (the concretisation follows from the rest)
+template <int M> __device__ __forceinline__ SB<M, float> shfl_form(const SB<M, float> &b, int lane_xor)
+{
+    SB<M, float> o;
+#pragma unroll
+    for (int j = 0; j < M; ++j) o.c[j] = __shfl_xor_sync(0xffffffffu, b.c[j], lane_xor);
+    o.klo = __shfl_xor_sync(0xffffffffu, b.klo, lane_xor);
+    o.khi = __shfl_xor_sync(0xffffffffu, b.khi, lane_xor);
+    o.r = __shfl_xor_sync(0xffffffffu, b.r, lane_xor);
+    o.vlo = __fsub_rd(o.klo, o.r);
+    o.vhi = __fadd_ru(o.khi, o.r);
+    return o;
+}
+
+// matinv_box<M, float> by a group: lane q = 2 r + c passes XA = X[r][0] and XB =
+// X[r][1] and gets Conic[r][c].  Returns false in all four lanes where the
+// assertion of Algorithm 3 fails (conic is then undefined).  Every lane of the
+// warp calls it.
+template <int M>
+__device__ __forceinline__ bool coop_matinv(const SB<M, double> &XA, const SB<M, double> &XB, int q, SB<M, double> &conic)
+{
+    typedef SB<M, float> B;
+    typedef SAcc<M, double> AD;
+    constexpr unsigned FULL = 0xffffffffu;
+    const int g0 = (threadIdx.x & 31) & ~3, r = q >> 1, c = q & 1;
+    const double ha = 0.5 * (XA.vlo + XA.vhi), hb = 0.5 * (XB.vlo + XB.vhi);
+    const double h00 = __shfl_sync(FULL, ha, g0), h01 = __shfl_sync(FULL, hb, g0), h11 = __shfl_sync(FULL, hb, g0 + 2);
+    const double det = h00 * h11 - h01 * h01;
+    bool good = det > 0.0 && h00 > 0.0 && isfinite(det);
+    const double x0 = (q == 0 ? h11 : q == 3 ? h00 : -h01) / det;
+    double X0[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) X0[e] = __shfl_sync(FULL, x0, g0 + e);
+    B E;
+    double rho2 = 0.0;
+    {
+        AD p;
+        const double dl = (r == c) ? 1.0 : 0.0;
+        p.init(dl, dl);
+        p.term(-(c ? X0[1] : X0[0]), XA);
+        p.term(-(c ? X0[3] : X0[2]), XB);
+        const SB<M, double> e64 = p.result();
+        const double m = fmax(fabs(e64.vlo), fabs(e64.vhi));
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const double me = __shfl_sync(FULL, m, g0 + e);
+            rho2 = __fma_ru(me, me, rho2);
+        }
+        sb_to_f32<M>(e64, E);
+    }
+    const double rho64 = __dsqrt_ru(rho2);
+    good = good && rho64 < RHO_MAX;
+    int k = KTAYLOR;
+    if (good) {
+        double rk = 1.0;  // rho^(k+1), for the adaptive order
+        for (int i = 0; i <= KTAYLOR; ++i) rk *= rho64;
+        while (k < KMAX && rk / (1.0 - rho64) > EPS_TOL) {
+            rk *= rho64;
+            ++k;
+        }
+    }
+    const int kw = __reduce_max_sync(FULL, k);
+    B P = E, T = E;
+    // column c of E
+    B E1 = shfl_form<M>(E, 2), E2 = E;
+    if (r == 0) {
+        const B t = E1;
+        E1 = E2;
+        E2 = t;
+    }
+#pragma unroll 1
+    for (int i = 2; i <= kw; ++i) {
+        B A = shfl_form<M>(P, 1), Bq = P;  // row r of the power
+        if (c == 0) {
+            const B t = A;
+            A = Bq;
+            Bq = t;
+        }
+        SAcc<M, float> p;
+        p.init(0, 0);
+        p.mul(A, E1);
+        p.mul(Bq, E2);
+        const B Q = p.result();
+        if (i <= k) {
+            P = Q;
+            T = sb_add<M, float>(T, Q);
+        }
+    }
+    B T1 = shfl_form<M>(T, 2), T2 = T;  // column c of the sum
+    if (r == 0) {
+        const B t = T1;
+        T1 = T2;
+        T2 = t;
+    }
+    double nX0 = 0.0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) nX0 = __fma_ru(X0[e], X0[e], nX0);
+    nX0 = __dsqrt_ru(nX0);
+    double rk = 1.0;
+    for (int i = 0; i <= k; ++i) rk = __dmul_ru(rk, rho64);
+    const double eps = __ddiv_ru(__dmul_ru(nX0, rk), __dsub_rd(1.0, rho64));
+    AD p;
+    p.init(__dsub_rd(x0, eps), __dadd_ru(x0, eps));
+    p.term(r ? X0[2] : X0[0], to_f64<M>(T1));
+    p.term(r ? X0[3] : X0[1], to_f64<M>(T2));
+    conic = p.result();
+    return good;
+}
+
+// W = Conic Mp of a group (Conic in the slots of J), stored to rec; returns
+// whether this lane's entries are finite.
+template <int M> __device__ __forceinline__ bool coop_w(const double *s, int q, float *rec, bool store)
+{
+    using G = Coop<M>;
+    bool fin = true;
+#pragma unroll 1
+    for (int i = q; i < 6; i += 4) {
+        const int r = i / 3, c = i - 3 * r;
+        SAcc<M, double> p;
+        p.init(0.0, 0.0);
+        p.mul(ld_form<M>(s, G::J + 2 * r), ld_form<M>(s, G::MP + c));
+        p.mul(ld_form<M>(s, G::J + 2 * r + 1), ld_form<M>(s, G::MP + 3 + c));
+        SB<M, float> w;
+        sb_to_f32<M>(p.result(), w);
+        fin = fin && sb_finite(w);
+        if (store) store_sbw<M>(rec + Rec<M>::W0 + i * Rec<M>::WS, w);
+    }
+    return fin;
+}
+
+// whether f holds in all four lanes of this lane's group (every lane of the warp calls it)
+__device__ __forceinline__ bool group_all(bool f)
+{
+    const uint32_t m = __ballot_sync(0xffffffffu, f);
+    return ((m >> ((threadIdx.x & 31) & ~3)) & 15u) == 15u;
+}
+
+// One record by a group, from its decision part to the flags word, which is
+// returned; a record whose MatrixInv fails on the cell returns with
+// F_SPLIT_PENDING, its flags not stored.  act = false: a group without a record
+// (it computes along and stores nothing).
+template <int M>
+__device__ __forceinline__ uint32_t coop_record(double *s, int q, const double *__restrict__ v, float fx, float fy,
+                                                float cx, float cy, const CellData<M> &cd, float *rec, bool act)
+{
+    using RL = Rec<M>;
+    using G = Coop<M>;
+    uint32_t flags = __float_as_uint(rec[RL::FLAGS]);
+    const bool ok = group_all(coop_chain<M>(s, q, v, fx, fy, cx, cy, cd, rec[RL::MU_X], rec[RL::MU_Y], rec, act));
+    SB<M, double> conic;
+    const bool inv = coop_matinv<M>(ld_form<M>(s, G::X + (q >> 1)), ld_form<M>(s, G::X + 1 + (q >> 1)), q, conic);
+    st_form<M>(s, G::J + q, conic);
+    const bool conic_ok = group_all(sb_finite(conic));
+    __syncwarp();
+    const bool w_ok = group_all(coop_w<M>(s, q, rec, act && inv && conic_ok));
+    __syncwarp();  // the group's forms are read: the next record may overwrite them
+    if (!inv) return flags | F_SPLIT_PENDING;
+    if (!ok || !conic_ok || !w_ok) flags |= F_FALLBACK;
+    if (act && q == 0) rec_put_flags(rec + RL::FLAGS, flags);
+    return flags;
+}
+
+// record_build_kernel for a list of at most COOP_MAX records: eight groups of
+// four lanes per warp, the warps of the grid in turn so that a short list
+// spreads over the SMs.
+constexpr int COOP_T = 64;  // threads: at six pose variables 35 KB of forms per block
+template <int M>
+__global__ void __launch_bounds__(COOP_T) record_build_coop_kernel(
+    const double *__restrict__ vN, float fx, float fy, float cx, float cy, const CellData<M> *__restrict__ cells,
+    int64_t n_gauss, const uint32_t *__restrict__ work, const uint32_t *__restrict__ count, float *__restrict__ recs,
+    unsigned long long *__restrict__ counters, uint32_t *__restrict__ split_list, uint32_t *__restrict__ split_count)
+{
+    extern __shared__ double s_forms[];
+    const uint32_t n = *count;
+    if (n == 0 || n > COOP_MAX) return;
+    const int ln = threadIdx.x & 31, w = threadIdx.x >> 5, q = ln & 3;
+    double *s = s_forms + (threadIdx.x >> 2) * Coop<M>::STRIDE;
+    uint32_t built = 0, fb = 0;
+    for (uint32_t i0 = (w * gridDim.x + blockIdx.x) * 8u; i0 < n; i0 += gridDim.x * (COOP_T / 4)) {
+        const uint32_t i = i0 + (uint32_t)(ln >> 2);
+        const bool act = i < n;
+        const uint32_t p = work[act ? i : n - 1u];
+        const int cell = (int)(p / (uint64_t)n_gauss);
+        const int64_t g = (int64_t)p - (int64_t)cell * n_gauss;
+        const uint32_t f = coop_record<M>(s, q, vN + VN_STRIDE * g, fx, fy, cx, cy, cells[cell],
+                                          recs + (size_t)p * Rec<M>::WIDTH, act);
+        if (act && q == 0) {
+            if (f & F_SPLIT_PENDING) split_list[atomicAdd(split_count, 1u)] = p;
+            else if (f & F_FALLBACK) ++fb;
+            ++built;
+        }
+    }
+    if (counters) {
+        const uint32_t a = __reduce_add_sync(0xffffffffu, fb);
+        const uint32_t b = __reduce_add_sync(0xffffffffu, built);
+        if (ln == 0) {
+            if (a) atomicAdd(&counters[0], (unsigned long long)a);
+            if (b) atomicAdd(&counters[1], (unsigned long long)b);
+        }
+    }
+}
+
 // Builds the value part of the records listed in work[0, *count) (pair
 // indices within the batch, cell * n_gauss + g), whose decision part the
-// record kernel wrote.  Grid-stride over the list; the grid is sized on the
-// host without knowing the count.
+// record kernel wrote, where the list is longer than COOP_MAX (a shorter one is
+// record_build_coop_kernel's).  Grid-stride over the list; the grid is sized on
+// the host without knowing the count.
 // counters: [0] MatrixInv fallbacks among the records built, [1] records
 // built, [2] records whose MatrixInv needed input splitting.  A pair whose
 // MatrixInv fails on its cell is appended to the front of list (split_count
-// counts them) and finished by split_build_kernel; one whose Taylor order
-// exceeds the default is appended to the back (list_cap - 1 downwards;
-// khigh_count counts them) and finished by khigh_build_kernel.
+// counts them), one whose Taylor order exceeds the default to the back
+// (list_cap - 1 downwards; khigh_count counts them); finish_build_kernel
+// finishes both.
 template <int M>
 __global__ void __launch_bounds__(128) record_build_kernel(
     const double *__restrict__ vN, float fx, float fy, float cx, float cy, const CellData<M> *__restrict__ cells,
@@ -1345,6 +1596,7 @@ __global__ void __launch_bounds__(128) record_build_kernel(
 {
     using RL = Rec<M>;
     const uint32_t n = *count;
+    if (n <= COOP_MAX) return;
     uint32_t built = 0, fb = 0, sp = 0;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const uint32_t p = work[i];
@@ -1372,71 +1624,147 @@ __global__ void __launch_bounds__(128) record_build_kernel(
     }
 }
 
-// Finishes the records of the pairs record_build_kernel deferred (list[0,
-// *count)): one warp per pair, every lane running the value chain of the pair
-// (the same values), the warp splitting its cell (SPLIT_WARP).  Grid-stride
-// over the list by warps, pair i on block i mod gridDim.x first, so that a
-// short list puts one pair on each SM instead of four on a few SMs sharing
-// their FP64 pipes.  counters as in record_build_kernel ([0] fallbacks,
-// [2] splits; the pairs were counted as built there).
+// The records record_build_kernel deferred, by groups of four lanes.
+//
+// The pairs on whose cell MatrixInv failed (split_list[0, *split_count)), one
+// block per pair: its first group runs the value chain, then the block tries
+// the pieces of each bisection level, a group per piece (the pieces of
+// matinv_split: each failing piece bisected along its own split_var, down to
+// SPLIT_DEPTH; the hull and the outcome do not depend on the order), and the
+// first group finishes the record.  A warp per pair with every lane repeating
+// the chain took 192 us for the three pairs of a 10k-Gaussian cell.
+//
+// The pairs whose Taylor order exceeds the default (the back of split_list,
+// khigh_count of them): eight records per warp.
+//
+// counters as in record_build_kernel ([0] fallbacks, [2] splits; the pairs were
+// counted as built there).
+constexpr int FINISH_T = 128, FINISH_GROUPS = FINISH_T / 4;
 template <int M>
-__global__ void __launch_bounds__(128) split_build_kernel(
+__global__ void __launch_bounds__(FINISH_T) finish_build_kernel(
     const double *__restrict__ vN, float fx, float fy, float cx, float cy, const CellData<M> *__restrict__ cells,
-    int64_t n_gauss, const uint32_t *__restrict__ list, const uint32_t *__restrict__ count, float *__restrict__ recs,
-    unsigned long long *__restrict__ counters)
+    int64_t n_gauss, const uint32_t *__restrict__ list, const uint32_t *__restrict__ split_count, uint32_t list_cap,
+    const uint32_t *__restrict__ khigh_count, float *__restrict__ recs, unsigned long long *__restrict__ counters)
 {
     using RL = Rec<M>;
-    __shared__ uint64_t pieces[4][2 * 64];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t n = *count;
+    using G = Coop<M>;
+    extern __shared__ double s_forms[];
+    __shared__ uint64_t s_piece[2][64];
+    __shared__ double s_hull[FINISH_T / 32][4][2];
+    __shared__ int s_next, s_failed, s_ok;
+    constexpr unsigned FULL = 0xffffffffu;
+    const int tid = threadIdx.x, ln = tid & 31, wp = tid >> 5, q = ln & 3, grp = tid >> 2;
+    double *s = s_forms + grp * G::STRIDE;
     uint32_t fb = 0, sp = 0;
-    for (uint32_t i = (uint32_t)w * gridDim.x + blockIdx.x; i < n; i += gridDim.x * 4) {
+    // high orders: groups of the last blocks first (the splits take the first)
+    const uint32_t nk = *khigh_count, rb = gridDim.x - 1u - blockIdx.x;
+    for (uint32_t i0 = (wp * gridDim.x + rb) * 8u; i0 < nk; i0 += gridDim.x * FINISH_GROUPS) {
+        const uint32_t i = i0 + (uint32_t)(ln >> 2);
+        const bool act = i < nk;
+        const uint32_t p = list[list_cap - 1u - (act ? i : nk - 1u)];
+        const int cell = (int)(p / (uint64_t)n_gauss);
+        const int64_t g = (int64_t)p - (int64_t)cell * n_gauss;
+        const uint32_t f = coop_record<M>(s, q, vN + VN_STRIDE * g, fx, fy, cx, cy, cells[cell],
+                                          recs + (size_t)p * RL::WIDTH, act);
+        if (act && q == 0 && (f & F_FALLBACK)) ++fb;
+    }
+    __syncthreads();
+    const uint32_t ns = *split_count;
+    for (uint32_t i = blockIdx.x; i < ns; i += gridDim.x) {
         const uint32_t p = list[i];
         const int cell = (int)(p / (uint64_t)n_gauss);
         const int64_t g = (int64_t)p - (int64_t)cell * n_gauss;
         float *rec = recs + (size_t)p * RL::WIDTH;
-        const uint32_t f0 = __float_as_uint(rec[RL::FLAGS]);
-        __syncwarp();
-        const uint32_t f = record_value<M, float, SPLIT_WARP>(vN + VN_STRIDE * g, fx, fy, cx, cy, cells[cell],
-                                                             rec[RL::MU_X], rec[RL::MU_Y], f0, rec, pieces[w]);
-        if (lane == 0) {
-            if (f & F_FALLBACK) ++fb;
-            if (f & F_SPLIT) ++sp;
+        if (wp == 0) {
+            const bool ok = group_all(coop_chain<M>(s, q, vN + VN_STRIDE * g, fx, fy, cx, cy, cells[cell], rec[RL::MU_X],
+                                                    rec[RL::MU_Y], rec, grp == 0));
+            if (tid == 0) {
+                s_ok = ok;
+                s_failed = 0;
+                SB<M, double> X[4];
+                X[0] = ld_form<M>(s, G::X);
+                X[1] = ld_form<M>(s, G::X + 1);
+                X[3] = ld_form<M>(s, G::X + 2);
+                const int js = split_var<M>(X);
+                s_piece[0][0] = piece_child(0, js, 0);
+                s_piece[0][1] = piece_child(0, js, 1);
+            }
         }
-    }
-    if (counters && lane == 0) {
-        if (fb) atomicAdd(&counters[0], (unsigned long long)fb);
-        if (sp) atomicAdd(&counters[2], (unsigned long long)sp);
-    }
-}
-
-// Finishes the records of the pairs record_build_kernel deferred for their
-// Taylor order (list[list_cap - 1 - i], i < *count): one thread per pair, as
-// record_build_kernel without deferral.  counters as there ([0], [2]).
-template <int M>
-__global__ void __launch_bounds__(128) khigh_build_kernel(
-    const double *__restrict__ vN, float fx, float fy, float cx, float cy, const CellData<M> *__restrict__ cells,
-    int64_t n_gauss, const uint32_t *__restrict__ list, uint32_t list_cap, const uint32_t *__restrict__ count,
-    float *__restrict__ recs, unsigned long long *__restrict__ counters)
-{
-    using RL = Rec<M>;
-    const uint32_t n = *count;
-    uint32_t fb = 0, sp = 0;
-    // pair i on block i mod gridDim.x first (a short list spreads over the SMs)
-    for (uint32_t i = threadIdx.x * gridDim.x + blockIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const uint32_t p = list[list_cap - 1u - i];
-        const int cell = (int)(p / (uint64_t)n_gauss);
-        const int64_t g = (int64_t)p - (int64_t)cell * n_gauss;
-        float *rec = recs + (size_t)p * RL::WIDTH;
-        const uint32_t f = record_value<M, float>(vN + VN_STRIDE * g, fx, fy, cx, cy, cells[cell], rec[RL::MU_X],
-                                                  rec[RL::MU_Y], __float_as_uint(rec[RL::FLAGS]), rec);
-        if (f & F_FALLBACK) ++fb;
-        if (f & F_SPLIT) ++sp;
+        int cnt = 2, cur = 0;
+        double lo = Num<double>::BIG, hi = -Num<double>::BIG;  // the hull of Conic's entry q
+        for (int depth = 1; depth <= SPLIT_DEPTH && cnt > 0; ++depth) {
+            if (tid == 0) s_next = 0;
+            __syncthreads();
+            for (int base = 0; base < cnt; base += FINISH_GROUPS) {
+                const bool act = base + grp < cnt;
+                const uint64_t pc = s_piece[cur][act ? base + grp : 0];
+                double ctr[M], h[M];
+                piece_box<M>(pc, ctr, h);
+                SB<M, double> C;
+                const bool inv = coop_matinv<M>(sb_restrict<M>(ld_form<M>(s_forms, G::X + (q >> 1)), ctr, h),
+                                                sb_restrict<M>(ld_form<M>(s_forms, G::X + 1 + (q >> 1)), ctr, h), q, C);
+                if (act && inv) {
+                    lo = fmin(lo, C.vlo);
+                    hi = fmax(hi, C.vhi);
+                } else if (act && q == 0) {
+                    if (depth < SPLIT_DEPTH) {
+                        SB<M, double> X[4];
+                        X[0] = ld_form<M>(s_forms, G::X);
+                        X[1] = ld_form<M>(s_forms, G::X + 1);
+                        X[3] = ld_form<M>(s_forms, G::X + 2);
+                        for (int j = 0; j < M; ++j) {
+                            X[0].c[j] *= h[j];
+                            X[1].c[j] *= h[j];
+                            X[3].c[j] *= h[j];
+                        }
+                        const int js = split_var<M>(X), at = atomicAdd(&s_next, 2);
+                        s_piece[cur ^ 1][at] = piece_child(pc, js, 0);
+                        s_piece[cur ^ 1][at + 1] = piece_child(pc, js, 1);
+                    } else {
+                        s_failed = 1;
+                    }
+                }
+            }
+            __syncthreads();
+            cnt = s_failed ? 0 : s_next;
+            cur ^= 1;
+            __syncthreads();
+        }
+        for (int off = 4; off < 32; off <<= 1) {
+            lo = fmin(lo, __shfl_xor_sync(FULL, lo, off));
+            hi = fmax(hi, __shfl_xor_sync(FULL, hi, off));
+        }
+        if (ln < 4) {
+            s_hull[wp][q][0] = lo;
+            s_hull[wp][q][1] = hi;
+        }
+        __syncthreads();
+        if (wp == 0) {
+            for (int w = 1; w < FINISH_T / 32; ++w) {
+                lo = fmin(lo, s_hull[w][q][0]);
+                hi = fmax(hi, s_hull[w][q][1]);
+            }
+            const SB<M, double> conic = sb_cst<M, double>(lo, hi);
+            st_form<M>(s, G::J + q, conic);
+            const bool whole = !s_failed;
+            const bool conic_ok = group_all(sb_finite(conic));
+            __syncwarp();
+            const bool w_ok = group_all(coop_w<M>(s, q, rec, grp == 0 && whole && conic_ok));
+            if (tid == 0) {
+                uint32_t flags = __float_as_uint(rec[RL::FLAGS]);
+                if (whole) flags |= F_SPLIT;
+                if (!whole || !s_ok || !conic_ok || !w_ok) flags |= F_FALLBACK;
+                rec_put_flags(rec + RL::FLAGS, flags);
+                if (flags & F_FALLBACK) ++fb;
+                if (flags & F_SPLIT) ++sp;
+            }
+        }
+        __syncthreads();  // the forms and lists are read
     }
     if (counters) {
-        const uint32_t a = __reduce_add_sync(0xffffffffu, fb);
-        const uint32_t c = __reduce_add_sync(0xffffffffu, sp);
-        if ((threadIdx.x & 31) == 0) {
+        const uint32_t a = __reduce_add_sync(FULL, fb);
+        const uint32_t c = __reduce_add_sync(FULL, sp);
+        if (ln == 0) {
             if (a) atomicAdd(&counters[0], (unsigned long long)a);
             if (c) atomicAdd(&counters[2], (unsigned long long)c);
         }
