@@ -83,6 +83,12 @@ __global__ void __launch_bounds__(SC_THREADS) scan_sums_kernel(const uint32_t *_
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
+// offs: the block's offset (scanned sums), or (SUMS) the blocks' sums, of which
+// each block adds up those before it: for SC_SUM_BLOCKS blocks at most, that
+// costs less than the launches of a scan of the sums (a small render has ten
+// scans, each some 3 us per launch).
+constexpr uint32_t SC_SUM_BLOCKS = 2048;
+template <bool SUMS>
 __global__ void __launch_bounds__(SC_THREADS) scan_apply_kernel(const uint32_t *__restrict__ in, uint32_t n,
                                                                 const uint32_t *__restrict__ offs,
                                                                 uint32_t *__restrict__ out, DevLen dl)
@@ -90,6 +96,14 @@ __global__ void __launch_bounds__(SC_THREADS) scan_apply_kernel(const uint32_t *
     __shared__ uint32_t s_warp[32];
     n = dev_len(dl, n);
     if ((uint64_t)blockIdx.x * SC_TILE >= n) return;  // uniform over the block
+    uint32_t before = 0;
+    if (SUMS) {
+        uint32_t part = 0;
+        for (uint32_t b = threadIdx.x; b < blockIdx.x; b += SC_THREADS) part += offs[b];
+        block_exclusive_scan(part, s_warp, before);
+    } else if (offs) {
+        before = offs[blockIdx.x];
+    }
     const uint64_t base = (uint64_t)blockIdx.x * SC_TILE + (uint64_t)threadIdx.x * SC_IPT;
     uint32_t v[SC_IPT];
     uint32_t t = 0;
@@ -99,7 +113,7 @@ __global__ void __launch_bounds__(SC_THREADS) scan_apply_kernel(const uint32_t *
         t += v[i];
     }
     uint32_t total;
-    uint32_t run = block_exclusive_scan(t, s_warp, total) + (offs ? offs[blockIdx.x] : 0u);
+    uint32_t run = block_exclusive_scan(t, s_warp, total) + before;
 #pragma unroll
     for (int i = 0; i < SC_IPT; ++i) {
         if (base + i < n) out[base + i] = run;
@@ -126,15 +140,21 @@ static void exclusive_scan_dl(const uint32_t *in, uint32_t *out, uint64_t n, uin
     if (n == 0) return;
     const uint64_t nb = (n + SC_TILE - 1) / SC_TILE;
     if (nb == 1) {
-        scan_apply_kernel<<<1, SC_THREADS, 0, st>>>(in, (uint32_t)n, nullptr, out, dl);
+        scan_apply_kernel<false><<<1, SC_THREADS, 0, st>>>(in, (uint32_t)n, nullptr, out, dl);
         ++*launches;
+        return;
+    }
+    if (nb <= SC_SUM_BLOCKS) {
+        scan_sums_kernel<<<(unsigned)nb, SC_THREADS, 0, st>>>(in, (uint32_t)n, tmp, dl);
+        scan_apply_kernel<true><<<(unsigned)nb, SC_THREADS, 0, st>>>(in, (uint32_t)n, tmp, out, dl);
+        *launches += 2;
         return;
     }
     uint32_t *sums = tmp, *offs = tmp + nb;
     scan_sums_kernel<<<(unsigned)nb, SC_THREADS, 0, st>>>(in, (uint32_t)n, sums, dl);
     ++*launches;
     exclusive_scan_dl(sums, offs, nb, tmp + 2 * nb, st, launches, DevLen{});
-    scan_apply_kernel<<<(unsigned)nb, SC_THREADS, 0, st>>>(in, (uint32_t)n, offs, out, dl);
+    scan_apply_kernel<false><<<(unsigned)nb, SC_THREADS, 0, st>>>(in, (uint32_t)n, offs, out, dl);
     ++*launches;
 }
 
@@ -220,6 +240,59 @@ __global__ void __launch_bounds__(RS_THREADS) rs_hist_kernel(const K *__restrict
     }
 }
 
+// The histogram's rows (one per digit, a word per block) scanned in place, a
+// block per row, with the row totals in tot[digit]: one launch where a scan of
+// the whole histogram took three (the scatter adds up the totals of the digits
+// below its own).
+constexpr int RW_THREADS = 1024, RW_IPT = 4;  // (blocks of 128 where the rows are short)
+__global__ void __launch_bounds__(RW_THREADS) rs_rows_kernel(uint32_t *__restrict__ hist, uint32_t n, uint32_t nblocks,
+                                                             const uint32_t *__restrict__ n_dev,
+                                                             uint32_t *__restrict__ tot)
+{
+    __shared__ uint32_t s_warp[RW_THREADS / 32];
+    if (n_dev) nblocks = (min(n, *n_dev) + RS_TILE - 1) / RS_TILE;
+    uint32_t *row = hist + (uint64_t)blockIdx.x * nblocks;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t carry = 0;
+    const int warps = blockDim.x >> 5;
+    for (uint32_t base = 0; base < nblocks; base += blockDim.x * RW_IPT) {
+        const uint32_t i0 = base + threadIdx.x * RW_IPT;
+        uint32_t v[RW_IPT], t = 0;
+#pragma unroll
+        for (int i = 0; i < RW_IPT; ++i) {
+            v[i] = i0 + i < nblocks ? row[i0 + i] : 0u;
+            t += v[i];
+        }
+        uint32_t x = t;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, d);
+            if (lane >= d) x += y;
+        }
+        if (lane == 31) s_warp[warp] = x;
+        __syncthreads();
+        if (warp == 0) {
+            uint32_t w = lane < warps ? s_warp[lane] : 0u;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, w, d);
+                if (lane >= d) w += y;
+            }
+            s_warp[lane] = w;
+        }
+        __syncthreads();
+        uint32_t run = carry + x - t + (warp ? s_warp[warp - 1] : 0u);
+#pragma unroll
+        for (int i = 0; i < RW_IPT; ++i) {
+            if (i0 + i < nblocks) row[i0 + i] = run;
+            run += v[i];
+        }
+        carry += s_warp[31];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) tot[blockIdx.x] = carry;
+}
+
 // Scatter of one radix pass.  Each block ranks its RS_TILE items by digit
 // (stable: warps in order, rounds in order, lanes in order), reorders them by
 // digit in shared memory, then writes every digit run to its global offset
@@ -230,14 +303,15 @@ __global__ void __launch_bounds__(RS_THREADS) rs_scatter_kernel(const K *__restr
                                                                 K *__restrict__ kout, uint32_t *__restrict__ vout,
                                                                 uint32_t n, int shift, uint64_t n_gauss,
                                                                 const uint32_t *__restrict__ offs,
+                                                                const uint32_t *__restrict__ tot,
                                                                 uint32_t nblocks, const uint32_t *__restrict__ n_dev)
 {
     constexpr uint32_t NB = 1u << RB;
-    static_assert(NB <= RS_THREADS, "one thread per digit");
+    static_assert(NB <= RS_THREADS && RS_THREADS == SC_THREADS, "one thread per digit");
     __shared__ uint32_t wcnt[RS_WARPS][NB];
     __shared__ uint32_t dstart[NB];   // block-local start of each digit run
     __shared__ uint32_t gbase[NB];    // global start of each digit run of this block
-    __shared__ uint32_t s_warp[RS_WARPS];
+    __shared__ uint32_t s_warp[32];
     __shared__ K s_key[RS_TILE];
     __shared__ uint32_t s_val[RS_TILE];
     if (n_dev) {
@@ -246,6 +320,9 @@ __global__ void __launch_bounds__(RS_THREADS) rs_scatter_kernel(const K *__restr
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t ltmask = (1u << lane) - 1u;
+    uint32_t all;
+    // items of the digits below this thread's
+    const uint32_t digit0 = block_exclusive_scan(threadIdx.x < NB ? tot[threadIdx.x] : 0u, s_warp, all);
     for (uint32_t blk = blockIdx.x; blk < nblocks; blk += gridDim.x) {
         const uint64_t blk0 = (uint64_t)blk * RS_TILE;
         if (blk0 >= n) break;  // uniform over the block; later tiles are empty too
@@ -308,7 +385,7 @@ __global__ void __launch_bounds__(RS_THREADS) rs_scatter_kernel(const K *__restr
                 uint32_t wpre = 0;
                 for (int w = 0; w < warp; ++w) wpre += s_warp[w];
                 dstart[d] = wpre + x - run;
-                gbase[d] = offs[(uint64_t)d * nblocks + blk];
+                gbase[d] = digit0 + (offs ? offs[(uint64_t)d * nblocks + blk] : 0u);
             }
         }
         __syncthreads();
@@ -337,25 +414,28 @@ __global__ void __launch_bounds__(RS_THREADS) rs_scatter_kernel(const K *__restr
 size_t radix_hist_words(uint64_t n)
 {
     const uint64_t nb = (n + RS_TILE - 1) / RS_TILE;
-    return 256 * nb;
+    return 256 * nb + 256;  // and the digits' totals
 }
 
 // n_dev: see rs_hist_kernel; n is then an upper bound, and the grid is at
 // most a few blocks per SM
 template <class K, int RB, bool CELL = false>
 static void radix_pass(const K *ka, const uint32_t *va, K *kb, uint32_t *vb, uint64_t n, int shift, uint32_t *hist,
-                       uint32_t *scan_tmp, cudaStream_t st, int *launches, uint64_t n_gauss = 0,
+                       cudaStream_t st, int *launches, uint64_t n_gauss = 0,
                        const uint32_t *n_dev = nullptr)
 {
     const uint32_t nb = (uint32_t)((n + RS_TILE - 1) / RS_TILE);
     const uint32_t grid = n_dev ? (nb < kDevGrid ? nb : kDevGrid) : nb;
     rs_hist_kernel<K, RB, CELL><<<grid, RS_THREADS, 0, st>>>(ka, va, (uint32_t)n, shift, n_gauss, hist, nb, n_dev);
     ++*launches;
-    DevLen dl;
-    if (n_dev) dl = DevLen{n_dev, 1u << RB, (uint32_t)RS_TILE};
-    exclusive_scan_dl(hist, hist, ((uint64_t)1 << RB) * nb, scan_tmp, st, launches, dl);
-    rs_scatter_kernel<K, RB, CELL><<<grid, RS_THREADS, 0, st>>>(ka, va, kb, vb, (uint32_t)n, shift, n_gauss, hist, nb,
-                                                                n_dev);
+    // one tile: its histogram is the digits' totals
+    uint32_t *tot = nb > 1 ? hist + ((uint64_t)1 << RB) * nb : hist;
+    if (nb > 1) {
+        rs_rows_kernel<<<1u << RB, nb <= 512u ? 128 : RW_THREADS, 0, st>>>(hist, (uint32_t)n, nb, n_dev, tot);
+        ++*launches;
+    }
+    rs_scatter_kernel<K, RB, CELL><<<grid, RS_THREADS, 0, st>>>(ka, va, kb, vb, (uint32_t)n, shift, n_gauss,
+                                                                nb > 1 ? hist : nullptr, tot, nb, n_dev);
     ++*launches;
 }
 
@@ -363,8 +443,7 @@ static void radix_pass(const K *ka, const uint32_t *va, K *kb, uint32_t *vb, uin
 // [0, bits) of it, in passes of at most 8 bits; returns 1 if the result
 // ended in the alt buffers.
 static int radix_sort_cells(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, uint64_t n,
-                            int bits, uint64_t n_gauss, uint32_t *hist, uint32_t *scan_tmp, cudaStream_t st,
-                            int *launches)
+                            int bits, uint64_t n_gauss, uint32_t *hist, cudaStream_t st, int *launches)
 {
     if (n == 0 || bits <= 0) return 0;
     const int passes = (bits + 7) / 8;
@@ -375,11 +454,11 @@ static int radix_sort_cells(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, 
     for (int p = 0, shift = 0; p < passes; ++p, shift += rb) {
         switch (rb) {
         case 1: case 2: case 3: case 4:
-            radix_pass<uint64_t, 4, true>(ka, va, kb, vb, n, shift, hist, scan_tmp, st, launches, n_gauss); break;
-        case 5: radix_pass<uint64_t, 5, true>(ka, va, kb, vb, n, shift, hist, scan_tmp, st, launches, n_gauss); break;
-        case 6: radix_pass<uint64_t, 6, true>(ka, va, kb, vb, n, shift, hist, scan_tmp, st, launches, n_gauss); break;
-        case 7: radix_pass<uint64_t, 7, true>(ka, va, kb, vb, n, shift, hist, scan_tmp, st, launches, n_gauss); break;
-        default: radix_pass<uint64_t, 8, true>(ka, va, kb, vb, n, shift, hist, scan_tmp, st, launches, n_gauss); break;
+            radix_pass<uint64_t, 4, true>(ka, va, kb, vb, n, shift, hist, st, launches, n_gauss); break;
+        case 5: radix_pass<uint64_t, 5, true>(ka, va, kb, vb, n, shift, hist, st, launches, n_gauss); break;
+        case 6: radix_pass<uint64_t, 6, true>(ka, va, kb, vb, n, shift, hist, st, launches, n_gauss); break;
+        case 7: radix_pass<uint64_t, 7, true>(ka, va, kb, vb, n, shift, hist, st, launches, n_gauss); break;
+        default: radix_pass<uint64_t, 8, true>(ka, va, kb, vb, n, shift, hist, st, launches, n_gauss); break;
         }
         uint64_t *tk = ka; ka = kb; kb = tk;
         uint32_t *tv = va; va = vb; vb = tv;
@@ -395,7 +474,7 @@ static int radix_sort_cells(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, 
 // buffers.  n_dev: the count on the device, n its upper bound (radix_pass).
 template <class K>
 static int radix_sort(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, uint64_t n, int bits,
-                      uint32_t *hist, uint32_t *scan_tmp, cudaStream_t st, int *launches, int shift0 = 0,
+                      uint32_t *hist, cudaStream_t st, int *launches, int shift0 = 0,
                       const uint32_t *n_dev = nullptr)
 {
     if (n == 0 || bits <= 0) return 0;
@@ -406,11 +485,11 @@ static int radix_sort(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, 
     int flips = 0;
     for (int p = 0, shift = shift0; p < passes; ++p, shift += rb) {
         switch (rb) {
-        case 1: case 2: case 3: case 4: radix_pass<K, 4>(ka, va, kb, vb, n, shift, hist, scan_tmp, st, launches, 0, n_dev); break;
-        case 5: radix_pass<K, 5>(ka, va, kb, vb, n, shift, hist, scan_tmp, st, launches, 0, n_dev); break;
-        case 6: radix_pass<K, 6>(ka, va, kb, vb, n, shift, hist, scan_tmp, st, launches, 0, n_dev); break;
-        case 7: radix_pass<K, 7>(ka, va, kb, vb, n, shift, hist, scan_tmp, st, launches, 0, n_dev); break;
-        default: radix_pass<K, 8>(ka, va, kb, vb, n, shift, hist, scan_tmp, st, launches, 0, n_dev); break;
+        case 1: case 2: case 3: case 4: radix_pass<K, 4>(ka, va, kb, vb, n, shift, hist, st, launches, 0, n_dev); break;
+        case 5: radix_pass<K, 5>(ka, va, kb, vb, n, shift, hist, st, launches, 0, n_dev); break;
+        case 6: radix_pass<K, 6>(ka, va, kb, vb, n, shift, hist, st, launches, 0, n_dev); break;
+        case 7: radix_pass<K, 7>(ka, va, kb, vb, n, shift, hist, st, launches, 0, n_dev); break;
+        default: radix_pass<K, 8>(ka, va, kb, vb, n, shift, hist, st, launches, 0, n_dev); break;
         }
         K *tk = ka; ka = kb; kb = tk;
         uint32_t *tv = va; va = vb; vb = tv;
@@ -832,13 +911,11 @@ static int sort_entries(const BinArgs &a, bool packed, int cb, int tb, const uin
     const int T = 256;
     int h;
     if (packed) {
-        h = radix_sort<uint32_t>(a.ent_seg[0], a.ent_ev[0], a.ent_seg[1], a.ent_ev[1], a.n_entries, tb, a.hist,
-                                 a.scan_tmp, st, launches, cb, n_dev);
+        h = radix_sort<uint32_t>(a.ent_seg[0], a.ent_ev[0], a.ent_seg[1], a.ent_ev[1], a.n_entries, tb, a.hist, st, launches, cb, n_dev);
     } else {
         int bits = 0;
         while ((1ull << bits) < a.n_segments) ++bits;
-        h = radix_sort<uint32_t>(a.ent_seg[0], a.ent_ev[0], a.ent_seg[1], a.ent_ev[1], a.n_entries, bits, a.hist,
-                                 a.scan_tmp, st, launches, 0, n_dev);
+        h = radix_sort<uint32_t>(a.ent_seg[0], a.ent_ev[0], a.ent_seg[1], a.ent_ev[1], a.n_entries, bits, a.hist, st, launches, 0, n_dev);
     }
     const uint32_t *keys = a.ent_seg[h];
     if (packed) {
@@ -892,16 +969,14 @@ int run_binning(const BinArgs &a, BinOut &o, cudaStream_t st, int *launches)
         ++*launches;
     }
     // 3. sort by key bits, then stably by cell
-    int f = radix_sort<uint64_t>(a.ev_key[0], a.ev_val[0], a.ev_key[1], a.ev_val[1], ne, 64, a.hist, a.scan_tmp,
-                                 st, launches);
+    int f = radix_sort<uint64_t>(a.ev_key[0], a.ev_val[0], a.ev_key[1], a.ev_val[1], ne, 64, a.hist, st, launches);
     uint64_t *evk = a.ev_key[f];
     uint32_t *evv = a.ev_val[f];
     if (a.n_cells > 1) {
         // stably by cell, the digits taken from the pair index in the value
         int bits = 0;
         while ((1ull << bits) < (uint64_t)a.n_cells) ++bits;
-        const int g = radix_sort_cells(evk, evv, a.ev_key[f ^ 1], a.ev_val[f ^ 1], ne, bits, a.n_gauss, a.hist,
-                                       a.scan_tmp, st, launches);
+        const int g = radix_sort_cells(evk, evv, a.ev_key[f ^ 1], a.ev_val[f ^ 1], ne, bits, a.n_gauss, a.hist, st, launches);
         evk = a.ev_key[f ^ g];
         evv = a.ev_val[f ^ g];
     }
@@ -963,8 +1038,7 @@ int run_binning(const BinArgs &a, BinOut &o, cudaStream_t st, int *launches)
     seg_len_kernel<<<blocks_for(a.n_segments, T), T, 0, st>>>(a.seg_start, a.seg_end, a.n_segments, a.seg_k[0],
                                                                a.seg_v[0]);
     ++*launches;
-    int q = radix_sort<uint32_t>(a.seg_k[0], a.seg_v[0], a.seg_k[1], a.seg_v[1], a.n_segments, 8, a.hist,
-                                 a.scan_tmp, st, launches);
+    int q = radix_sort<uint32_t>(a.seg_k[0], a.seg_v[0], a.seg_k[1], a.seg_v[1], a.n_segments, 8, a.hist, st, launches);
     o.seg_order = a.seg_v[q];
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
@@ -1024,8 +1098,7 @@ int run_rebin(const BinArgs &a, const BinOut &first, const uint32_t *active, con
     active_keys_kernel<<<(unsigned)(mg < kDevGrid ? mg : kDevGrid), T, 0, st>>>(active, n_active, a.seg_total,
                                                                                a.seg_k[0], a.seg_v[0]);
     ++*launches;
-    const int q = radix_sort<uint32_t>(a.seg_k[0], a.seg_v[0], a.seg_k[1], a.seg_v[1], a.n_segments, 8, a.hist,
-                                       a.scan_tmp, st, launches, 0, n_active);
+    const int q = radix_sort<uint32_t>(a.seg_k[0], a.seg_v[0], a.seg_k[1], a.seg_v[1], a.n_segments, 8, a.hist, st, launches, 0, n_active);
     o.seg_order = a.seg_v[q];
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
