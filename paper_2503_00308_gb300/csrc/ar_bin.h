@@ -63,7 +63,8 @@ int run_rebin(const BinArgs &a, const BinOut &first, const uint32_t *active, con
 // pairs whose lower endpoints lie in the first `window` entries of the
 // active segments and lists them in work (count is incremented); the grid is
 // sized from max_active, the count of active segments is read on the device.
-void launch_set_u32(uint32_t *p, uint32_t v, cudaStream_t st);
+// launch_init_words: words[0] = v, words[1 .. 31] = 0 (the rounds' counters).
+void launch_init_words(uint32_t *words, uint32_t v, cudaStream_t st);
 void launch_demand(const uint32_t *active, const uint32_t *n_active, uint32_t max_active, const uint32_t *seg_start,
                    const uint32_t *seg_end, const uint32_t *ent_ev, const uint32_t *ev_val, uint32_t window,
                    uint32_t *state, uint32_t *work, uint32_t *count, cudaStream_t st);

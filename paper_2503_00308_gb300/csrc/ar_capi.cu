@@ -234,7 +234,7 @@ void Workspace::append_pointers(std::vector<uint64_t> &key) const
 {
     const DevBuf *all[] = {&cells_lohi, &cells, &vN, &recs, &boxes, &keys, &counters, &evk0, &evk1, &evv0, &evv1,
                            &ents0, &ents1, &ente0, &ente1, &ua, &ub, &uc, &ud, &hist, &scan, &segs, &sege, &segt, &cellev, &bwords, &smask, &ssat, &clist,
-                           &segk0, &segk1, &segv0, &segv1, &work, &state, &wlist, &act0, &act1, &words,
+                           &segk0, &segk1, &segv0, &segv1, &state, &wlist, &act0, &act1, &words,
                            &slist, &plist, &pmask, &whist};
     for (const DevBuf *b : all) key.push_back((uint64_t)(uintptr_t)b->p);
 }
@@ -247,7 +247,7 @@ void Workspace::release()
     cap_stream = nullptr;
     DevBuf *all[] = {&cells_lohi, &cells, &vN, &recs, &boxes, &keys, &counters, &evk0, &evk1, &evv0, &evv1,
                      &ents0, &ents1, &ente0, &ente1, &ua, &ub, &uc, &ud, &hist, &scan, &segs, &sege, &segt, &cellev, &bwords, &smask, &ssat, &clist, &segk0,
-                     &segk1, &segv0, &segv1, &work, &state, &wlist, &act0, &act1, &words, &slist, &plist, &pmask, &whist, &out_lo,
+                     &segk1, &segv0, &segv1, &state, &wlist, &act0, &act1, &words, &slist, &plist, &pmask, &whist, &out_lo,
                      &out_hi, &part_lo, &part_hi, &lvl_lo, &lvl_hi, &wpart};
     for (DevBuf *b : all) b->release();
     if (h_whist) cudaFreeHost(h_whist);
@@ -263,7 +263,7 @@ size_t Workspace::bytes() const
 {
     const DevBuf *all[] = {&cells_lohi, &cells, &vN, &recs, &boxes, &keys, &counters, &evk0, &evk1, &evv0, &evv1,
                            &ents0, &ents1, &ente0, &ente1, &ua, &ub, &uc, &ud, &hist, &scan, &segs, &sege, &segt, &cellev, &bwords, &smask, &ssat, &clist,
-                           &segk0, &segk1, &segv0, &segv1, &work, &state, &wlist, &act0, &act1, &words,
+                           &segk0, &segk1, &segv0, &segv1, &state, &wlist, &act0, &act1, &words,
                            &slist, &plist, &pmask, &whist, &out_lo, &out_hi, &part_lo, &part_hi, &lvl_lo, &lvl_hi, &wpart};
     size_t s = 0;
     for (const DevBuf *b : all) s += b->cap;
@@ -583,7 +583,6 @@ static int bin_pairs(Workspace &ws, const PixBox *boxes, const double *keys, uin
     RK(ws.segk1.ensure(sizeof(uint32_t) * n_seg));
     RK(ws.segv0.ensure(sizeof(uint32_t) * n_seg));
     RK(ws.segv1.ensure(sizeof(uint32_t) * n_seg));
-    RK(ws.work.ensure(256));
     if (ba_out) {
         RK(ws.cellev.ensure(sizeof(uint32_t) * 2 * (n_cells + 1)));
         RK(ws.bwords.ensure(sizeof(uint32_t) * 4));
@@ -731,7 +730,7 @@ static int render_batch(ar_scene *s, Workspace &ws, const CallConst &cc, int M, 
         RK(ws.wlist.ensure(sizeof(uint32_t) * n_pairs));
         RK(ws.act0.ensure(sizeof(uint32_t) * n_seg));
         RK(ws.act1.ensure(sizeof(uint32_t) * n_seg));
-        RK(ws.words.ensure(sizeof(uint32_t) * 8));
+        RK(ws.words.ensure(sizeof(uint32_t) * kRoundWords));
         RK(ws.slist.ensure(sizeof(uint32_t) * n_pairs));
         RK(ws.plist.ensure(sizeof(uint32_t) * n_seg));
         RK(ws.pmask.ensure(sizeof(uint32_t) * n_seg * (TS * TS / 32 + 1)));  // pixel mask + a flag per slot
@@ -834,7 +833,6 @@ static int enqueue_rest(ar_scene *s, Workspace &ws, const CallConst &cc, int M, 
     rl.seg_start = ws.segs.as<uint32_t>();
     rl.seg_end = ws.sege.as<uint32_t>();
     rl.seg_order = bo.seg_order;
-    rl.work = ws.work.as<unsigned int>();
     rl.ent_ev = bo.ent_ev;
     rl.ev_val = bo.ev_val;
     rl.ev_key = bo.ev_key;
@@ -931,21 +929,19 @@ int run_windowed_render(int M, int TS, RenderLaunch rl, const CallConst &cc, con
     const uint32_t *round1_order = nullptr;
     uint32_t *act[2] = {act0, act1};
     CK(cudaMemsetAsync(state, 0, sizeof(uint32_t) * n_pairs, st));
-    launch_set_u32(words + 1, (uint32_t)n_seg, st);
+    launch_init_words(words, (uint32_t)n_seg, st);
     ++*launches;
     static const char *kRoundName[3] = {"ar.round 0: build + render", "ar.round 1: build + render",
                                         "ar.round 2: build + render"};
     for (int r = 0; r < 3; ++r) {
         NvtxRange round_range(kRoundName[r]);
-        uint32_t *cur_n = words + 1 + (r & 1), *nxt_n = words + 1 + ((r + 1) & 1);
+        // the segments of this round and of the next, and this round's counts
+        uint32_t *cur_n = words + r, *nxt_n = words + r + 1, *cnt = words + 8 + 8 * r;
         const uint32_t *cur = r == 0 ? rl.seg_order : (r == 1 && round1_order ? round1_order : act[(r - 1) & 1]);
-        CK(cudaMemsetAsync(words, 0, sizeof(uint32_t), st));
-        CK(cudaMemsetAsync(nxt_n, 0, sizeof(uint32_t), st));
-        CK(cudaMemsetAsync(words + 3, 0, 2 * sizeof(uint32_t), st));
         launch_demand(cur, cur_n, (uint32_t)n_seg, rl.seg_start, rl.seg_end, rl.ent_ev, rl.ev_val, kWindow[r], state,
-                      wlist, words, st);
-        if (launch_record_build(M, vN, cc, cells, rl.n_gauss, wlist, words, rl.recs, build_counters, split_list,
-                                words + 3, (uint32_t)n_pairs, words + 4, st))
+                      wlist, cnt, st);
+        if (launch_record_build(M, vN, cc, cells, rl.n_gauss, wlist, cnt, rl.recs, build_counters, split_list,
+                                cnt + 1, (uint32_t)n_pairs, cnt + 2, st))
             return fail(AR_EDEVICE, "record build launch: %s", cudaGetErrorString(cudaGetLastError()));
         *launches += 2;
         if (ev) CK(record_stage(ev[2 * r], st));
@@ -955,9 +951,9 @@ int run_windowed_render(int M, int TS, RenderLaunch rl, const CallConst &cc, con
         rl.next_active = act[r & 1];
         rl.n_next = nxt_n;
         rl.precise = precise_list;
-        rl.n_precise = words + 5;
+        rl.n_precise = cnt + 3;
         rl.precise_mask = precise_mask;
-        CK(cudaMemsetAsync(words + 5, 0, sizeof(uint32_t), st));
+        rl.work = cnt + 4;
         rl.f64 = 0;
         rl.direct = rl.interleave && r == 0;
         if (launch_render(M, TS, rl, st))
@@ -967,7 +963,8 @@ int run_windowed_render(int M, int TS, RenderLaunch rl, const CallConst &cc, con
         // instance (window abandons go to the same next list)
         RenderLaunch rp = rl;
         rp.active = precise_list;
-        rp.n_active = words + 5;
+        rp.n_active = cnt + 3;
+        rp.work = cnt + 5;
         rp.f64 = 1;
         rp.direct = 0;
         if (launch_render(M, TS, rp, st))
@@ -980,7 +977,7 @@ int run_windowed_render(int M, int TS, RenderLaunch rl, const CallConst &cc, con
             if (two) {
                 NvtxRange rebin_range("ar.bin: full lists of the segments left");
                 BinOut full;
-                if (run_rebin(*rebin, *first, act[0], words + 2, full, st, launches))
+                if (run_rebin(*rebin, *first, act[0], nxt_n, full, st, launches))
                     return fail(AR_EDEVICE, "second binning phase: %s", cudaGetErrorString(cudaGetLastError()));
                 rl.ent_ev = full.ent_ev;
                 round1_order = full.seg_order;

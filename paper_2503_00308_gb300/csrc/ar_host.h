@@ -36,7 +36,7 @@ constexpr size_t kMaxGraphs = 32;  // cached graphs per workspace (least recentl
 struct Workspace {
     DevBuf cells_lohi, cells, vN, recs, boxes, keys, counters;
     DevBuf evk0, evk1, evv0, evv1, ents0, ents1, ente0, ente1;
-    DevBuf ua, ub, uc, ud, hist, scan, segs, sege, segk0, segk1, segv0, segv1, work;
+    DevBuf ua, ub, uc, ud, hist, scan, segs, sege, segk0, segk1, segv0, segv1;
     DevBuf clist;                              // pairs left by the cull (then their count)
     bool cull_on = true;                       // the last render found culling worth it
     DevBuf segt, cellev, bwords, smask, ssat;  // two-phase binning: full-list lengths, cell event ranges,
@@ -74,12 +74,14 @@ int validate_call(const ar_intrinsics *in, const ar_nominal_pose *pose, const ar
                   int32_t tile);
 struct RenderLaunch;
 struct CallConst;
+constexpr int kRoundWords = 32;  // active segments of rounds 0 to 3, then eight counters per round
 struct TunedTile {
     int W, H, M, TS, CH;  // key (image size, pose variables) -> tile edge, events per staged chunk
 };
 // The FP32 render of one batch in windowed rounds (see render_kernel):
 // demand -> build -> render per round, windows w0, 8192, then unlimited.
-// state [n_pairs] (zeroed here), wlist [n_pairs], act0/act1 [n_seg], words [8];
+// state [n_pairs] (zeroed here), wlist [n_pairs], act0/act1 [n_seg], words
+// [kRoundWords] (the rounds' counters, set here by one launch);
 // build_counters: [0] fallbacks, [1] records built, [2] splits (optional);
 // split_list [n_pairs]: pairs whose MatrixInv needs input splitting or a high
 // order, which a last kernel finishes; precise_list [n_seg]: segments that

@@ -37,7 +37,7 @@ struct RenderLaunch {
     unsigned long long *counters;     // optional: [0] opacity evaluations, [1] re-evaluations,
                                       // [5] segments abandoned for a wider window ([2]-[4]: record build),
                                       // [6] evaluations taken again in FP64, [7] segments swept again for them
-    unsigned int *work;               // segment counter of the persistent grid (zeroed by the launcher)
+    unsigned int *work;               // segment counter of the persistent grid (zeroed before the first round)
     int rel = 0;                      // 1: relational upper transmittance (AR_BLEND_RELATIONAL)
     int ch = 16;                      // events per staged chunk of the FP32 sweep (8, 16 or 32 at tile 16)
     // interleave: the first round's FP32 sweep (whose active list is all n_seg

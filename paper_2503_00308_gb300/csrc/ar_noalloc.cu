@@ -153,10 +153,9 @@ int ar_render_abstract_noalloc(ar_scene *s, const ar_intrinsics *in, const ar_no
     uint32_t *seg_start = A.take<uint32_t>(n_seg), *seg_end = A.take<uint32_t>(n_seg);
     uint32_t *seg_k0 = A.take<uint32_t>(n_seg), *seg_k1 = A.take<uint32_t>(n_seg);
     uint32_t *seg_v0 = A.take<uint32_t>(n_seg), *seg_v1 = A.take<uint32_t>(n_seg);
-    unsigned int *work = A.take<unsigned int>(64);
     uint32_t *state = A.take<uint32_t>(n_pairs), *wlist = A.take<uint32_t>(n_pairs);
     uint32_t *slist = A.take<uint32_t>(n_pairs);
-    uint32_t *act0 = A.take<uint32_t>(n_seg), *act1 = A.take<uint32_t>(n_seg), *words = A.take<uint32_t>(8);
+    uint32_t *act0 = A.take<uint32_t>(n_seg), *act1 = A.take<uint32_t>(n_seg), *words = A.take<uint32_t>(kRoundWords);
     uint32_t *plist = A.take<uint32_t>(n_seg), *pmask = A.take<uint32_t>(n_seg * (TS * TS / 32 + 1));
     if (A.over) return too_big("the per-(Gaussian, cell) records", A.used);
 
@@ -216,7 +215,6 @@ int ar_render_abstract_noalloc(ar_scene *s, const ar_intrinsics *in, const ar_no
     rl.seg_start = seg_start;
     rl.seg_end = seg_end;
     rl.seg_order = bo.seg_order;
-    rl.work = work;
     rl.ent_ev = bo.ent_ev;
     rl.ev_val = bo.ev_val;
     rl.ev_key = bo.ev_key;

@@ -1104,7 +1104,9 @@ int run_rebin(const BinArgs &a, const BinOut &first, const uint32_t *active, con
 }
 
 // ------------------------------------------------------------ windowed rounds
-__global__ void set_u32_kernel(uint32_t *p, uint32_t v) { *p = v; }
+// every counter of the windowed rounds in one launch (they were fifteen
+// memsets, a tenth of a small render's graph)
+__global__ void init_words_kernel(uint32_t *words, uint32_t v) { words[threadIdx.x] = threadIdx.x ? 0u : v; }
 
 // For each active segment, the lower endpoints among its first `window`
 // entries: every pair not yet claimed (state 0 -> 1) is appended to work.
@@ -1145,7 +1147,7 @@ __global__ void __launch_bounds__(256) demand_kernel(const uint32_t *__restrict_
     }
 }
 
-void launch_set_u32(uint32_t *p, uint32_t v, cudaStream_t st) { set_u32_kernel<<<1, 1, 0, st>>>(p, v); }
+void launch_init_words(uint32_t *words, uint32_t v, cudaStream_t st) { init_words_kernel<<<1, 32, 0, st>>>(words, v); }
 
 void launch_demand(const uint32_t *active, const uint32_t *n_active, uint32_t max_active, const uint32_t *seg_start,
                    const uint32_t *seg_end, const uint32_t *ent_ev, const uint32_t *ev_val, uint32_t window,

@@ -108,7 +108,6 @@ static int launch_render_ts(const RenderLaunch &a, cudaStream_t st)
     // direct launches (a.direct: the active list holds all nseg segments) take
     // one CTA per segment
     if (a.direct) grid = nseg;
-    if (cudaMemsetAsync(a.work, 0, sizeof(unsigned int), st) != cudaSuccess) return 1;
     kern<<<grid, SH::NTH, SM::BYTES, st>>>(a.recs, a.boxes, a.seg_start, a.seg_end, a.seg_total, a.cell_ev,
                                            a.active, a.n_active,
                                            a.window,
