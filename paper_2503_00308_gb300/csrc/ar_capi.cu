@@ -861,7 +861,7 @@ static int enqueue_rest(ar_scene *s, Workspace &ws, const CallConst &cc, int M, 
                                ws.wlist.as<uint32_t>(), ws.act0.as<uint32_t>(), ws.act1.as<uint32_t>(),
                                ws.words.as<uint32_t>(), rl.counters + 2, q, &launches,
                                profiling ? ev + 3 : nullptr, ws.w0, ws.slist.as<uint32_t>(), ws.plist.as<uint32_t>(),
-                               ws.pmask.as<uint32_t>(), bo.seg_total ? &ba : nullptr, &bo));
+                               ws.pmask.as<uint32_t>(), ws.segk0.as<uint32_t>(), bo.seg_total ? &ba : nullptr, &bo));
     }
     return AR_OK;
 }
@@ -920,7 +920,7 @@ int run_windowed_render(int M, int TS, RenderLaunch rl, const CallConst &cc, con
                         uint64_t n_pairs, uint64_t n_seg, uint32_t *state, uint32_t *wlist, uint32_t *act0,
                         uint32_t *act1, uint32_t *words, unsigned long long *build_counters, cudaStream_t st,
                         int *launches, cudaEvent_t *ev, uint32_t w0, uint32_t *split_list, uint32_t *precise_list,
-                        uint32_t *precise_mask, const BinArgs *rebin, const BinOut *first)
+                        uint32_t *precise_mask, uint32_t *precise_first, const BinArgs *rebin, const BinOut *first)
 {
     // two phases: a segment restarts in the second round mostly because its
     // depth prefix ran out, so that round keeps the first window
@@ -951,23 +951,13 @@ int run_windowed_render(int M, int TS, RenderLaunch rl, const CallConst &cc, con
         rl.next_active = act[r & 1];
         rl.n_next = nxt_n;
         rl.precise = precise_list;
-        rl.n_precise = cnt + 3;
         rl.precise_mask = precise_mask;
         rl.work = cnt + 4;
-        rl.f64 = 0;
+        rl.precise_first = precise_first;
+        rl.n_precise = reinterpret_cast<unsigned long long *>(cnt + 6);
+        rl.work_fp64 = cnt + 5;
         rl.direct = rl.interleave && r == 0;
         if (launch_render(M, TS, rl, st))
-            return fail(AR_EDEVICE, "render launch: %s", cudaGetErrorString(cudaGetLastError()));
-        // the segments where some pixel met an evaluation needing FP64, swept
-        // again from their start for those pixels by the FP64-capable
-        // instance (window abandons go to the same next list)
-        RenderLaunch rp = rl;
-        rp.active = precise_list;
-        rp.n_active = cnt + 3;
-        rp.work = cnt + 5;
-        rp.f64 = 1;
-        rp.direct = 0;
-        if (launch_render(M, TS, rp, st))
             return fail(AR_EDEVICE, "render launch: %s", cudaGetErrorString(cudaGetLastError()));
         if (ev) CK(record_stage(ev[2 * r + 1], st));
         *launches += 6;

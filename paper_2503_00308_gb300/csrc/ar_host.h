@@ -86,8 +86,9 @@ struct TunedTile {
 // split_list [n_pairs]: pairs whose MatrixInv needs input splitting or a high
 // order, which a last kernel finishes; precise_list [n_seg]: segments that
 // meet an opacity evaluation needing FP64, swept again by the FP64-capable
-// render instance in the same round, and precise_mask [n_seg * TS * TS / 32]
-// the pixels of each that do.
+// render instance in the same round, and precise_mask [n_seg * (TS * TS / 32 + 1)]
+// the pixels of each that do, precise_first [n_seg] its first work item (the
+// binning's seg_k[0], free once the schedule is sorted).
 // rebin / first: the binning of a two-phase render, whose second phase runs
 // between the first and the second round (null: one phase, lists complete)
 struct BinArgs;
@@ -96,7 +97,7 @@ int run_windowed_render(int M, int TS, RenderLaunch rl, const CallConst &cc, con
                         uint64_t n_pairs, uint64_t n_seg, uint32_t *state, uint32_t *wlist, uint32_t *act0,
                         uint32_t *act1, uint32_t *words, unsigned long long *build_counters, cudaStream_t st,
                         int *launches, cudaEvent_t *ev, uint32_t w0, uint32_t *split_list, uint32_t *precise_list,
-                        uint32_t *precise_mask, const BinArgs *rebin = nullptr, const BinOut *first = nullptr);
+                        uint32_t *precise_mask, uint32_t *precise_first, const BinArgs *rebin = nullptr, const BinOut *first = nullptr);
 // Depth prefix of the next render's first binning phase, from the stop
 // histograms of an earlier render (64 buckets of full-list entries, and of
 // segments, by where in its cell's depth order a segment stopped): the shift

@@ -44,11 +44,15 @@ struct RenderLaunch {
     // segments) launches one CTA per segment (direct) instead of persistent
     // CTAs, so that work on a higher-priority stream can take SMs as they free
     int interleave = 0, direct = 0;
-    // precision: the FP32 sweep (f64 = 0) appends a segment that needs an FP64
-    // evaluation to precise[*n_precise], with the mask of the pixels that do in
-    // precise_mask[slot * (TS * TS / 32 + 1) ...] (then a flag word); the f64 = 1 instance sweeps them
-    int f64 = 0;
-    uint32_t *precise = nullptr, *n_precise = nullptr, *precise_mask = nullptr;
+    // precision: the FP32 sweep appends a segment that needs an FP64
+    // evaluation to precise, with the mask of the pixels that do in
+    // precise_mask[slot * (TS * TS / 32 + 1) ...] (then a flag word) and the
+    // number of its first work item in precise_first; *n_precise: the segments
+    // (high word) and their work items; render_fp64_kernel takes them
+    // (work_fp64: its item counter)
+    uint32_t *precise = nullptr, *precise_mask = nullptr, *precise_first = nullptr;
+    unsigned long long *n_precise = nullptr;
+    unsigned int *work_fp64 = nullptr;
 };
 
 size_t cell_data_bytes(int M);

@@ -228,5 +228,5 @@ int ar_render_abstract_noalloc(ar_scene *s, const ar_intrinsics *in, const ar_no
     rl.out_hi = out_upper;
     rl.counters = nullptr;
     return run_windowed_render(M, TS, rl, cc, cellbuf, vN, n_pairs, n_seg, state, wlist, act0, act1, words, nullptr,
-                               st, &launches, nullptr, 512u, slist, plist, pmask);
+                               st, &launches, nullptr, 512u, slist, plist, pmask, seg_k0);
 }

@@ -81,40 +81,61 @@ int AR_CAT(launch_render_plain_m, AR_M)(int TS, const RenderLaunch &a, cudaStrea
     return TS == 16 ? launch_render_plain_ts<16>(a, st) : launch_render_plain_ts<8>(a, st);
 }
 
-template <int TS, bool REL, bool F64, int CH = 16>
+template <int TS, bool REL, int CH = 16>
 static int launch_render_ts(const RenderLaunch &a, cudaStream_t st)
 {
     // double-buffered chunks of CH events (16 unless the autotuner picks 8 or
-    // 32 for the FP32 sweep at tile 16: the exit vote, taken once per chunk,
+    // 32 at tile 16: the exit vote, taken once per chunk,
     // stops a tile sooner with short chunks, while long chunks take fewer
     // barriers) and a ring of 4 (rings of 3-8 measured: 4 keeps the ring's
     // shared memory small)
     constexpr int RING = 4;
-    typedef RenderShape<TS, F64> SH;
-    typedef RenderSmem<AR_M, TS, CH, RING, SH::NTH, SH::NBUF> SM;
-    auto kern = render_kernel<AR_M, TS, CH, RING, REL, F64>;
+    typedef RenderSmem<AR_M, TS, CH, RING> SM;
+    auto kern = render_kernel<AR_M, TS, CH, RING, REL>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::BYTES) != cudaSuccess)
         return 1;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SH::NTH, SM::BYTES) != cudaSuccess || per_sm < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SM::NT, SM::BYTES) != cudaSuccess || per_sm < 1)
         per_sm = 1;
     const uint32_t nseg = (uint32_t)a.n_cells * (uint32_t)a.n_tiles;
-    // work items: segments, or for the FP64 instance (segment, group of 32 pixels)
-    const uint64_t items = (uint64_t)nseg * (F64 ? (uint64_t)(TS * TS / 32) : 1u);
     uint32_t grid = (uint32_t)(sms * per_sm);
-    if (grid > items) grid = (uint32_t)items;
+    if (grid > nseg) grid = nseg;
     // direct launches (a.direct: the active list holds all nseg segments) take
     // one CTA per segment
     if (a.direct) grid = nseg;
-    kern<<<grid, SH::NTH, SM::BYTES, st>>>(a.recs, a.boxes, a.seg_start, a.seg_end, a.seg_total, a.cell_ev,
+    kern<<<grid, SM::NT, SM::BYTES, st>>>(a.recs, a.boxes, a.seg_start, a.seg_end, a.seg_total, a.cell_ev,
                                            a.active, a.n_active,
                                            a.window,
-                                           a.next_active, a.n_next, a.precise, a.n_precise, a.precise_mask, a.sweep_hist,
+                                           a.next_active, a.n_next, a.precise, a.n_precise, a.precise_mask, a.precise_first, a.sweep_hist,
                                            a.ent_ev, a.ev_val,
                                            a.ev_key, a.W, a.H, a.ntx, a.n_tiles, a.n_gauss, a.k_open, a.fp64_dev, a.out_lo,
                                            a.out_hi, a.counters, a.work, a.direct);
+    return cudaGetLastError() == cudaSuccess ? 0 : 1;
+}
+
+// the FP64-capable sweep of the segments listed in a.precise (it stages 16
+// entries at a time whatever the FP32 sweep's chunk is)
+template <int TS, bool REL>
+static int launch_render_fp64_ts(const RenderLaunch &a, cudaStream_t st)
+{
+    constexpr int CH = 16, RING = 4;
+    typedef PreciseSmem<AR_M, CH, RING> SM;
+    auto kern = render_fp64_kernel<AR_M, TS, CH, RING, REL>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SM)) != cudaSuccess) return 1;
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32, sizeof(SM)) != cudaSuccess || per_sm < 1)
+        per_sm = 1;
+    const uint64_t items = (uint64_t)a.n_cells * (uint64_t)a.n_tiles * (uint64_t)(TS * TS / PRECISE_PX);
+    uint32_t grid = (uint32_t)(sms * per_sm);
+    if (grid > items) grid = (uint32_t)items;
+    kern<<<grid, 32, sizeof(SM), st>>>(a.recs, a.boxes, a.seg_start, a.seg_end, a.seg_total, a.precise,
+                                       a.precise_first, a.n_precise, a.window, a.next_active, a.n_next, a.precise_mask, a.ent_ev, a.ev_val, a.ev_key,
+                                       a.W, a.H, a.ntx, a.n_tiles, a.n_gauss, a.k_open, a.fp64_dev, a.out_lo, a.out_hi,
+                                       a.counters, a.work_fp64);
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
 
@@ -163,15 +184,16 @@ int AR_CAT(launch_debug_alpha_m, AR_M)(const float *recs, int n, const int64_t *
 
 int AR_CAT(launch_render_m, AR_M)(int TS, const RenderLaunch &a, cudaStream_t st)
 {
-    if (a.f64) {
-        if (a.rel) return TS == 16 ? launch_render_ts<16, true, true>(a, st) : launch_render_ts<8, true, true>(a, st);
-        return TS == 16 ? launch_render_ts<16, false, true>(a, st) : launch_render_ts<8, false, true>(a, st);
-    }
-    if (TS == 8) return a.rel ? launch_render_ts<8, true, false>(a, st) : launch_render_ts<8, false, false>(a, st);
-    if (a.ch == 8) return a.rel ? launch_render_ts<16, true, false, 8>(a, st) : launch_render_ts<16, false, false, 8>(a, st);
-    if (a.ch == 32)
-        return a.rel ? launch_render_ts<16, true, false, 32>(a, st) : launch_render_ts<16, false, false, 32>(a, st);
-    return a.rel ? launch_render_ts<16, true, false>(a, st) : launch_render_ts<16, false, false>(a, st);
+    int r;
+    if (TS == 8) r = a.rel ? launch_render_ts<8, true>(a, st) : launch_render_ts<8, false>(a, st);
+    else if (a.ch == 8) r = a.rel ? launch_render_ts<16, true, 8>(a, st) : launch_render_ts<16, false, 8>(a, st);
+    else if (a.ch == 32) r = a.rel ? launch_render_ts<16, true, 32>(a, st) : launch_render_ts<16, false, 32>(a, st);
+    else r = a.rel ? launch_render_ts<16, true>(a, st) : launch_render_ts<16, false>(a, st);
+    if (r) return r;
+    // the segments where some pixel met an evaluation needing FP64 (window
+    // abandons go to the same next list)
+    if (TS == 8) return a.rel ? launch_render_fp64_ts<8, true>(a, st) : launch_render_fp64_ts<8, false>(a, st);
+    return a.rel ? launch_render_fp64_ts<16, true>(a, st) : launch_render_fp64_ts<16, false>(a, st);
 }
 
 }  // namespace ar

@@ -601,7 +601,7 @@ __device__ __forceinline__ float open_ratio_up(float a)
 
 // Shared-memory layout of the render kernel (dynamic; about 70 KB at six
 // pose variables, tile 16, chunks of 16 and a ring of 4, so two CTAs fit on an SM):
-//   two buffers (one in the FP64 instance), each with the records staged for
+//   two buffers, each with the records staged for
 //   a chunk of CH events, their event info and pixel boxes (the next chunk is
 //   copied in while the current one is swept),
 //   and a per-thread ring of the last RING opacity evaluations made at lower
@@ -609,11 +609,9 @@ __device__ __forceinline__ float open_ratio_up(float a)
 //   stored column-per-thread so that every access is bank-conflict free.  The ring lets the upper endpoint of
 //   a Gaussian reuse the evaluation made at its lower endpoint; an upper
 //   endpoint whose evaluation has left the ring evaluates again.
-// NTH: threads per CTA (the tile's pixels, or one warp for the FP64 instance);
-// NBUF: chunk buffers (two, or one for the FP64 instance, whose one-warp CTAs
-// then fit fourteen to an SM instead of nine)
-template <int M, int TS, int CH, int RING, int NTH = TS * TS, int NBUF = 2> struct RenderSmem {
-    static constexpr int NT = NTH;
+template <int M, int TS, int CH, int RING> struct RenderSmem {
+    static constexpr int NT = TS * TS;
+    static constexpr int NBUF = 2;
     static constexpr int PAY = M + 4;  // alo, ahi, rL, L.k, L.c[M]
     static constexpr int PV = (PAY + 3) / 4;  // ... as 16-byte vectors (the last one padded)
     static constexpr size_t REC = NBUF * sizeof(float) * CH * Rec<M>::WIDTH;  // chunk buffers
@@ -646,13 +644,11 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 template <int TS> struct RenderOcc {
     static constexpr int MIN_BLOCKS = TS * TS >= 256 ? 2 : 1;
 };
-// The FP64 instance runs one warp per CTA, sixteen CTAs per SM (the same
-// registers per thread as two 256-thread CTAs)
-template <int TS, bool F64> struct RenderShape {
-    static constexpr int NTH = F64 ? 32 : TS * TS;
-    static constexpr int NBUF = F64 ? 1 : 2;  // chunk buffers (see RenderSmem)
-    static constexpr int MIN_BLOCKS = F64 ? 16 : RenderOcc<TS>::MIN_BLOCKS;
-    static constexpr int MASKW = TS * TS / 32 + 1;  // words per listed segment: pixel mask, abandon flag
+// pixels per work item of the FP64 sweep
+constexpr int PRECISE_PX = 8;
+// words per listed segment of the FP64 sweep: the pixel mask, the abandon flag
+template <int TS> struct PreciseMask {
+    static constexpr int WORDS = TS * TS / 32 + 1;
 };
 
 // Persistent grid: each CTA takes (cell, tile) segments from the active list
@@ -667,25 +663,24 @@ template <int TS, bool F64> struct RenderShape {
 // from its start.  The sweep is deterministic, so the restarted segment
 // gives the same bounds it would have given in one pass.
 //
-// Precision (F64): the opacity evaluations whose weighted FP32 deviation
-// estimate exceeds fp64_dev are taken in FP64 (pixel_alpha_fp64).  The FP32
-// sweep (F64 = false) keeps that out-of-line call out of its code: it sweeps
+// Precision: the opacity evaluations whose weighted FP32 deviation
+// estimate exceeds fp64_dev are taken in FP64 (pixel_alpha_fp64).  This FP32
+// sweep keeps that out-of-line call out of its code: it sweeps
 // every segment in FP32, writes the bounds of the pixels that met no such
 // evaluation, and appends a segment where some pixel did to precise_list,
-// with the mask of those pixels (one word per warp) in precise_mask.  The
-// F64 = true instance sweeps the listed segments again from their start for
-// the masked pixels alone (the others start as stopped and write nothing).
+// with the mask of those pixels (one word per warp) in precise_mask.
+// render_fp64_kernel sweeps the listed segments again from their start for
+// the masked pixels alone.
 // The decision is per pixel, taken from the pixel's own sweep, so every pixel
-// gets the bounds one FP64-capable sweep would give it.  The FP64 instance
-// runs one warp per CTA: each work item is a listed segment and a group of up
-// to 32 of its listed pixels, so that many segments are in flight at once.
-template <int M, int TS, int CH, int RING, bool REL, bool F64>
-__global__ void __launch_bounds__(RenderShape<TS, F64>::NTH, RenderShape<TS, F64>::MIN_BLOCKS) render_kernel(
+// gets the bounds one FP64-capable sweep would give it.
+template <int M, int TS, int CH, int RING, bool REL>
+__global__ void __launch_bounds__(TS *TS, RenderOcc<TS>::MIN_BLOCKS) render_kernel(
     const float *__restrict__ recs, const PixBox *__restrict__ boxes, const uint32_t *__restrict__ seg_start,
     const uint32_t *__restrict__ seg_end, const uint32_t *__restrict__ seg_total,
     const uint32_t *__restrict__ cell_ev, const uint32_t *__restrict__ active, const uint32_t *__restrict__ n_active,
     uint32_t window, uint32_t *__restrict__ next_active, uint32_t *__restrict__ n_next,
-    uint32_t *__restrict__ precise_list, uint32_t *__restrict__ n_precise, uint32_t *__restrict__ precise_mask,
+    uint32_t *__restrict__ precise_list, unsigned long long *__restrict__ n_precise,
+    uint32_t *__restrict__ precise_mask, uint32_t *__restrict__ precise_first,
     uint32_t *__restrict__ sweep_hist,
     const uint32_t *__restrict__ entry_ev, const uint32_t *__restrict__ ev_val,
     const uint64_t *__restrict__ ev_key, int W, int H, int ntx, int n_tiles, int64_t n_gauss,
@@ -693,11 +688,8 @@ __global__ void __launch_bounds__(RenderShape<TS, F64>::NTH, RenderShape<TS, F64
     unsigned long long *__restrict__ counters, unsigned int *__restrict__ work, int direct)
 {
     using RL = Rec<M>;
-    using SH = RenderShape<TS, F64>;
-    using SM = RenderSmem<M, TS, CH, RING, SH::NTH, SH::NBUF>;
-    constexpr int NT = SH::NTH;      // threads
-    constexpr int NPIX = TS * TS;    // pixels of a tile
-    constexpr int GROUPS = F64 ? NPIX / 32 : 1;  // work items per listed segment
+    using SM = RenderSmem<M, TS, CH, RING>;
+    constexpr int NT = SM::NT;  // threads, the pixels of a tile
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float(*s_rec2)[RL::WIDTH] = reinterpret_cast<float(*)[RL::WIDTH]>(smem_raw);        // [2 * CH]
     EvInfo *s_ev2 = reinterpret_cast<EvInfo *>(smem_raw + SM::REC);                    // [2 * CH]
@@ -706,7 +698,7 @@ __global__ void __launch_bounds__(RenderShape<TS, F64>::NTH, RenderShape<TS, F64
     float4 *s_pay = reinterpret_cast<float4 *>(smem_raw + SM::REC + SM::EV + SM::BOX + SM::RID);
     uint32_t *s_next = reinterpret_cast<uint32_t *>(smem_raw + SM::REC + SM::EV + SM::BOX + SM::RID + SM::RPAY);
     const int tid = threadIdx.x;
-    uint32_t evals = 0, recomp = 0, wide = 0;
+    uint32_t evals = 0, recomp = 0;
     const uint32_t n_seg = *n_active;
 
     // direct: one CTA per active segment (the grid covers them all), so that
@@ -715,9 +707,8 @@ __global__ void __launch_bounds__(RenderShape<TS, F64>::NTH, RenderShape<TS, F64
     for (uint32_t round = 0;; ++round) {
         if (tid == 0) *s_next = direct ? (round == 0 ? blockIdx.x : 0xffffffffu) : atomicAdd(work, 1u);
         __syncthreads();
-        const uint32_t item = *s_next;
+        const uint32_t wk = *s_next;
         __syncthreads();
-        const uint32_t wk = item / GROUPS, grp = item % GROUPS;
         if (wk >= n_seg) break;
         const uint32_t seg = active[wk];
         const int cell = (int)(seg / (uint32_t)n_tiles);
@@ -726,33 +717,8 @@ __global__ void __launch_bounds__(RenderShape<TS, F64>::NTH, RenderShape<TS, F64
         // each warp covers an 8 x 4 block of the tile, so that the pixel boxes
         // of small Gaussians cut fewer warps and warps finish together
         const int wb = tid >> 5, ln = tid & 31;
-        // the pixel this thread sweeps, by its thread index in the FP32
-        // sweep's layout; the FP64 instance takes the listed pixels of rank
-        // 32 grp + tid among the mask's set bits
-        int pid = tid;
-        bool active = true;
-        if (F64) {
-            const uint32_t *pm = precise_mask + (size_t)wk * SH::MASKW;
-            int rem = (int)grp * 32 + tid;
-            pid = -1;
-#pragma unroll
-            for (int w = 0; w < NPIX / 32; ++w) {
-                uint32_t m = pm[w];
-                const int c = __popc(m);
-                if (pid < 0 && rem < c) {
-                    for (int k = 0; k < rem; ++k) m &= m - 1u;
-                    pid = w * 32 + __ffs(m) - 1;
-                } else if (pid < 0) {
-                    rem -= c;
-                }
-            }
-            active = pid >= 0;
-            if (!active) pid = 0;  // a position of the tile; the thread sweeps nothing
-            if (!__syncthreads_or(active)) continue;  // a group past the segment's listed pixels
-        }
-        const int pwb = pid >> 5, pln = pid & 31;
-        const int px = tx * TS + (pwb % (TS / 8)) * 8 + (pln & 7);
-        const int py = ty * TS + (pwb / (TS / 8)) * 4 + (pln >> 3);
+        const int px = tx * TS + (wb % (TS / 8)) * 8 + (ln & 7);
+        const int py = ty * TS + (wb / (TS / 8)) * 4 + (ln >> 3);
         const bool inside = px < W && py < H;
         const float ux = px + 0.5f, uy = py + 0.5f;
         const uint32_t b0 = seg_start[seg], b1 = seg_end[seg];
@@ -786,8 +752,7 @@ __global__ void __launch_bounds__(RenderShape<TS, F64>::NTH, RenderShape<TS, F64
 #pragma unroll
         for (int k = 0; k < RING; ++k) s_rid[k * NT + tid] = 0xffffffffu;
         uint32_t head = 0;
-        // the FP64 instance sweeps only the pixels the FP32 sweep listed
-        bool done = !inside || !active;
+        bool done = !inside;
         float lo_adj = 0.f, hi_adj = 0.f;  // -1: decided 0 / 1; >= 0: widening for skipped events
         // the upper sums' constants have reached 1 in every channel (interval
         // blend): final, because they only grow, so the upper bounds are 1
@@ -795,8 +760,8 @@ __global__ void __launch_bounds__(RenderShape<TS, F64>::NTH, RenderShape<TS, F64
         bool hi_fix = false;
         bool abandoned = false;
         uint32_t swept = b1 - b0;  // entries swept before the tile stopped
-        uint32_t seg_evals = 0, seg_recomp = 0, seg_wide = 0;
-        bool wide_hit = false;  // F64 = false: an evaluation needed FP64
+        uint32_t seg_evals = 0, seg_recomp = 0;
+        bool wide_hit = false;  // an evaluation needed FP64
 
         // Copy the chunk starting at entry sb into buffer bf: warp w takes
         // events EPW w .. EPW w + EPW - 1, its first EPW lanes read their event
@@ -840,7 +805,7 @@ __global__ void __launch_bounds__(RenderShape<TS, F64>::NTH, RenderShape<TS, F64
         // chunk it does not hold in full (the next binning phase gives the
         // segment its full list, and the sweep starts again: the exit tests
         // fall at the same entries, so the bounds are those of one sweep)
-        for (uint32_t base = b0; !abandoned && (base < b1 || incomplete); base += CH, buf = (buf + 1) % SH::NBUF) {
+        for (uint32_t base = b0; !abandoned && (base < b1 || incomplete); base += CH, buf ^= 1) {
             if (!done) {
                 const float left = (float)(total - (base - b0));
                 // PA is rounded down; 1.01 covers its relative error for < 10^5 factors
@@ -862,12 +827,6 @@ __global__ void __launch_bounds__(RenderShape<TS, F64>::NTH, RenderShape<TS, F64
                     hi_adj = hi_one ? -1.f : ehi2;
                 }
             }
-            // one buffer: the chunk is copied in once every thread has swept
-            // the previous one
-            if (SH::NBUF == 1 && base != b0) {
-                __syncthreads();
-                stage(0, base);
-            }
             cp_async_wait_all();  // this thread's copies of the current chunk
             if (__syncthreads_and(done)) {  // ... and everyone's, now visible
                 swept = base - b0;
@@ -884,7 +843,7 @@ __global__ void __launch_bounds__(RenderShape<TS, F64>::NTH, RenderShape<TS, F64
             }
             // the next chunk streams in while this one is swept; the buffer it
             // overwrites was swept by every thread before the barrier above
-            if (SH::NBUF == 2 && base + CH < b1) stage(buf ^ 1, base + CH);
+            if (base + CH < b1) stage(buf ^ 1, base + CH);
             const EvInfo *s_ev = s_ev2 + buf * CH;
             const PixBox *s_box = s_box2 + buf * CH;
             float(*s_rec)[RL::WIDTH] = s_rec2 + buf * CH;
@@ -948,14 +907,7 @@ __global__ void __launch_bounds__(RenderShape<TS, F64>::NTH, RenderShape<TS, F64
                         }
                         const float tlo = dead ? 0.f
                                                : (lower ? PA : fminf(1.f, __fdividef(PA, fmaxf(1.f - cache.ahi, 1e-6f))));
-                        if (cache.dev * ((sat ? 0.f : PB) + tlo) > fp64_dev) {
-                            if (F64) {
-                                cache = pixel_alpha_fp64<M>(r, ux, uy);
-                                ++seg_wide;
-                            } else {
-                                wide_hit = true;
-                            }
-                        }
+                        if (cache.dev * ((sat ? 0.f : PB) + tlo) > fp64_dev) wide_hit = true;
                     }
                     // a MatrixInv fallback is a constant [0, o]: not an evaluation
                     if (!(__float_as_uint(r[RL::FLAGS]) & F_FALLBACK)) {
@@ -1006,33 +958,36 @@ __global__ void __launch_bounds__(RenderShape<TS, F64>::NTH, RenderShape<TS, F64
             }
         }
         if (abandoned) {
-            // (the FP64 instance's groups of one segment list it once)
-            if (tid == 0 && (!F64 || atomicOr(&precise_mask[(size_t)wk * SH::MASKW + NPIX / 32], 1u) == 0u)) {
+            if (tid == 0) {
                 next_active[atomicAdd(n_next, 1u)] = seg;
                 if (counters) atomicAdd(&counters[5], 1ull);
             }
             continue;
         }
-        if (!F64 && __syncthreads_or(wide_hit)) {
-            // list the segment with the mask of its pixels that need FP64
+        if (const int n_wide = __syncthreads_count(wide_hit)) {
+            // list the segment with the mask of its pixels that need FP64; a
+            // work item takes PRECISE_PX of them
             // (the slot goes through s_next[1]: s_next[0], the work index, is
             // rewritten at the next segment's start while others may read this)
             if (tid == 0) {
-                const uint32_t slot = atomicAdd(n_precise, 1u);
+                const uint32_t parts = (uint32_t)(n_wide + PRECISE_PX - 1) / PRECISE_PX;
+                const unsigned long long at = atomicAdd(n_precise, (1ull << 32) | parts);
+                const uint32_t slot = (uint32_t)(at >> 32);
                 precise_list[slot] = seg;
-                precise_mask[(size_t)slot * SH::MASKW + NPIX / 32] = 0u;  // the FP64 instance's abandon flag
+                precise_first[slot] = (uint32_t)at;  // (ascending: slots and items are taken together)
+                precise_mask[(size_t)slot * PreciseMask<TS>::WORDS + TS * TS / 32] = 0u;  // the FP64 sweep's abandon flag
                 s_next[1] = slot;
                 if (counters) atomicAdd(&counters[7], 1ull);
             }
             __syncthreads();
             const uint32_t m = __ballot_sync(0xffffffffu, wide_hit);
-            if ((tid & 31) == 0) precise_mask[(size_t)s_next[1] * SH::MASKW + (tid >> 5)] = m;
+            if ((tid & 31) == 0) precise_mask[(size_t)s_next[1] * PreciseMask<TS>::WORDS + (tid >> 5)] = m;
         }
-        if (!F64 && sweep_hist && tid == 0) atomicAdd(&sweep_hist[min(swept / 32u, 255u)], 1u);
+        if (sweep_hist && tid == 0) atomicAdd(&sweep_hist[min(swept / 32u, 255u)], 1u);
         // where in its cell's depth order the segment stopped (64 buckets of
         // the cell's sorted events), weighted by its full length and counted:
         // the host sizes the next render's depth prefix from them
-        if (!F64 && sweep_hist && cell_ev && tid == 0 && b1 > b0) {
+        if (sweep_hist && cell_ev && tid == 0 && b1 > b0) {
             const uint32_t c0 = cell_ev[cell], ec = cell_ev[cell + 1] - c0;
             const uint32_t stop = entry_ev[b0 + (swept ? swept : 1u) - 1u];
             const uint32_t bkt = ec ? (uint32_t)min((uint64_t)(stop - c0) * 64u / ec, (uint64_t)63) : 0u;
@@ -1041,11 +996,9 @@ __global__ void __launch_bounds__(RenderShape<TS, F64>::NTH, RenderShape<TS, F64
         }
         evals += seg_evals;
         recomp += seg_recomp;
-        wide += seg_wide;
         if (REL && hk[0] >= 1.f && hk[1] >= 1.f && hk[2] >= 1.f) hi_adj = -1.f;
-        // pixels listed for the FP64 sweep, and in it the pixels not listed,
-        // leave their outputs to the other instance
-        if (inside && active && (F64 || !wide_hit)) {
+        // pixels listed for the FP64 sweep leave their outputs to it
+        if (inside && !wide_hit) {
             const size_t o = ((size_t)cell * H * W + (size_t)py * W + px) * 3;
 #pragma unroll
             for (int ch = 0; ch < 3; ++ch) {
@@ -1057,8 +1010,379 @@ __global__ void __launch_bounds__(RenderShape<TS, F64>::NTH, RenderShape<TS, F64
     if (counters) {
         const uint32_t a = __reduce_add_sync(0xffffffffu, evals);
         const uint32_t b = __reduce_add_sync(0xffffffffu, recomp);
-        const uint32_t c = __reduce_add_sync(0xffffffffu, wide);
         if ((tid & 31) == 0) {
+            if (a) atomicAdd(&counters[0], (unsigned long long)a);
+            if (b) atomicAdd(&counters[1], (unsigned long long)b);
+        }
+    }
+}
+
+// pixel_alpha from a record in global memory, out of line
+template <int M> __device__ __noinline__ AlphaOut<M> pixel_alpha_again(const float *r, float ux, float uy)
+{
+    AlphaOut<M> out;
+    pixel_alpha<M>(r, ux, uy, out);
+    return out;
+}
+
+// The FP64-capable sweep: the segments and pixels that render_kernel listed,
+// from their start.  A segment lists one pixel or a few, so a warp takes up to
+// PX of them and puts its lanes to their evaluations, which do not
+// depend on one another, instead of to pixels: per chunk of entries,
+//   - the (entry, pixel) pairs of the lower endpoints that a pixel's box test
+//     passes are listed, and the records of the entries that any passes staged;
+//   - the pairs are evaluated in FP32, one per lane, into shared memory;
+//   - lane k blends pixel k's entries in order, taking an evaluation in FP64
+//     where the pixel's state asks for it.
+// With a lane per pixel the warp's one or two busy lanes made every evaluation
+// in turn, about a thousand instructions each.  The render stage (both sweeps):
+// 16 cells of 10k Gaussians 0.797 -> 0.731 ms, 32 cells at 400 x 300 3.37 ->
+// 3.14, 64 cells of 300k 48.94 -> 48.34.
+// One warp per CTA; a work item is a listed segment and up to PX of its listed
+// pixels.
+template <int M, int CH, int RING> struct PreciseSmem {
+    static constexpr int PX = PRECISE_PX;
+    static constexpr int PAIRS = CH * PX;
+    static constexpr int RES = (2 * M + 7 + 3) / 4;  // L.c, U.c, L.k, U.k, rL, rU, alo, ahi, dev as 16-byte vectors
+    float rec[CH][Rec<M>::WIDTH];
+    float4 res[PAIRS][RES];
+    float4 ring[RING][(M + 4 + 3) / 4][PX];          // alo, ahi, rL, L.k, L.c
+    PixBox box[CH];
+    EvInfo ev[CH];
+    uint32_t rid[RING][PX];
+    float ux[PX], uy[PX];
+    uint8_t pair[PAIRS], slot[PAIRS];                // pair i's (entry, pixel) and the inverse
+};
+
+template <int M, int TS, int CH, int RING, bool REL>
+__global__ void __launch_bounds__(32, 11) render_fp64_kernel(
+    const float *__restrict__ recs, const PixBox *__restrict__ boxes, const uint32_t *__restrict__ seg_start,
+    const uint32_t *__restrict__ seg_end, const uint32_t *__restrict__ seg_total,
+    const uint32_t *__restrict__ listed, const uint32_t *__restrict__ first_item,
+    const unsigned long long *__restrict__ n_listed, uint32_t window, uint32_t *__restrict__ next_active, uint32_t *__restrict__ n_next,
+    uint32_t *__restrict__ precise_mask, const uint32_t *__restrict__ entry_ev, const uint32_t *__restrict__ ev_val,
+    const uint64_t *__restrict__ ev_key, int W, int H, int ntx, int n_tiles, int64_t n_gauss,
+    float k_open, float fp64_dev, float *__restrict__ out_lo, float *__restrict__ out_hi,
+    unsigned long long *__restrict__ counters, unsigned int *__restrict__ work)
+{
+    using RL = Rec<M>;
+    using SM = PreciseSmem<M, CH, RING>;
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int PX = SM::PX, NPIX = TS * TS, ROW4 = RL::WIDTH / 4, SC4 = RL::SCW / 4;
+    constexpr int PER = SM::PAIRS / 32;  // (entry, pixel) pairs per lane
+    static_assert(CH <= 32 && ROW4 <= 32 && PX == 8, "lane l tests pixel l mod 8");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    SM &sm = *reinterpret_cast<SM *>(smem_raw);
+    const int ln = threadIdx.x;
+    const uint32_t below = (1u << ln) - 1u;
+    uint32_t evals = 0, recomp = 0, wide = 0;
+    const uint32_t n_work = (uint32_t)*n_listed, n_seg = (uint32_t)(*n_listed >> 32);
+    for (;;) {
+        uint32_t at = 0;
+        if (ln == 0) at = atomicAdd(work, 1u);
+        at = __shfl_sync(FULL, at, 0);
+        if (at >= n_work) break;
+        // the listed segment wk that holds the item: first_item[wk] <= at
+        uint32_t wk = 0;
+        for (uint32_t end = n_seg; end - wk > 1u;) {
+            const uint32_t mid = wk + (end - wk) / 2u;
+            if (first_item[mid] <= at) wk = mid; else end = mid;
+        }
+        const uint32_t part = at - first_item[wk];
+        const uint32_t seg = listed[wk];
+        uint32_t *pm = precise_mask + (size_t)wk * PreciseMask<TS>::WORDS;
+        const int cell = (int)(seg / (uint32_t)n_tiles);
+        const int tile = (int)(seg - (uint32_t)cell * (uint32_t)n_tiles);
+        // lane l: the listed pixel of rank PX part + (l mod PX)
+        int pid = -1, rem = (int)part * PX + (ln & (PX - 1));
+#pragma unroll
+        for (int w = 0; w < NPIX / 32; ++w) {
+            uint32_t m = pm[w];
+            const int c = __popc(m);
+            if (pid < 0 && rem < c) {
+                for (int k = 0; k < rem; ++k) m &= m - 1u;
+                pid = w * 32 + __ffs(m) - 1;
+            } else if (pid < 0) {
+                rem -= c;
+            }
+        }
+        const uint32_t b0 = seg_start[seg], b1 = seg_end[seg];
+        const uint32_t total = seg_total ? seg_total[seg] : b1 - b0;
+        const bool incomplete = total > b1 - b0;
+        const float *rec_cell = recs + (size_t)cell * n_gauss * RL::WIDTH;
+        const PixBox *box_cell = boxes + (size_t)cell * n_gauss;
+        bool abandoned = incomplete && total <= SHORT_DEFER;  // (as in render_kernel)
+        if (!abandoned) {
+            const bool active = ln < PX && pid >= 0;  // this lane blends a pixel
+            const int px = tile % ntx * TS + ((pid >> 5) % (TS / 8)) * 8 + (pid & 7);
+            const int py = tile / ntx * TS + ((pid >> 5) / (TS / 8)) * 4 + ((pid >> 3) & 3);
+            ColourAcc<M, true> lo;
+            ColourAcc<M, false> hi;
+            lo.init();
+            hi.init();
+            float PA = 1.f, PB = 1.f, PAp = 1.f, PBp = 1.f;
+            RelT<M> rel;
+            bool rel_tie = false;
+            float hk[3] = {0.f, 0.f, 0.f};
+            if (REL) rel.init();
+            int n_open = 0;
+            float open_w = 0.f;
+            uint32_t head = 0;
+            bool done = !active, hi_fix = false;
+            float lo_adj = 0.f, hi_adj = 0.f;
+            uint32_t px_evals = 0, px_recomp = 0, px_wide = 0;
+            __syncwarp();
+            if (ln < PX) {
+#pragma unroll
+                for (int k = 0; k < RING; ++k) sm.rid[k][ln] = 0xffffffffu;
+                sm.ux[ln] = px + 0.5f;
+                sm.uy[ln] = py + 0.5f;
+            }
+            for (uint32_t base = b0; base < b1 || incomplete; base += CH) {
+                if (!done) {
+                    const float left = (float)(total - (base - b0));
+                    const float ow = fminf(open_w, __fmul_ru((float)n_open, k_open));
+                    const float elo2 = __fmul_ru(__fmul_ru(PA, 1.01f), __fadd_ru(ow, 1.f));
+                    const float ehi2 = __fmul_ru(1.1f, __fmul_ru(left, PB));
+                    bool lo_zero = true, hi_one = true;
+#pragma unroll
+                    for (int ch = 0; ch < 3; ++ch) {
+                        lo_zero = lo_zero && __fadd_ru(lo.upper_min(ch), elo2) <= 0.f;
+                        hi_one = hi_one && (REL ? hk[ch] : hi.k[ch]) >= 1.f;
+                    }
+                    if (!REL) hi_fix = hi_one;
+                    const bool lo_dec = lo_zero || elo2 <= EXIT_EPS;
+                    const bool hi_dec = hi_one || ehi2 <= EXIT_EPS;
+                    if (lo_dec && hi_dec) {
+                        done = true;
+                        lo_adj = lo_zero ? -1.f : elo2;
+                        hi_adj = hi_one ? -1.f : ehi2;
+                    }
+                }
+                const uint32_t alive = __ballot_sync(FULL, !done);
+                if (alive == 0u) break;
+                const int cnt = base < b1 ? (int)min((uint32_t)CH, b1 - base) : 0;
+                if ((incomplete && base + CH > b1) || base + (uint32_t)cnt - b0 > window) {
+                    abandoned = true;
+                    break;
+                }
+                __syncwarp();  // the previous chunk is swept
+                uint32_t rec = 0;
+                bool up = false;
+                if (ln < cnt) {
+                    const uint32_t i = base + (uint32_t)ln;
+                    const uint32_t e = entry_ev[i];
+                    const uint32_t v = ev_val[e];
+                    uint32_t bits = v & 1u;
+                    if (i > b0 && ev_key[entry_ev[i - 1]] == ev_key[e]) bits |= 2u;
+                    rec = (v >> 1) - (uint32_t)(cell * n_gauss);
+                    up = v & 1u;
+                    sm.ev[ln] = EvInfo{rec, bits};
+                    sm.box[ln] = box_cell[rec];
+                }
+                const uint32_t uppers = __ballot_sync(FULL, up);
+                __syncwarp();
+                // lane l tests entries (l / 8) + 4 j against pixel l mod 8
+                int n_pairs = 0;
+                uint32_t hits = 0;  // the entries that meet a pixel
+#pragma unroll
+                for (int j = 0; j < PER; ++j) {
+                    const int e = (ln >> 3) + 4 * j;
+                    bool in = false;
+                    if (e < cnt && ((alive >> (ln & 7)) & 1u)) {
+                        const PixBox bx = sm.box[e];
+                        in = px >= bx.x0 && px <= bx.x1 && py >= bx.y0 && py <= bx.y1;
+                    }
+                    const uint32_t m = __ballot_sync(FULL, in);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) hits |= ((m >> (8 * q)) & 255u ? 1u : 0u) << (4 * j + q);
+                    const bool ev = in && !((uppers >> e) & 1u);
+                    const uint32_t mp = __ballot_sync(FULL, ev);
+                    if (ev) {
+                        const int i = n_pairs + __popc(mp & below);
+                        sm.pair[i] = (uint8_t)(e * PX + (ln & 7));
+                        sm.slot[e * PX + (ln & 7)] = (uint8_t)i;
+                    }
+                    n_pairs += __popc(mp);
+                }
+                // the whole row for a lower endpoint, its scalars for an upper one
+                for (uint32_t h = hits; h; h &= h - 1u) {
+                    const int e = __ffs(h) - 1;
+                    const uint32_t rk = __shfl_sync(FULL, rec, e);
+                    const bool upk = (uppers >> e) & 1u;
+                    const int at = (upk ? RL::SC : 0) + 4 * ln;
+                    if (ln < (upk ? SC4 : ROW4)) cp_async16(&sm.rec[e][at], rec_cell + (size_t)rk * RL::WIDTH + at);
+                }
+                cp_async_wait_all();
+                __syncwarp();
+                for (int i = ln; i < n_pairs; i += 32) {
+                    const int c = sm.pair[i];
+                    AlphaOut<M> o;
+                    pixel_alpha<M>(sm.rec[c / PX], sm.ux[c % PX], sm.uy[c % PX], o);
+                    float f[4 * SM::RES] = {};
+#pragma unroll
+                    for (int j = 0; j < M; ++j) {
+                        f[j] = o.L.c[j];
+                        f[M + j] = o.U.c[j];
+                    }
+                    f[2 * M] = o.L.k;
+                    f[2 * M + 1] = o.U.k;
+                    f[2 * M + 2] = o.rL;
+                    f[2 * M + 3] = o.rU;
+                    f[2 * M + 4] = o.alo;
+                    f[2 * M + 5] = o.ahi;
+                    f[2 * M + 6] = o.dev;
+#pragma unroll
+                    for (int q = 0; q < SM::RES; ++q)
+                        sm.res[i][q] = make_float4(f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
+                }
+                __syncwarp();
+                if (done) continue;
+                for (int e = 0; e < cnt; ++e) {
+                    const EvInfo ev = sm.ev[e];
+                    if (!(ev.bits & 2u)) {
+                        PA = __fmul_rd(PA, PAp);
+                        PB = __fmul_ru(PB, PBp);
+                        PAp = 1.f;
+                        PBp = 1.f;
+                        rel_tie = false;
+                    }
+                    const PixBox bx = sm.box[e];
+                    if (px < bx.x0 || px > bx.x1 || py < bx.y0 || py > bx.y1) continue;
+                    const float *r = sm.rec[e];
+                    const float *row = rec_cell + (size_t)ev.rec * RL::WIDTH;  // (an upper endpoint's is not staged)
+                    const bool lower = !(ev.bits & 1u);
+                    const float ux = px + 0.5f, uy = py + 0.5f;
+                    n_open += lower ? 1 : -1;
+                    AlphaOut<M> cache;
+                    bool have = lower;
+                    if (lower) {
+                        float4 v[SM::RES];
+                        const int i = sm.slot[e * PX + ln];
+#pragma unroll
+                        for (int q = 0; q < SM::RES; ++q) v[q] = sm.res[i][q];
+#pragma unroll
+                        for (int j = 0; j < M; ++j) {
+                            cache.L.c[j] = f4_at(v, j);
+                            cache.U.c[j] = f4_at(v, M + j);
+                        }
+                        cache.L.k = f4_at(v, 2 * M);
+                        cache.U.k = f4_at(v, 2 * M + 1);
+                        cache.rL = f4_at(v, 2 * M + 2);
+                        cache.rU = f4_at(v, 2 * M + 3);
+                        cache.alo = f4_at(v, 2 * M + 4);
+                        cache.ahi = f4_at(v, 2 * M + 5);
+                        cache.dev = f4_at(v, 2 * M + 6);
+                    } else {
+                        int hit = -1;
+#pragma unroll
+                        for (int k = 0; k < RING; ++k)
+                            if (sm.rid[k][ln] == ev.rec) hit = k;
+                        if (hit >= 0) {
+                            float4 v[(M + 4 + 3) / 4];
+#pragma unroll
+                            for (int q = 0; q < (M + 4 + 3) / 4; ++q) v[q] = sm.ring[hit][q][ln];
+                            cache.alo = v[0].x;
+                            cache.ahi = v[0].y;
+                            cache.rL = v[0].z;
+                            cache.L.k = v[0].w;
+#pragma unroll
+                            for (int j = 0; j < M; ++j) cache.L.c[j] = f4_at(v, 4 + j);
+                            have = true;
+                        }
+                    }
+                    if (!have) cache = pixel_alpha_again<M>(row, ux, uy);
+                    if (lower || !have) {
+                        // (the test of render_kernel)
+                        if (cache.dev > 0.5f * fp64_dev) {
+                            bool sat = true, dead = true;
+                            const int nb = n_open + (lower ? -1 : 1);  // before this event
+                            const float ow = fminf(open_w, __fmul_ru((float)nb, k_open));
+                            const float elo = __fmul_ru(__fmul_ru(PA, 1.01f), __fadd_ru(ow, 1.f));
+#pragma unroll
+                            for (int ch = 0; ch < 3; ++ch) {
+                                sat = sat && (REL ? hk[ch] : hi.k[ch]) >= 1.f;
+                                dead = dead && __fadd_ru(lo.upper_min(ch), elo) <= 0.f;
+                            }
+                            const float tlo = dead ? 0.f
+                                                   : (lower ? PA : fminf(1.f, __fdividef(PA, fmaxf(1.f - cache.ahi, 1e-6f))));
+                            if (cache.dev * ((sat ? 0.f : PB) + tlo) > fp64_dev) {
+                                cache = pixel_alpha_fp64<M>(row, ux, uy);
+                                ++px_wide;
+                            }
+                        }
+                        if (!(__float_as_uint(r[RL::FLAGS]) & F_FALLBACK)) {
+                            if (lower) ++px_evals; else ++px_recomp;
+                        }
+                    }
+                    const float col[3] = {r[RL::COL], r[RL::COL + 1], r[RL::COL + 2]};
+                    const float colh[3] = {r[RL::COL_HI], r[RL::COL_HI + 1], r[RL::COL_HI + 2]};
+                    if (lower) {
+                        if (!hi_fix) hi.add(PB, colh, cache.U, cache.rU);
+                        if (REL) {
+#pragma unroll
+                            for (int ch = 0; ch < 3; ++ch)
+                                hk[ch] = __fmaf_ru(__fmul_ru(PB, colh[ch]), cache.U.k, hk[ch]);
+                        }
+                        if (REL && !rel_tie && cache.alo > 0.f) {
+                            LF<M, float> D = rel.F;
+                            D.k = __fsub_ru(rel.F.k, PB);
+                            hi.add(cache.alo, colh, D, rel.rF);
+                        }
+                        PAp = __fmul_rd(PAp, __fsub_rd(1.f, cache.ahi));
+                        open_w = __fadd_ru(open_w, open_ratio_up(cache.ahi));
+                        const int k = (int)(head % RING);
+                        ++head;
+                        sm.rid[k][ln] = ev.rec;
+                        auto pay = [&](int i) { return i < 4 ? (i == 0 ? cache.alo : i == 1 ? cache.ahi : i == 2 ? cache.rL : cache.L.k)
+                                                             : (i < 4 + M ? cache.L.c[i < 4 + M ? i - 4 : 0] : 0.f); };
+#pragma unroll
+                        for (int q = 0; q < (M + 4 + 3) / 4; ++q)
+                            sm.ring[k][q][ln] = make_float4(pay(4 * q), pay(4 * q + 1), pay(4 * q + 2), pay(4 * q + 3));
+                    } else {
+                        open_w = fmaxf(0.f, __fsub_ru(open_w, open_ratio_up(cache.ahi)));
+                        const uint32_t flags = __float_as_uint(r[RL::FLAGS]);
+                        float T = PA;
+                        if (flags & F_OPEN) {
+                            const float den = __fsub_ru(1.f, cache.ahi);
+                            T = (den > 0.f) ? Num<float>::div_pos_dn(PA, den) : 0.f;
+                        }
+                        lo.add(T, col, cache.L, cache.rL);
+                        PBp = __fmul_ru(PBp, __fsub_ru(1.f, cache.alo));
+                        if (REL) {
+                            rel.absorb(cache.L, cache.rL, cache.alo, cache.ahi);
+                            rel_tie = true;
+                        }
+                    }
+                }
+            }
+            if (!abandoned) {
+                evals += px_evals;
+                recomp += px_recomp;
+                wide += px_wide;
+            }
+            if (REL && hk[0] >= 1.f && hk[1] >= 1.f && hk[2] >= 1.f) hi_adj = -1.f;
+            if (active && !abandoned) {
+                const size_t o = ((size_t)cell * H * W + (size_t)py * W + px) * 3;
+#pragma unroll
+                for (int ch = 0; ch < 3; ++ch) {
+                    out_lo[o + ch] = lo_adj < 0.f ? 0.f : clamp01(__fsub_rd(lo.bound(ch), lo_adj));
+                    out_hi[o + ch] = hi_adj < 0.f ? 1.f : clamp01(__fadd_ru(hi.bound(ch), hi_adj));
+                }
+            }
+        }
+        // (a segment that one of its items abandons is listed once)
+        if (abandoned && ln == 0 && atomicOr(&pm[NPIX / 32], 1u) == 0u) {
+            next_active[atomicAdd(n_next, 1u)] = seg;
+            if (counters) atomicAdd(&counters[5], 1ull);
+        }
+        __syncwarp();
+    }
+    if (counters) {
+        const uint32_t a = __reduce_add_sync(FULL, evals);
+        const uint32_t b = __reduce_add_sync(FULL, recomp);
+        const uint32_t c = __reduce_add_sync(FULL, wide);
+        if (ln == 0) {
             if (a) atomicAdd(&counters[0], (unsigned long long)a);
             if (b) atomicAdd(&counters[1], (unsigned long long)b);
             if (c) atomicAdd(&counters[6], (unsigned long long)c);

@@ -43,7 +43,7 @@ def test_builders_give_the_same_records(arlib, move):
     cam = synth.look_camera(256, 144, 180.0, centre=(0.0, 0.0, 0.0))
     on = {"x": (1, 0, 0, 0, 0, 0), "xyz_yaw": (1, 1, 1, 0, 1, 0), "6dof": (1, 1, 1, 1, 1, 1)}[move]
     hw = np.array(on) * np.array([0.05] * 3 + [0.02] * 3)
-    lo, hi = synth.cell_grid(hw, [4, 1, 1, 1, 1, 1])
+    lo, hi = synth.cell_grid(hw, [12, 1, 1, 1, 1, 1])
     a1, b1, one = render(arlib, sc, cam, lo, hi)
     a2, b2, each = render(arlib, sc, cam, lo, hi, limit=1 << 20)   # a cell per batch: at most 20000 records
     assert one["n_built"] > COOP_MAX and one["n_built"] == each["n_built"]
