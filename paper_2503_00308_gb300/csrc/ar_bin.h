@@ -21,7 +21,7 @@ struct BinArgs {
     uint32_t *ev_val[2];     // [n_events] x2
     uint32_t *ent_seg[2];    // [n_entries] x2
     uint32_t *ent_ev[2];     // [n_entries] x2
-    uint32_t *u32_a, *u32_b, *u32_c, *u32_d;  // scratch, >= max(n_pairs, n_events) words each
+    uint32_t *u32_a, *u32_b;  // scratch, >= max(n_pairs, n_events) words each
     uint32_t *hist;          // >= radix_hist_words(max(n_events, n_entries))
     uint32_t *scan_tmp;      // >= scan_temp_words(largest scanned length)
     uint32_t *seg_start, *seg_end;  // [n_segments]
@@ -63,8 +63,9 @@ int run_rebin(const BinArgs &a, const BinOut &first, const uint32_t *active, con
 // pairs whose lower endpoints lie in the first `window` entries of the
 // active segments and lists them in work (count is incremented); the grid is
 // sized from max_active, the count of active segments is read on the device.
-// launch_init_words: words[0] = v, words[1 .. 31] = 0 (the rounds' counters).
-void launch_init_words(uint32_t *words, uint32_t v, cudaStream_t st);
+// launch_init_rounds: words[0] = n_seg, words[1 .. 31] = 0 (the rounds'
+// counters), seg_state[n_seg] = seg_swept[n_seg] = 0.
+void launch_init_rounds(uint32_t *words, uint32_t n_seg, uint32_t *seg_state, uint32_t *seg_swept, cudaStream_t st);
 void launch_demand(const uint32_t *active, const uint32_t *n_active, uint32_t max_active, const uint32_t *seg_start,
                    const uint32_t *seg_end, const uint32_t *ent_ev, const uint32_t *ev_val, uint32_t window,
                    uint32_t *state, uint32_t *work, uint32_t *count, cudaStream_t st);

@@ -233,9 +233,9 @@ void DevBuf::release()
 void Workspace::append_pointers(std::vector<uint64_t> &key) const
 {
     const DevBuf *all[] = {&cells_lohi, &cells, &vN, &recs, &boxes, &keys, &counters, &evk0, &evk1, &evv0, &evv1,
-                           &ents0, &ents1, &ente0, &ente1, &ua, &ub, &uc, &ud, &hist, &scan, &segs, &sege, &segt, &cellev, &bwords, &smask, &ssat, &clist,
+                           &ents0, &ents1, &ente0, &ente1, &ua, &ub, &hist, &scan, &segs, &sege, &segt, &cellev, &bwords, &smask, &ssat, &clist,
                            &segk0, &segk1, &segv0, &segv1, &state, &wlist, &act0, &act1, &words,
-                           &slist, &plist, &pmask, &whist};
+                           &slist, &plist, &pmask, &sstate, &whist};
     for (const DevBuf *b : all) key.push_back((uint64_t)(uintptr_t)b->p);
 }
 
@@ -246,8 +246,8 @@ void Workspace::release()
     if (cap_stream) cudaStreamDestroy(cap_stream);
     cap_stream = nullptr;
     DevBuf *all[] = {&cells_lohi, &cells, &vN, &recs, &boxes, &keys, &counters, &evk0, &evk1, &evv0, &evv1,
-                     &ents0, &ents1, &ente0, &ente1, &ua, &ub, &uc, &ud, &hist, &scan, &segs, &sege, &segt, &cellev, &bwords, &smask, &ssat, &clist, &segk0,
-                     &segk1, &segv0, &segv1, &state, &wlist, &act0, &act1, &words, &slist, &plist, &pmask, &whist, &out_lo,
+                     &ents0, &ents1, &ente0, &ente1, &ua, &ub, &hist, &scan, &segs, &sege, &segt, &cellev, &bwords, &smask, &ssat, &clist, &segk0,
+                     &segk1, &segv0, &segv1, &state, &wlist, &act0, &act1, &words, &slist, &plist, &pmask, &sstate, &whist, &out_lo,
                      &out_hi, &part_lo, &part_hi, &lvl_lo, &lvl_hi, &wpart};
     for (DevBuf *b : all) b->release();
     if (h_whist) cudaFreeHost(h_whist);
@@ -262,9 +262,9 @@ void Workspace::release()
 size_t Workspace::bytes() const
 {
     const DevBuf *all[] = {&cells_lohi, &cells, &vN, &recs, &boxes, &keys, &counters, &evk0, &evk1, &evv0, &evv1,
-                           &ents0, &ents1, &ente0, &ente1, &ua, &ub, &uc, &ud, &hist, &scan, &segs, &sege, &segt, &cellev, &bwords, &smask, &ssat, &clist,
+                           &ents0, &ents1, &ente0, &ente1, &ua, &ub, &hist, &scan, &segs, &sege, &segt, &cellev, &bwords, &smask, &ssat, &clist,
                            &segk0, &segk1, &segv0, &segv1, &state, &wlist, &act0, &act1, &words,
-                           &slist, &plist, &pmask, &whist, &out_lo, &out_hi, &part_lo, &part_hi, &lvl_lo, &lvl_hi, &wpart};
+                           &slist, &plist, &pmask, &sstate, &whist, &out_lo, &out_hi, &part_lo, &part_hi, &lvl_lo, &lvl_hi, &wpart};
     size_t s = 0;
     for (const DevBuf *b : all) s += b->cap;
     return s;
@@ -573,8 +573,6 @@ static int bin_pairs(Workspace &ws, const PixBox *boxes, const double *keys, uin
     RK(ws.ente1.ensure(sizeof(uint32_t) * (nent + 1)));
     RK(ws.ua.ensure(sizeof(uint32_t) * (nsc + 1)));
     RK(ws.ub.ensure(sizeof(uint32_t) * (nsc + 1)));
-    RK(ws.uc.ensure(sizeof(uint32_t) * (nsc + 1)));
-    RK(ws.ud.ensure(sizeof(uint32_t) * (nsc + 1)));
     RK(ws.hist.ensure(sizeof(uint32_t) * hist_words));
     RK(ws.scan.ensure(sizeof(uint32_t) * (scan_temp_words(scan_len) + 64)));
     RK(ws.segs.ensure(sizeof(uint32_t) * n_seg));
@@ -608,7 +606,6 @@ static int bin_pairs(Workspace &ws, const PixBox *boxes, const double *keys, uin
     ba.ent_seg[0] = ws.ents0.as<uint32_t>(); ba.ent_seg[1] = ws.ents1.as<uint32_t>();
     ba.ent_ev[0] = ws.ente0.as<uint32_t>(); ba.ent_ev[1] = ws.ente1.as<uint32_t>();
     ba.u32_a = ws.ua.as<uint32_t>(); ba.u32_b = ws.ub.as<uint32_t>();
-    ba.u32_c = ws.uc.as<uint32_t>(); ba.u32_d = ws.ud.as<uint32_t>();
     ba.hist = ws.hist.as<uint32_t>();
     ba.scan_tmp = ws.scan.as<uint32_t>();
     ba.seg_start = ws.segs.as<uint32_t>();
@@ -733,7 +730,8 @@ static int render_batch(ar_scene *s, Workspace &ws, const CallConst &cc, int M, 
         RK(ws.words.ensure(sizeof(uint32_t) * kRoundWords));
         RK(ws.slist.ensure(sizeof(uint32_t) * n_pairs));
         RK(ws.plist.ensure(sizeof(uint32_t) * n_seg));
-        RK(ws.pmask.ensure(sizeof(uint32_t) * n_seg * (TS * TS / 32 + 1)));  // pixel mask + a flag per slot
+        RK(ws.pmask.ensure(sizeof(uint32_t) * n_seg * (TS * TS / 32)));
+        RK(ws.sstate.ensure(sizeof(uint32_t) * 2 * n_seg));
     }
     // The rest of the batch (binning, then the windowed rounds of build and
     // render) depends on the host only through the sizes read above, so with
@@ -839,6 +837,7 @@ static int enqueue_rest(ar_scene *s, Workspace &ws, const CallConst &cc, int M, 
     rl.seg_total = bo.seg_total;
     rl.cell_ev = plain ? nullptr : ba.cell_ev;
     rl.W = W; rl.H = H; rl.ntx = ntx; rl.n_tiles = n_tiles; rl.n_cells = n_cells;
+    rl.n_entries = nent;
     rl.n_gauss = s->n;
     rl.k_open = s->k_open;
     rl.rel = s->blend == AR_BLEND_RELATIONAL;
@@ -861,7 +860,8 @@ static int enqueue_rest(ar_scene *s, Workspace &ws, const CallConst &cc, int M, 
                                ws.wlist.as<uint32_t>(), ws.act0.as<uint32_t>(), ws.act1.as<uint32_t>(),
                                ws.words.as<uint32_t>(), rl.counters + 2, q, &launches,
                                profiling ? ev + 3 : nullptr, ws.w0, ws.slist.as<uint32_t>(), ws.plist.as<uint32_t>(),
-                               ws.pmask.as<uint32_t>(), ws.segk0.as<uint32_t>(), bo.seg_total ? &ba : nullptr, &bo));
+                               ws.pmask.as<uint32_t>(), ws.segk0.as<uint32_t>(), ws.sstate.as<uint32_t>(),
+                               ws.sstate.as<uint32_t>() + n_seg, bo.seg_total ? &ba : nullptr, &bo));
     }
     return AR_OK;
 }
@@ -920,7 +920,8 @@ int run_windowed_render(int M, int TS, RenderLaunch rl, const CallConst &cc, con
                         uint64_t n_pairs, uint64_t n_seg, uint32_t *state, uint32_t *wlist, uint32_t *act0,
                         uint32_t *act1, uint32_t *words, unsigned long long *build_counters, cudaStream_t st,
                         int *launches, cudaEvent_t *ev, uint32_t w0, uint32_t *split_list, uint32_t *precise_list,
-                        uint32_t *precise_mask, uint32_t *precise_first, const BinArgs *rebin, const BinOut *first)
+                        uint32_t *precise_mask, uint32_t *precise_first, uint32_t *seg_state, uint32_t *seg_swept,
+                        const BinArgs *rebin, const BinOut *first)
 {
     // two phases: a segment restarts in the second round mostly because its
     // depth prefix ran out, so that round keeps the first window
@@ -929,7 +930,9 @@ int run_windowed_render(int M, int TS, RenderLaunch rl, const CallConst &cc, con
     const uint32_t *round1_order = nullptr;
     uint32_t *act[2] = {act0, act1};
     CK(cudaMemsetAsync(state, 0, sizeof(uint32_t) * n_pairs, st));
-    launch_init_words(words, (uint32_t)n_seg, st);
+    launch_init_rounds(words, (uint32_t)n_seg, seg_state, seg_swept, st);
+    rl.seg_state = seg_state;
+    rl.seg_swept = seg_swept;
     ++*launches;
     static const char *kRoundName[3] = {"ar.round 0: build + render", "ar.round 1: build + render",
                                         "ar.round 2: build + render"};
@@ -956,6 +959,7 @@ int run_windowed_render(int M, int TS, RenderLaunch rl, const CallConst &cc, con
         rl.precise_first = precise_first;
         rl.n_precise = reinterpret_cast<unsigned long long *>(cnt + 6);
         rl.work_fp64 = cnt + 5;
+        rl.round_no = r;
         rl.direct = rl.interleave && r == 0;
         if (launch_render(M, TS, rl, st))
             return fail(AR_EDEVICE, "render launch: %s", cudaGetErrorString(cudaGetLastError()));

@@ -36,13 +36,14 @@ constexpr size_t kMaxGraphs = 32;  // cached graphs per workspace (least recentl
 struct Workspace {
     DevBuf cells_lohi, cells, vN, recs, boxes, keys, counters;
     DevBuf evk0, evk1, evv0, evv1, ents0, ents1, ente0, ente1;
-    DevBuf ua, ub, uc, ud, hist, scan, segs, sege, segk0, segk1, segv0, segv1;
+    DevBuf ua, ub, hist, scan, segs, sege, segk0, segk1, segv0, segv1;
     DevBuf clist;                              // pairs left by the cull (then their count)
     bool cull_on = true;                       // the last render found culling worth it
     DevBuf segt, cellev, bwords, smask, ssat;  // two-phase binning: full-list lengths, cell event ranges,
                                                // counts, active mask and its summed-area tables
     DevBuf state, wlist, act0, act1, words, slist;  // windowed rounds: pair states, build list, active segments
-    DevBuf plist, pmask;                     // segments swept again with FP64 evaluations, their pixel masks
+    DevBuf plist, pmask;                     // segments swept again with FP64 evaluations, the pixel masks
+    DevBuf sstate;                           // [2][n_seg] the segments' state over the windowed rounds
     DevBuf whist;                            // [256] sweep-length histogram of the current render, then
                                              // [64] 64-bit: full-list entries by where the segments stopped
     uint32_t *h_whist = nullptr;             // page-locked copy of the last render's histogram
@@ -86,9 +87,10 @@ struct TunedTile {
 // split_list [n_pairs]: pairs whose MatrixInv needs input splitting or a high
 // order, which a last kernel finishes; precise_list [n_seg]: segments that
 // meet an opacity evaluation needing FP64, swept again by the FP64-capable
-// render instance in the same round, and precise_mask [n_seg * (TS * TS / 32 + 1)]
-// the pixels of each that do, precise_first [n_seg] its first work item (the
-// binning's seg_k[0], free once the schedule is sorted).
+// render instance in the same round, and precise_mask [n_seg * TS * TS / 32]
+// the pixels of each segment that do, precise_first [n_seg] its first work item (the
+// binning's seg_k[0], free once the schedule is sorted); seg_state, seg_swept [n_seg]
+// (zeroed here): the segments' state over the rounds.
 // rebin / first: the binning of a two-phase render, whose second phase runs
 // between the first and the second round (null: one phase, lists complete)
 struct BinArgs;
@@ -97,7 +99,8 @@ int run_windowed_render(int M, int TS, RenderLaunch rl, const CallConst &cc, con
                         uint64_t n_pairs, uint64_t n_seg, uint32_t *state, uint32_t *wlist, uint32_t *act0,
                         uint32_t *act1, uint32_t *words, unsigned long long *build_counters, cudaStream_t st,
                         int *launches, cudaEvent_t *ev, uint32_t w0, uint32_t *split_list, uint32_t *precise_list,
-                        uint32_t *precise_mask, uint32_t *precise_first, const BinArgs *rebin = nullptr, const BinOut *first = nullptr);
+                        uint32_t *precise_mask, uint32_t *precise_first, uint32_t *seg_state, uint32_t *seg_swept,
+                        const BinArgs *rebin = nullptr, const BinOut *first = nullptr);
 // Depth prefix of the next render's first binning phase, from the stop
 // histograms of an earlier render (64 buckets of full-list entries, and of
 // segments, by where in its cell's depth order a segment stopped): the shift

@@ -29,6 +29,7 @@ struct RenderLaunch {
                                       // depth order they stopped, and [64] their counts
     const uint64_t *ev_key;
     int W, H, ntx, n_tiles, n_cells;
+    uint64_t n_entries = 0;           // of the segments' full lists
     int64_t n_gauss;
     float k_open;                     // 1 / (1 - largest opacity), rounded up
     float fp64_dev = 3.0e38f;         // opacity evaluations whose FP32 deviation estimate exceeds this
@@ -41,13 +42,17 @@ struct RenderLaunch {
     int rel = 0;                      // 1: relational upper transmittance (AR_BLEND_RELATIONAL)
     int ch = 16;                      // events per staged chunk of the FP32 sweep (8, 16 or 32 at tile 16)
     // interleave: the first round's FP32 sweep (whose active list is all n_seg
-    // segments) launches one CTA per segment (direct) instead of persistent
+    // segments) launches one CTA per work item (direct) instead of persistent
     // CTAs, so that work on a higher-priority stream can take SMs as they free
     int interleave = 0, direct = 0;
+    // the windowed rounds' state of the segments, zeroed before the first (see
+    // render_kernel), and the most entries that a part of each swept
+    int round_no = 0;
+    uint32_t *seg_state = nullptr, *seg_swept = nullptr;
     // precision: the FP32 sweep appends a segment that needs an FP64
     // evaluation to precise, with the mask of the pixels that do in
-    // precise_mask[slot * (TS * TS / 32 + 1) ...] (then a flag word) and the
-    // number of its first work item in precise_first; *n_precise: the segments
+    // precise_mask[segment * TS * TS / 32 ...] and the number of its first
+    // work item in precise_first; *n_precise: the segments
     // (high word) and their work items; render_fp64_kernel takes them
     // (work_fp64: its item counter)
     uint32_t *precise = nullptr, *precise_mask = nullptr, *precise_first = nullptr;

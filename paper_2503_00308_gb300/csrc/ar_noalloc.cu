@@ -156,7 +156,7 @@ int ar_render_abstract_noalloc(ar_scene *s, const ar_intrinsics *in, const ar_no
     uint32_t *state = A.take<uint32_t>(n_pairs), *wlist = A.take<uint32_t>(n_pairs);
     uint32_t *slist = A.take<uint32_t>(n_pairs);
     uint32_t *act0 = A.take<uint32_t>(n_seg), *act1 = A.take<uint32_t>(n_seg), *words = A.take<uint32_t>(kRoundWords);
-    uint32_t *plist = A.take<uint32_t>(n_seg), *pmask = A.take<uint32_t>(n_seg * (TS * TS / 32 + 1));
+    uint32_t *plist = A.take<uint32_t>(n_seg), *pmask = A.take<uint32_t>(n_seg * (TS * TS / 32));
     if (A.over) return too_big("the per-(Gaussian, cell) records", A.used);
 
     // pose cells: lo and hi rows straight from the caller's array (no staging copy)
@@ -197,8 +197,6 @@ int ar_render_abstract_noalloc(ar_scene *s, const ar_intrinsics *in, const ar_no
     }
     ba.u32_a = A.take<uint32_t>(nsc + 1);
     ba.u32_b = A.take<uint32_t>(nsc + 1);
-    ba.u32_c = A.take<uint32_t>(nsc + 1);
-    ba.u32_d = A.take<uint32_t>(nsc + 1);
     ba.hist = A.take<uint32_t>(hist_words);
     ba.scan_tmp = A.take<uint32_t>(scan_temp_words(scan_len) + 64);
     ba.seg_start = seg_start;
@@ -219,6 +217,7 @@ int ar_render_abstract_noalloc(ar_scene *s, const ar_intrinsics *in, const ar_no
     rl.ev_val = bo.ev_val;
     rl.ev_key = bo.ev_key;
     rl.W = W; rl.H = H; rl.ntx = ntx; rl.n_tiles = n_tiles; rl.n_cells = n_cells;
+    rl.n_entries = nent;
     rl.n_gauss = s->n;
     rl.k_open = s->k_open;
     rl.rel = s->blend == AR_BLEND_RELATIONAL;
@@ -227,6 +226,7 @@ int ar_render_abstract_noalloc(ar_scene *s, const ar_intrinsics *in, const ar_no
     rl.out_lo = out_lower;
     rl.out_hi = out_upper;
     rl.counters = nullptr;
+    // (the schedule ends in seg_v1: its other buffers hold the rounds' state)
     return run_windowed_render(M, TS, rl, cc, cellbuf, vN, n_pairs, n_seg, state, wlist, act0, act1, words, nullptr,
-                               st, &launches, nullptr, 512u, slist, plist, pmask, seg_k0);
+                               st, &launches, nullptr, 512u, slist, plist, pmask, seg_k0, seg_k1, seg_v0);
 }

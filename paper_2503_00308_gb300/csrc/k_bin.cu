@@ -954,9 +954,9 @@ int run_binning(const BinArgs &a, BinOut &o, cudaStream_t st, int *launches)
         o.ent_ev = a.ent_ev[0];
         cudaMemsetAsync(a.seg_start, 0, sizeof(uint32_t) * a.n_segments, st);
         cudaMemsetAsync(a.seg_end, 0, sizeof(uint32_t) * a.n_segments, st);
-        iota_kernel<<<blocks_for(a.n_segments, T), T, 0, st>>>(a.seg_v[0], a.n_segments);
+        iota_kernel<<<blocks_for(a.n_segments, T), T, 0, st>>>(a.seg_v[1], a.n_segments);
         ++*launches;
-        o.seg_order = a.seg_v[0];
+        o.seg_order = a.seg_v[1];  // where a sorted one ends
         return cudaGetLastError() == cudaSuccess ? 0 : 1;
     }
     // the first phase bins only each cell's depth prefix (see in_prefix): the
@@ -1105,8 +1105,16 @@ int run_rebin(const BinArgs &a, const BinOut &first, const uint32_t *active, con
 
 // ------------------------------------------------------------ windowed rounds
 // every counter of the windowed rounds in one launch (they were fifteen
-// memsets, a tenth of a small render's graph)
-__global__ void init_words_kernel(uint32_t *words, uint32_t v) { words[threadIdx.x] = threadIdx.x ? 0u : v; }
+// memsets, a tenth of a small render's graph), and the segments' state
+__global__ void init_rounds_kernel(uint32_t *words, uint32_t n_seg, uint32_t *seg_state, uint32_t *seg_swept)
+{
+    const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    if (i < 32) words[i] = i ? 0u : n_seg;
+    if (i < n_seg) {
+        seg_state[i] = 0u;
+        seg_swept[i] = 0u;
+    }
+}
 
 // For each active segment, the lower endpoints among its first `window`
 // entries: every pair not yet claimed (state 0 -> 1) is appended to work.
@@ -1147,7 +1155,10 @@ __global__ void __launch_bounds__(256) demand_kernel(const uint32_t *__restrict_
     }
 }
 
-void launch_init_words(uint32_t *words, uint32_t v, cudaStream_t st) { init_words_kernel<<<1, 32, 0, st>>>(words, v); }
+void launch_init_rounds(uint32_t *words, uint32_t n_seg, uint32_t *seg_state, uint32_t *seg_swept, cudaStream_t st)
+{
+    init_rounds_kernel<<<blocks_for((uint64_t)n_seg + 32, 256), 256, 0, st>>>(words, n_seg, seg_state, seg_swept);
+}
 
 void launch_demand(const uint32_t *active, const uint32_t *n_active, uint32_t max_active, const uint32_t *seg_start,
                    const uint32_t *seg_end, const uint32_t *ent_ev, const uint32_t *ev_val, uint32_t window,

@@ -81,38 +81,54 @@ int AR_CAT(launch_render_plain_m, AR_M)(int TS, const RenderLaunch &a, cudaStrea
     return TS == 16 ? launch_render_plain_ts<16>(a, st) : launch_render_plain_ts<8>(a, st);
 }
 
-template <int TS, bool REL, int CH = 16>
-static int launch_render_ts(const RenderLaunch &a, cudaStream_t st)
+template <int TS, bool REL, int CH, int PARTS>
+static int launch_render_parts(const RenderLaunch &a, cudaStream_t st)
 {
     // double-buffered chunks of CH events (16 unless the autotuner picks 8 or
     // 32 at tile 16: the exit vote, taken once per chunk,
-    // stops a tile sooner with short chunks, while long chunks take fewer
+    // stops a part sooner with short chunks, while long chunks take fewer
     // barriers) and a ring of 4 (rings of 3-8 measured: 4 keeps the ring's
     // shared memory small)
-    constexpr int RING = 4;
-    typedef RenderSmem<AR_M, TS, CH, RING> SM;
-    auto kern = render_kernel<AR_M, TS, CH, RING, REL>;
+    constexpr int RING = 4, NT = Part<TS, PARTS>::NT;
+    typedef RenderSmem<AR_M, NT, CH, RING> SM;
+    auto kern = render_kernel<AR_M, TS, CH, RING, REL, PARTS>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::BYTES) != cudaSuccess)
         return 1;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SM::NT, SM::BYTES) != cudaSuccess || per_sm < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, SM::BYTES) != cudaSuccess || per_sm < 1)
         per_sm = 1;
-    const uint32_t nseg = (uint32_t)a.n_cells * (uint32_t)a.n_tiles;
+    // work items: the parts of every segment
+    const uint64_t items = (uint64_t)a.n_cells * (uint64_t)a.n_tiles * PARTS;
     uint32_t grid = (uint32_t)(sms * per_sm);
-    if (grid > nseg) grid = nseg;
-    // direct launches (a.direct: the active list holds all nseg segments) take
-    // one CTA per segment
-    if (a.direct) grid = nseg;
-    kern<<<grid, SM::NT, SM::BYTES, st>>>(a.recs, a.boxes, a.seg_start, a.seg_end, a.seg_total, a.cell_ev,
-                                           a.active, a.n_active,
-                                           a.window,
-                                           a.next_active, a.n_next, a.precise, a.n_precise, a.precise_mask, a.precise_first, a.sweep_hist,
-                                           a.ent_ev, a.ev_val,
-                                           a.ev_key, a.W, a.H, a.ntx, a.n_tiles, a.n_gauss, a.k_open, a.fp64_dev, a.out_lo,
-                                           a.out_hi, a.counters, a.work, a.direct);
+    if (grid > items) grid = (uint32_t)items;
+    // direct launches (a.direct: the active list holds every segment) take
+    // one CTA per item
+    if (a.direct) grid = (uint32_t)items;
+    kern<<<grid, NT, SM::BYTES, st>>>(a.recs, a.boxes, a.seg_start, a.seg_end, a.seg_total, a.cell_ev,
+                                      a.active, a.n_active, a.window, a.round_no,
+                                      a.next_active, a.n_next, a.seg_state, a.seg_swept, a.precise, a.n_precise,
+                                      a.precise_mask, a.precise_first, a.sweep_hist, a.ent_ev, a.ev_val,
+                                      a.ev_key, a.W, a.H, a.ntx, a.n_tiles, a.n_gauss, a.k_open, a.fp64_dev, a.out_lo,
+                                      a.out_hi, a.counters, a.work, a.direct);
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
+}
+
+// the parts of a tile that a render sweeps, over all its rounds (see Part; the
+// grid of a direct launch has one CTA per part, so their number stays below 2^31)
+static int render_parts(int TS, const RenderLaunch &a)
+{
+    const uint64_t n_seg = (uint64_t)a.n_cells * (uint64_t)a.n_tiles;
+    return TS == 16 && n_seg >= HALVES_SEGMENTS && n_seg < (1ull << 30) && a.n_entries >= HALVES_ENTRIES * n_seg ? 2 : 1;
+}
+
+template <int TS, bool REL, int CH = 16>
+static int launch_render_ts(const RenderLaunch &a, cudaStream_t st)
+{
+    if constexpr (TS == 16)
+        if (render_parts(TS, a) == 2) return launch_render_parts<TS, REL, CH, 2>(a, st);
+    return launch_render_parts<TS, REL, CH, 1>(a, st);
 }
 
 // the FP64-capable sweep of the segments listed in a.precise (it stages 16
@@ -133,7 +149,8 @@ static int launch_render_fp64_ts(const RenderLaunch &a, cudaStream_t st)
     uint32_t grid = (uint32_t)(sms * per_sm);
     if (grid > items) grid = (uint32_t)items;
     kern<<<grid, 32, sizeof(SM), st>>>(a.recs, a.boxes, a.seg_start, a.seg_end, a.seg_total, a.precise,
-                                       a.precise_first, a.n_precise, a.window, a.next_active, a.n_next, a.precise_mask, a.ent_ev, a.ev_val, a.ev_key,
+                                       a.precise_first, a.n_precise, a.seg_state, render_parts(TS, a), a.window,
+                                       a.round_no, a.next_active, a.n_next, a.precise_mask, a.ent_ev, a.ev_val, a.ev_key,
                                        a.W, a.H, a.ntx, a.n_tiles, a.n_gauss, a.k_open, a.fp64_dev, a.out_lo, a.out_hi,
                                        a.counters, a.work_fp64);
     return cudaGetLastError() == cudaSuccess ? 0 : 1;

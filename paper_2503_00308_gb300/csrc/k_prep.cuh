@@ -1252,7 +1252,7 @@ __global__ void __launch_bounds__(128, 5) record_prep_list_kernel(
 // 198 / 259, 18291 377 / 398, 27693 459 / 404, 76970 941 / 683.
 constexpr uint32_t COOP_MAX = 20480;
 
-// Forms of a group in shared memory, COOP_FORM<M> doubles each: c[M], klo, khi,
+// Forms of a group in shared memory, Coop<M>::FORM doubles each: c[M], klo, khi,
 // r, vlo, vhi.  (v - s takes the slots of X, Conic those of J.)
 template <int M> struct Coop {
     static constexpr int FORM = M + 5;

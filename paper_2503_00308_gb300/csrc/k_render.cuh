@@ -599,8 +599,31 @@ __device__ __forceinline__ float open_ratio_up(float a)
     return den > 0.f ? __fmul_ru(__fdividef(a, den), 1.000000477f) : 3.0e38f;
 }
 
-// Shared-memory layout of the render kernel (dynamic; about 70 KB at six
-// pose variables, tile 16, chunks of 16 and a ring of 4, so two CTAs fit on an SM):
+// A CTA sweeps a tile, or at tile 16 one of its two 16 x 8 halves (PARTS = 2).
+// The warps of a CTA meet at a barrier per chunk, and one whose pixels have
+// stopped waits there for the others: halves lose less to that (a fifth of the
+// warps' time with eight warps), but stage every chunk twice and join their ends
+// through a word per segment.  So a half suits many segments with work to do
+// (HALVES_*), a whole tile few segments, whose CTAs have an SM to
+// themselves, and short lists.  The render stage, whole / halves: 16 narrow
+// cells of the 300k scene 85.6 / 82.6 ms, 64 cells of it 48.3 / 47.0, 32 cells of
+// 10k at 400 x 300 3.14 / 2.99; 36 segments of 200k Gaussians 15.7 / 16.5 ms,
+// 2650 segments of 350 Gaussians 60 / 67 us.
+// (16 warps per SM at 128 registers, a few spills: halves at 168 registers and
+// 12 warps took 88.2 ms on the first.  8 x 8 parts took 86.4, and warps alone,
+// without a barrier but each staging its own records, 88.6.)
+// At tile 8, six CTAs of two warps: unlimited, 225 registers let four fit, and
+// the render stage of 16 cells of 10k Gaussians took 0.73 ms against 0.61.
+template <int TS, int PARTS> struct Part {
+    static constexpr int H = TS / PARTS;  // its rows
+    static constexpr int NT = TS * H;     // threads
+    static constexpr int CTAS = TS == 16 ? 2 * PARTS : 6;  // per SM
+};
+// a render takes halves with at least this many segments, and this many entries
+// per segment on average
+constexpr uint64_t HALVES_SEGMENTS = 152, HALVES_ENTRIES = 64;
+// Shared-memory layout (dynamic; about 70 KB at six pose variables, 256 threads,
+// chunks of 16 and a ring of 4, so two CTAs fit on an SM):
 //   two buffers, each with the records staged for
 //   a chunk of CH events, their event info and pixel boxes (the next chunk is
 //   copied in while the current one is swept),
@@ -609,8 +632,7 @@ __device__ __forceinline__ float open_ratio_up(float a)
 //   stored column-per-thread so that every access is bank-conflict free.  The ring lets the upper endpoint of
 //   a Gaussian reuse the evaluation made at its lower endpoint; an upper
 //   endpoint whose evaluation has left the ring evaluates again.
-template <int M, int TS, int CH, int RING> struct RenderSmem {
-    static constexpr int NT = TS * TS;
+template <int M, int NT, int CH, int RING> struct RenderSmem {
     static constexpr int NBUF = 2;
     static constexpr int PAY = M + 4;  // alo, ahi, rL, L.k, L.c[M]
     static constexpr int PV = (PAY + 3) / 4;  // ... as 16-byte vectors (the last one padded)
@@ -638,50 +660,51 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// Two 256-thread CTAs share an SM (16 warps: the sweep is latency-bound, and
-// 128 registers per thread cost it a few spills but double the warps that hide
-// the FMA latency).  Six 64-thread CTAs: at 225 registers four fitted, and the
-// render stage of 16 cells of 10k Gaussians took 0.73 ms against 0.61.
-template <int TS> struct RenderOcc {
-    static constexpr int MIN_BLOCKS = TS * TS >= 256 ? 2 : 6;
-};
 // pixels per work item of the FP64 sweep
 constexpr int PRECISE_PX = 8;
-// words per listed segment of the FP64 sweep: the pixel mask, the abandon flag
+// words per segment of the FP64 sweep's pixel mask
 template <int TS> struct PreciseMask {
-    static constexpr int WORDS = TS * TS / 32 + 1;
+    static constexpr int WORDS = TS * TS / 32;
 };
+// A segment's state word over the windowed rounds (zeroed before the first): its
+// parts that have ended this round (low byte), the parts that are complete (a
+// bit each from SEG_DONE on), and the rounds in which it was listed for the next
+// (a bit each from SEG_LISTED on).
+constexpr int SEG_DONE = 8, SEG_LISTED = 16;
 
-// Persistent grid: each CTA takes (cell, tile) segments from the active list
-// (longest first in the first round) through an atomic counter until none
-// are left; block = TS*TS threads.
+// Persistent grid: each CTA takes work items, (segment, part), from the active
+// list of (cell, tile) segments (longest first in the first round) through an
+// atomic counter until none are left.
 //
 // Windowed rounds: only the records of the pairs whose lower endpoints lie in
 // the first `window` entries of an active segment have been built.  A
-// segment that would stage an entry beyond its window before all its pixels
-// have stopped is abandoned (no output written) and appended to next_active;
-// the next round builds the records of a wider window and sweeps it again
-// from its start.  The sweep is deterministic, so the restarted segment
-// gives the same bounds it would have given in one pass.
+// part that would stage an entry beyond its window before all its pixels
+// have stopped is abandoned (no output written); the last of a segment's parts
+// to end appends it to next_active if one was, and
+// the next round builds the records of a wider window and sweeps the parts that
+// are not complete again from their start.  The sweep is deterministic, so the
+// restarted part gives the same bounds it would have given in one pass.
 //
 // Precision: the opacity evaluations whose weighted FP32 deviation
 // estimate exceeds fp64_dev are taken in FP64 (pixel_alpha_fp64).  This FP32
 // sweep keeps that out-of-line call out of its code: it sweeps
-// every segment in FP32, writes the bounds of the pixels that met no such
-// evaluation, and appends a segment where some pixel did to precise_list,
-// with the mask of those pixels (one word per warp) in precise_mask.
+// every part in FP32, writes the bounds of the pixels that met no such
+// evaluation, and leaves the mask of those that did in precise_mask (one word
+// per warp); the last of a segment's parts to end appends the segment to
+// precise_list if it has any.
 // render_fp64_kernel sweeps the listed segments again from their start for
 // the masked pixels alone.
 // The decision is per pixel, taken from the pixel's own sweep, so every pixel
 // gets the bounds one FP64-capable sweep would give it.
-template <int M, int TS, int CH, int RING, bool REL>
-__global__ void __launch_bounds__(TS *TS, RenderOcc<TS>::MIN_BLOCKS) render_kernel(
+template <int M, int TS, int CH, int RING, bool REL, int PARTS>
+__global__ void __launch_bounds__(Part<TS, PARTS>::NT, Part<TS, PARTS>::CTAS) render_kernel(
     const float *__restrict__ recs, const PixBox *__restrict__ boxes, const uint32_t *__restrict__ seg_start,
     const uint32_t *__restrict__ seg_end, const uint32_t *__restrict__ seg_total,
     const uint32_t *__restrict__ cell_ev, const uint32_t *__restrict__ active, const uint32_t *__restrict__ n_active,
-    uint32_t window, uint32_t *__restrict__ next_active, uint32_t *__restrict__ n_next,
+    uint32_t window, int round_no, uint32_t *__restrict__ next_active, uint32_t *__restrict__ n_next,
+    uint32_t *seg_state, uint32_t *seg_swept,
     uint32_t *__restrict__ precise_list, unsigned long long *__restrict__ n_precise,
-    uint32_t *__restrict__ precise_mask, uint32_t *__restrict__ precise_first,
+    uint32_t *precise_mask, uint32_t *__restrict__ precise_first,
     uint32_t *__restrict__ sweep_hist,
     const uint32_t *__restrict__ entry_ev, const uint32_t *__restrict__ ev_val,
     const uint64_t *__restrict__ ev_key, int W, int H, int ntx, int n_tiles, int64_t n_gauss,
@@ -689,37 +712,38 @@ __global__ void __launch_bounds__(TS *TS, RenderOcc<TS>::MIN_BLOCKS) render_kern
     unsigned long long *__restrict__ counters, unsigned int *__restrict__ work, int direct)
 {
     using RL = Rec<M>;
-    using SM = RenderSmem<M, TS, CH, RING>;
-    constexpr int NT = SM::NT;  // threads, the pixels of a tile
+    constexpr int NT = Part<TS, PARTS>::NT;
+    using SM = RenderSmem<M, NT, CH, RING>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float(*s_rec2)[RL::WIDTH] = reinterpret_cast<float(*)[RL::WIDTH]>(smem_raw);        // [2 * CH]
     EvInfo *s_ev2 = reinterpret_cast<EvInfo *>(smem_raw + SM::REC);                    // [2 * CH]
     PixBox *s_box2 = reinterpret_cast<PixBox *>(smem_raw + SM::REC + SM::EV);          // [2 * CH]
     uint32_t *s_rid = reinterpret_cast<uint32_t *>(smem_raw + SM::REC + SM::EV + SM::BOX);
     float4 *s_pay = reinterpret_cast<float4 *>(smem_raw + SM::REC + SM::EV + SM::BOX + SM::RID);
-    uint32_t *s_next = reinterpret_cast<uint32_t *>(smem_raw + SM::REC + SM::EV + SM::BOX + SM::RID + SM::RPAY);
+    uint32_t *s_next =
+        reinterpret_cast<uint32_t *>(smem_raw + SM::REC + SM::EV + SM::BOX + SM::RID + SM::RPAY);
     const int tid = threadIdx.x;
     uint32_t evals = 0, recomp = 0;
-    const uint32_t n_seg = *n_active;
+    const uint32_t n_items = *n_active * PARTS;
 
-    // direct: one CTA per active segment (the grid covers them all), so that
+    // direct: one CTA per work item (the grid covers them all), so that
     // CTAs finish one by one and a higher-priority stream's work can take
-    // their SMs; else persistent CTAs take segments from the work counter
+    // their SMs; else persistent CTAs take items from the work counter
     for (uint32_t round = 0;; ++round) {
         if (tid == 0) *s_next = direct ? (round == 0 ? blockIdx.x : 0xffffffffu) : atomicAdd(work, 1u);
         __syncthreads();
-        const uint32_t wk = *s_next;
+        const uint32_t item = *s_next;
         __syncthreads();
-        if (wk >= n_seg) break;
-        const uint32_t seg = active[wk];
+        if (item >= n_items) break;
+        const uint32_t seg = active[item / PARTS], part = item % PARTS;
         const int cell = (int)(seg / (uint32_t)n_tiles);
         const int tile = (int)(seg - (uint32_t)cell * (uint32_t)n_tiles);
         const int tx = tile % ntx, ty = tile / ntx;
-        // each warp covers an 8 x 4 block of the tile, so that the pixel boxes
+        // each warp covers an 8 x 4 block of the part, so that the pixel boxes
         // of small Gaussians cut fewer warps and warps finish together
         const int wb = tid >> 5, ln = tid & 31;
         const int px = tx * TS + (wb % (TS / 8)) * 8 + (ln & 7);
-        const int py = ty * TS + (wb / (TS / 8)) * 4 + (ln >> 3);
+        const int py = ty * TS + (int)part * Part<TS, PARTS>::H + (wb / (TS / 8)) * 4 + (ln >> 3);
         const bool inside = px < W && py < H;
         const float ux = px + 0.5f, uy = py + 0.5f;
         const uint32_t b0 = seg_start[seg], b1 = seg_end[seg];
@@ -800,13 +824,14 @@ __global__ void __launch_bounds__(TS *TS, RenderOcc<TS>::MIN_BLOCKS) render_kern
         // mostly short (sparse tiles), and a sweep of their prefix would be
         // done twice
         if (incomplete && total <= SHORT_DEFER) abandoned = true;
-        if (b0 < b1 && !abandoned) stage(0, b0);
+        const bool complete = PARTS > 1 && round_no > 0 && (__ldcg(seg_state + seg) >> (SEG_DONE + part)) & 1u;  // in an earlier round
+        if (b0 < b1 && !abandoned && !complete) stage(0, b0);
         // a complete list ends the sweep when it runs out; a prefix only when
         // every pixel has stopped, or by abandoning the segment at the first
         // chunk it does not hold in full (the next binning phase gives the
         // segment its full list, and the sweep starts again: the exit tests
         // fall at the same entries, so the bounds are those of one sweep)
-        for (uint32_t base = b0; !abandoned && (base < b1 || incomplete); base += CH, buf ^= 1) {
+        for (uint32_t base = b0; !abandoned && !complete && (base < b1 || incomplete); base += CH, buf ^= 1) {
             if (!done) {
                 const float left = (float)(total - (base - b0));
                 // PA is rounded down; 1.01 covers its relative error for < 10^5 factors
@@ -958,42 +983,75 @@ __global__ void __launch_bounds__(TS *TS, RenderOcc<TS>::MIN_BLOCKS) render_kern
                 }
             }
         }
-        if (abandoned) {
-            if (tid == 0) {
-                next_active[atomicAdd(n_next, 1u)] = seg;
-                if (counters) atomicAdd(&counters[5], 1ull);
-            }
-            continue;
-        }
-        if (const int n_wide = __syncthreads_count(wide_hit)) {
-            // list the segment with the mask of its pixels that need FP64; a
-            // work item takes PRECISE_PX of them
-            // (the slot goes through s_next[1]: s_next[0], the work index, is
-            // rewritten at the next segment's start while others may read this)
-            if (tid == 0) {
-                const uint32_t parts = (uint32_t)(n_wide + PRECISE_PX - 1) / PRECISE_PX;
-                const unsigned long long at = atomicAdd(n_precise, (1ull << 32) | parts);
-                const uint32_t slot = (uint32_t)(at >> 32);
-                precise_list[slot] = seg;
-                precise_first[slot] = (uint32_t)at;  // (ascending: slots and items are taken together)
-                precise_mask[(size_t)slot * PreciseMask<TS>::WORDS + TS * TS / 32] = 0u;  // the FP64 sweep's abandon flag
-                s_next[1] = slot;
-                if (counters) atomicAdd(&counters[7], 1ull);
-            }
-            __syncthreads();
-            const uint32_t m = __ballot_sync(0xffffffffu, wide_hit);
-            if ((tid & 31) == 0) precise_mask[(size_t)s_next[1] * PreciseMask<TS>::WORDS + (tid >> 5)] = m;
-        }
-        if (sweep_hist && tid == 0) atomicAdd(&sweep_hist[min(swept / 32u, 255u)], 1u);
         // where in its cell's depth order the segment stopped (64 buckets of
-        // the cell's sorted events), weighted by its full length and counted:
-        // the host sizes the next render's depth prefix from them
-        if (sweep_hist && cell_ev && tid == 0 && b1 > b0) {
-            const uint32_t c0 = cell_ev[cell], ec = cell_ev[cell + 1] - c0;
-            const uint32_t stop = entry_ev[b0 + (swept ? swept : 1u) - 1u];
-            const uint32_t bkt = ec ? (uint32_t)min((uint64_t)(stop - c0) * 64u / ec, (uint64_t)63) : 0u;
-            atomicAdd(reinterpret_cast<unsigned long long *>(sweep_hist + 256) + bkt, (unsigned long long)total);
-            atomicAdd(sweep_hist + 384 + bkt, 1u);
+        // the cell's sorted events), weighted by its full length and counted,
+        // and the entries it swept: the host sizes the next render's depth
+        // prefix and first window from them
+        auto count_stop = [&](uint32_t most) {
+            atomicAdd(&sweep_hist[min(most / 32u, 255u)], 1u);
+            if (cell_ev && b1 > b0) {
+                const uint32_t c0 = cell_ev[cell], ec = cell_ev[cell + 1] - c0;
+                const uint32_t stop = entry_ev[b0 + (most ? most : 1u) - 1u];
+                const uint32_t bkt = ec ? (uint32_t)min((uint64_t)(stop - c0) * 64u / ec, (uint64_t)63) : 0u;
+                atomicAdd(reinterpret_cast<unsigned long long *>(sweep_hist + 256) + bkt, (unsigned long long)total);
+                atomicAdd(sweep_hist + 384 + bkt, 1u);
+            }
+        };
+        // list the segment for the next round
+        auto list_next = [&]() {
+            next_active[atomicAdd(n_next, 1u)] = seg;
+            if (counters) atomicAdd(&counters[5], 1ull);
+        };
+        // list the segment for the FP64 sweep, a work item of which takes
+        // PRECISE_PX of its n pixels
+        auto list_precise = [&](uint32_t n) {
+            const unsigned long long at = atomicAdd(n_precise, (1ull << 32) | ((n + PRECISE_PX - 1) / PRECISE_PX));
+            precise_list[(uint32_t)(at >> 32)] = seg;
+            precise_first[(uint32_t)(at >> 32)] = (uint32_t)at;  // (ascending: both are taken together)
+            if (counters) atomicAdd(&counters[7], 1ull);
+        };
+        uint32_t *mask = precise_mask + (size_t)seg * PreciseMask<TS>::WORDS + part * (NT / 32);  // a word per warp
+        if (PARTS == 1) {
+            if (abandoned) {
+                if (tid == 0) list_next();
+                continue;
+            }
+            if (const int n_wide = __syncthreads_count(wide_hit)) {
+                const uint32_t m = __ballot_sync(0xffffffffu, wide_hit);
+                if (ln == 0) mask[wb] = m;
+                if (tid == 0) list_precise((uint32_t)n_wide);
+            }
+            if (sweep_hist && tid == 0) count_stop(swept);
+        } else {
+            const uint32_t m = __ballot_sync(0xffffffffu, wide_hit && !abandoned);
+            if (ln == 0) mask[wb] = m;
+            __syncthreads();
+            if (tid == 0) {
+                const bool now = !abandoned && !complete;
+                if (now) atomicMax(seg_swept + seg, swept);
+                __threadfence();
+                // ended, and complete (added once: a complete part is not swept again)
+                const uint32_t mine = 1u + (now ? 1u << (SEG_DONE + part) : 0u);
+                const uint32_t state = atomicAdd(seg_state + seg, mine) + mine;
+                if ((state & 255u) == PARTS) {
+                    // the last of the segment's parts to end
+                    __threadfence();
+                    constexpr uint32_t ALL = (1u << PARTS) - 1u;
+                    const bool whole = ((state >> SEG_DONE) & ALL) == ALL;
+                    // (ended: 0 for the next round; the FP64 sweep may list the segment too)
+                    seg_state[seg] = (state & ~255u) | (whole ? 0u : 1u << (SEG_LISTED + round_no));
+                    uint32_t n_wide = 0;
+#pragma unroll
+                    for (int w = 0; w < PreciseMask<TS>::WORDS / 4; ++w) {
+                        const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(precise_mask + (size_t)seg * PreciseMask<TS>::WORDS) + w);
+                        n_wide += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+                    }
+                    if (n_wide) list_precise(n_wide);
+                    if (!whole) list_next();
+                    else if (sweep_hist) count_stop(__ldcg(seg_swept + seg));
+                }
+            }
+            if (abandoned || complete) continue;
         }
         evals += seg_evals;
         recomp += seg_recomp;
@@ -1052,6 +1110,7 @@ template <int M, int CH, int RING> struct PreciseSmem {
     EvInfo ev[CH];
     uint32_t rid[RING][PX];
     float ux[PX], uy[PX];
+    uint32_t redo;                                   // the parts of the tile to sweep again, should the item be abandoned
     uint8_t pair[PAIRS], slot[PAIRS];                // pair i's (entry, pixel) and the inverse
 };
 
@@ -1060,8 +1119,9 @@ __global__ void __launch_bounds__(32, 11) render_fp64_kernel(
     const float *__restrict__ recs, const PixBox *__restrict__ boxes, const uint32_t *__restrict__ seg_start,
     const uint32_t *__restrict__ seg_end, const uint32_t *__restrict__ seg_total,
     const uint32_t *__restrict__ listed, const uint32_t *__restrict__ first_item,
-    const unsigned long long *__restrict__ n_listed, uint32_t window, uint32_t *__restrict__ next_active, uint32_t *__restrict__ n_next,
-    uint32_t *__restrict__ precise_mask, const uint32_t *__restrict__ entry_ev, const uint32_t *__restrict__ ev_val,
+    const unsigned long long *__restrict__ n_listed, uint32_t *__restrict__ seg_state, int parts, uint32_t window,
+    int round_no, uint32_t *__restrict__ next_active, uint32_t *__restrict__ n_next,
+    const uint32_t *__restrict__ precise_mask, const uint32_t *__restrict__ entry_ev, const uint32_t *__restrict__ ev_val,
     const uint64_t *__restrict__ ev_key, int W, int H, int ntx, int n_tiles, int64_t n_gauss,
     float k_open, float fp64_dev, float *__restrict__ out_lo, float *__restrict__ out_hi,
     unsigned long long *__restrict__ counters, unsigned int *__restrict__ work)
@@ -1091,7 +1151,7 @@ __global__ void __launch_bounds__(32, 11) render_fp64_kernel(
         }
         const uint32_t part = at - first_item[wk];
         const uint32_t seg = listed[wk];
-        uint32_t *pm = precise_mask + (size_t)wk * PreciseMask<TS>::WORDS;
+        const uint32_t *pm = precise_mask + (size_t)seg * PreciseMask<TS>::WORDS;
         const int cell = (int)(seg / (uint32_t)n_tiles);
         const int tile = (int)(seg - (uint32_t)cell * (uint32_t)n_tiles);
         // lane l: the listed pixel of rank PX part + (l mod PX)
@@ -1107,6 +1167,10 @@ __global__ void __launch_bounds__(32, 11) render_fp64_kernel(
                 rem -= c;
             }
         }
+        // (the warps of a tile are numbered by rows: its first half is the first part)
+        const uint32_t redo = __reduce_or_sync(FULL, pid < 0 ? 0u : 1u << (SEG_DONE + (pid >> 5) * parts / (NPIX / 32)));
+        __syncwarp();
+        if (ln == 0) sm.redo = redo;
         const uint32_t b0 = seg_start[seg], b1 = seg_end[seg];
         const uint32_t total = seg_total ? seg_total[seg] : b1 - b0;
         const bool incomplete = total > b1 - b0;
@@ -1372,10 +1436,15 @@ __global__ void __launch_bounds__(32, 11) render_fp64_kernel(
                 }
             }
         }
-        // (a segment that one of its items abandons is listed once)
-        if (abandoned && ln == 0 && atomicOr(&pm[NPIX / 32], 1u) == 0u) {
-            next_active[atomicAdd(n_next, 1u)] = seg;
-            if (counters) atomicAdd(&counters[5], 1ull);
+        // abandoned: the parts of the item's pixels are not complete after all, and
+        // the segment is listed for the next round, if it is not yet
+        if (abandoned && ln == 0) {
+            const uint32_t bit = 1u << (SEG_LISTED + round_no);
+            atomicAnd(seg_state + seg, ~sm.redo);
+            if (!(atomicOr(seg_state + seg, bit) & bit)) {
+                next_active[atomicAdd(n_next, 1u)] = seg;
+                if (counters) atomicAdd(&counters[5], 1ull);
+            }
         }
         __syncwarp();
     }
