@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(RS_THREADS) rs_scatter_kernel(const K *__restr
                 uint32_t wpre = 0;
                 for (int w = 0; w < warp; ++w) wpre += s_warp[w];
                 dstart[d] = wpre + x - run;
-                gbase[d] = digit0 + (offs ? offs[(uint64_t)d * nblocks + blk] : 0u);
+                gbase[d] = digit0 + offs[(uint64_t)d * nblocks + blk];
             }
         }
         __syncthreads();
@@ -411,10 +411,135 @@ __global__ void __launch_bounds__(RS_THREADS) rs_scatter_kernel(const K *__restr
     }
 }
 
+// Short sorts: one launch per pass.  A pass of a sort of some 20000 events was
+// three launches of 3 us each, most of that latency: blocks of 2048 items, so
+// that ten SMs worked, and the histogram's round trips.  Here a block takes 512
+// items, adds up the digit counts of the other blocks itself, and counts, while
+// it scatters, the digits of the next pass for the tiles its items go to (the
+// tile of a destination is known, and the order within it does not matter for a
+// count).  Three histograms take turns, [tile][digit]: this pass's, the next
+// one's, and one that is zeroed for the pass after.  The binning stage of 64
+// Gaussians took 87 us before and 62 now, of one cell of 10k 142 and 117.
+// The line: a call with its entries between 64 and 128 tiles took 546 us with a
+// short sort of them, 536 with a long one.  (Tiles of 1024 items: 551 us, and the
+// 10k cell 121.)
+constexpr int SS_ROUNDS = 2, SS_TILE = SS_ROUNDS * RS_THREADS;
+constexpr uint64_t SS_MAX = 64 * SS_TILE;
+
+// the first pass's histogram; the next one's is zeroed
+template <class K, int RB, bool CELL>
+__global__ void __launch_bounds__(RS_THREADS) ss_hist_kernel(const K *__restrict__ keys, const uint32_t *__restrict__ vals,
+                                                             uint32_t n, int shift, uint64_t n_gauss,
+                                                             uint32_t *__restrict__ hist, uint32_t *__restrict__ next,
+                                                             const uint32_t *__restrict__ n_dev)
+{
+    constexpr uint32_t NB = 1u << RB;
+    __shared__ uint32_t h[NB];
+    if (n_dev) n = min(n, *n_dev);
+    const uint32_t d = threadIdx.x;
+    if (d < NB) h[d] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < SS_ROUNDS; ++r) {
+        const uint64_t i = (uint64_t)blockIdx.x * SS_TILE + r * RS_THREADS + d;
+        if (i < n) atomicAdd(&h[rs_digit<K, RB, CELL>(CELL ? (K)0 : keys[i], CELL ? vals[i] : 0u, shift, n_gauss)], 1u);
+    }
+    __syncthreads();
+    if (d < NB) {
+        hist[(uint64_t)blockIdx.x * NB + d] = h[d];
+        next[(uint64_t)blockIdx.x * NB + d] = 0;
+    }
+}
+
+// next_shift < 0: the last pass
+template <class K, int RB, bool CELL>
+__global__ void __launch_bounds__(RS_THREADS) ss_scatter_kernel(const K *__restrict__ kin, const uint32_t *__restrict__ vin,
+                                                                K *__restrict__ kout, uint32_t *__restrict__ vout,
+                                                                uint32_t n, int shift, int next_shift, uint64_t n_gauss,
+                                                                const uint32_t *__restrict__ hist,
+                                                                uint32_t *__restrict__ next, uint32_t *__restrict__ zero,
+                                                                const uint32_t *__restrict__ n_dev)
+{
+    constexpr uint32_t NB = 1u << RB;
+    static_assert(NB <= RS_THREADS && RS_THREADS == SC_THREADS, "one thread per digit");
+    __shared__ uint32_t wcnt[RS_WARPS][NB];
+    __shared__ uint32_t s_warp[32];
+    if (n_dev) n = min(n, *n_dev);
+    const uint32_t tiles = (n + SS_TILE - 1) / SS_TILE, blk = blockIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t ltmask = (1u << lane) - 1u;
+    if (threadIdx.x < NB) zero[(uint64_t)blk * NB + threadIdx.x] = 0;
+    if (blk >= tiles) return;  // uniform over the block
+    K key[SS_ROUNDS];
+    uint32_t val[SS_ROUNDS], dig[SS_ROUNDS], rank[SS_ROUNDS];
+#pragma unroll
+    for (int r = 0; r < SS_ROUNDS; ++r) {
+        const uint64_t i = (uint64_t)blk * SS_TILE + (uint64_t)warp * (SS_ROUNDS * 32) + r * 32 + lane;
+        const bool ok = i < n;
+        key[r] = ok ? kin[i] : (K)0;
+        val[r] = ok ? vin[i] : 0u;
+        dig[r] = ok ? rs_digit<K, RB, CELL>(key[r], val[r], shift, n_gauss) : NB;
+    }
+    // this thread's digit: its items in the tiles before this one, and in all
+    uint32_t before = 0, total = 0;
+    if (threadIdx.x < NB) {
+#pragma unroll 8
+        for (uint32_t b = 0; b < tiles; ++b) {
+            const uint32_t h = hist[(uint64_t)b * NB + threadIdx.x];
+            total += h;
+            before += b < blk ? h : 0u;
+        }
+    }
+    for (int i = threadIdx.x; i < RS_WARPS * (int)NB; i += RS_THREADS) (&wcnt[0][0])[i] = 0;
+    uint32_t all;
+    const uint32_t digit0 = block_exclusive_scan(total, s_warp, all);  // (ends in a barrier: wcnt is zeroed)
+    __syncthreads();
+    // ranks within the warp, as in rs_scatter_kernel
+#pragma unroll
+    for (int r = 0; r < SS_ROUNDS; ++r) {
+        const bool ok = dig[r] < NB;
+        uint32_t peers = 0xffffffffu;
+#pragma unroll
+        for (int b = 0; b <= RB; ++b) {
+            const bool bit = (dig[r] >> b) & 1u;
+            const uint32_t m = __ballot_sync(0xffffffffu, bit);
+            peers &= bit ? m : ~m;
+        }
+        uint32_t at = 0;
+        if (ok) at = wcnt[warp][dig[r]];
+        rank[r] = at + __popc(peers & ltmask);
+        __syncwarp();
+        if (ok && lane == __ffs(peers) - 1) wcnt[warp][dig[r]] = at + __popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+    if (threadIdx.x < NB) {
+        uint32_t run = digit0 + before;
+#pragma unroll
+        for (int w = 0; w < RS_WARPS; ++w) {
+            const uint32_t t = wcnt[w][threadIdx.x];
+            wcnt[w][threadIdx.x] = run;
+            run += t;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < SS_ROUNDS; ++r) {
+        if (dig[r] < NB) {
+            const uint32_t pos = wcnt[warp][dig[r]] + rank[r];
+            kout[pos] = key[r];
+            vout[pos] = val[r];
+            if (next_shift >= 0)
+                atomicAdd(next + (uint64_t)(pos / SS_TILE) * NB + rs_digit<K, RB, CELL>(key[r], val[r], next_shift, n_gauss), 1u);
+        }
+    }
+}
+
 size_t radix_hist_words(uint64_t n)
 {
-    const uint64_t nb = (n + RS_TILE - 1) / RS_TILE;
-    return 256 * nb + 256;  // and the digits' totals
+    const uint64_t nb = (n + RS_TILE - 1) / RS_TILE, ns = ((n < SS_MAX ? n : SS_MAX) + SS_TILE - 1) / SS_TILE;
+    const uint64_t w = 256 * nb + 256, ws = 3 * 256 * ns;  // and the digits' totals; three of a short sort
+    return w > ws ? w : ws;
 }
 
 // n_dev: see rs_hist_kernel; n is then an upper bound, and the grid is at
@@ -422,21 +547,30 @@ size_t radix_hist_words(uint64_t n)
 template <class K, int RB, bool CELL = false>
 static void radix_pass(const K *ka, const uint32_t *va, K *kb, uint32_t *vb, uint64_t n, int shift, uint32_t *hist,
                        cudaStream_t st, int *launches, uint64_t n_gauss = 0,
-                       const uint32_t *n_dev = nullptr)
+                       const uint32_t *n_dev = nullptr, int pass = 0, bool last = true)
 {
+    if (n <= SS_MAX) {
+        const uint32_t ns = (uint32_t)((n + SS_TILE - 1) / SS_TILE);
+        uint32_t *h[3];
+        for (int i = 0; i < 3; ++i) h[i] = hist + (((uint64_t)((pass + i) % 3) * ns) << RB);
+        if (pass == 0) {
+            ss_hist_kernel<K, RB, CELL><<<ns, RS_THREADS, 0, st>>>(ka, va, (uint32_t)n, shift, n_gauss, h[0], h[1], n_dev);
+            ++*launches;
+        }
+        ss_scatter_kernel<K, RB, CELL><<<ns, RS_THREADS, 0, st>>>(ka, va, kb, vb, (uint32_t)n, shift, last ? -1 : shift + RB,
+                                                                  n_gauss, h[0], h[1], h[2], n_dev);
+        ++*launches;
+        return;
+    }
     const uint32_t nb = (uint32_t)((n + RS_TILE - 1) / RS_TILE);
     const uint32_t grid = n_dev ? (nb < kDevGrid ? nb : kDevGrid) : nb;
     rs_hist_kernel<K, RB, CELL><<<grid, RS_THREADS, 0, st>>>(ka, va, (uint32_t)n, shift, n_gauss, hist, nb, n_dev);
     ++*launches;
-    // one tile: its histogram is the digits' totals
-    uint32_t *tot = nb > 1 ? hist + ((uint64_t)1 << RB) * nb : hist;
-    if (nb > 1) {
-        rs_rows_kernel<<<1u << RB, nb <= 512u ? 128 : RW_THREADS, 0, st>>>(hist, (uint32_t)n, nb, n_dev, tot);
-        ++*launches;
-    }
-    rs_scatter_kernel<K, RB, CELL><<<grid, RS_THREADS, 0, st>>>(ka, va, kb, vb, (uint32_t)n, shift, n_gauss,
-                                                                nb > 1 ? hist : nullptr, tot, nb, n_dev);
-    ++*launches;
+    uint32_t *tot = hist + ((uint64_t)1 << RB) * nb;
+    rs_rows_kernel<<<1u << RB, nb <= 512u ? 128 : RW_THREADS, 0, st>>>(hist, (uint32_t)n, nb, n_dev, tot);
+    rs_scatter_kernel<K, RB, CELL><<<grid, RS_THREADS, 0, st>>>(ka, va, kb, vb, (uint32_t)n, shift, n_gauss, hist, tot, nb,
+                                                                n_dev);
+    *launches += 2;
 }
 
 // Stable sort of the events (keys, vals) by the cell of their pair, bits
@@ -454,11 +588,11 @@ static int radix_sort_cells(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, 
     for (int p = 0, shift = 0; p < passes; ++p, shift += rb) {
         switch (rb) {
         case 1: case 2: case 3: case 4:
-            radix_pass<uint64_t, 4, true>(ka, va, kb, vb, n, shift, hist, st, launches, n_gauss); break;
-        case 5: radix_pass<uint64_t, 5, true>(ka, va, kb, vb, n, shift, hist, st, launches, n_gauss); break;
-        case 6: radix_pass<uint64_t, 6, true>(ka, va, kb, vb, n, shift, hist, st, launches, n_gauss); break;
-        case 7: radix_pass<uint64_t, 7, true>(ka, va, kb, vb, n, shift, hist, st, launches, n_gauss); break;
-        default: radix_pass<uint64_t, 8, true>(ka, va, kb, vb, n, shift, hist, st, launches, n_gauss); break;
+            radix_pass<uint64_t, 4, true>(ka, va, kb, vb, n, shift, hist, st, launches, n_gauss, nullptr, p, p + 1 == passes); break;
+        case 5: radix_pass<uint64_t, 5, true>(ka, va, kb, vb, n, shift, hist, st, launches, n_gauss, nullptr, p, p + 1 == passes); break;
+        case 6: radix_pass<uint64_t, 6, true>(ka, va, kb, vb, n, shift, hist, st, launches, n_gauss, nullptr, p, p + 1 == passes); break;
+        case 7: radix_pass<uint64_t, 7, true>(ka, va, kb, vb, n, shift, hist, st, launches, n_gauss, nullptr, p, p + 1 == passes); break;
+        default: radix_pass<uint64_t, 8, true>(ka, va, kb, vb, n, shift, hist, st, launches, n_gauss, nullptr, p, p + 1 == passes); break;
         }
         uint64_t *tk = ka; ka = kb; kb = tk;
         uint32_t *tv = va; va = vb; vb = tv;
@@ -485,11 +619,11 @@ static int radix_sort(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, 
     int flips = 0;
     for (int p = 0, shift = shift0; p < passes; ++p, shift += rb) {
         switch (rb) {
-        case 1: case 2: case 3: case 4: radix_pass<K, 4>(ka, va, kb, vb, n, shift, hist, st, launches, 0, n_dev); break;
-        case 5: radix_pass<K, 5>(ka, va, kb, vb, n, shift, hist, st, launches, 0, n_dev); break;
-        case 6: radix_pass<K, 6>(ka, va, kb, vb, n, shift, hist, st, launches, 0, n_dev); break;
-        case 7: radix_pass<K, 7>(ka, va, kb, vb, n, shift, hist, st, launches, 0, n_dev); break;
-        default: radix_pass<K, 8>(ka, va, kb, vb, n, shift, hist, st, launches, 0, n_dev); break;
+        case 1: case 2: case 3: case 4: radix_pass<K, 4>(ka, va, kb, vb, n, shift, hist, st, launches, 0, n_dev, p, p + 1 == passes); break;
+        case 5: radix_pass<K, 5>(ka, va, kb, vb, n, shift, hist, st, launches, 0, n_dev, p, p + 1 == passes); break;
+        case 6: radix_pass<K, 6>(ka, va, kb, vb, n, shift, hist, st, launches, 0, n_dev, p, p + 1 == passes); break;
+        case 7: radix_pass<K, 7>(ka, va, kb, vb, n, shift, hist, st, launches, 0, n_dev, p, p + 1 == passes); break;
+        default: radix_pass<K, 8>(ka, va, kb, vb, n, shift, hist, st, launches, 0, n_dev, p, p + 1 == passes); break;
         }
         K *tk = ka; ka = kb; kb = tk;
         uint32_t *tv = va; va = vb; vb = tv;
