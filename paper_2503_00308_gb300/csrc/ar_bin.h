@@ -50,7 +50,6 @@ struct BinOut {
 
 size_t scan_temp_words(uint64_t n);
 size_t radix_hist_words(uint64_t n);
-void exclusive_scan(const uint32_t *in, uint32_t *out, uint64_t n, uint32_t *tmp, cudaStream_t st, int *launches);
 int run_binning(const BinArgs &a, BinOut &o, cudaStream_t st, int *launches);
 // The second phase: complete lists for the segments active[0, *n_active)
 // (a device count), sorted as run_binning sorts them, in place of the first
@@ -64,8 +63,9 @@ int run_rebin(const BinArgs &a, const BinOut &first, const uint32_t *active, con
 // active segments and lists them in work (count is incremented); the grid is
 // sized from max_active, the count of active segments is read on the device.
 // launch_init_rounds: words[0] = n_seg, words[1 .. 31] = 0 (the rounds'
-// counters), seg_state[n_seg] = seg_swept[n_seg] = 0.
-void launch_init_rounds(uint32_t *words, uint32_t n_seg, uint32_t *seg_state, uint32_t *seg_swept, cudaStream_t st);
+// counters), seg_state[n_seg] = seg_swept[n_seg] = state[n_pairs] = 0.
+void launch_init_rounds(uint32_t *words, uint32_t n_seg, uint32_t *seg_state, uint32_t *seg_swept, uint32_t *state,
+                        uint64_t n_pairs, cudaStream_t st);
 void launch_demand(const uint32_t *active, const uint32_t *n_active, uint32_t max_active, const uint32_t *seg_start,
                    const uint32_t *seg_end, const uint32_t *ent_ev, const uint32_t *ev_val, uint32_t window,
                    uint32_t *state, uint32_t *work, uint32_t *count, cudaStream_t st);

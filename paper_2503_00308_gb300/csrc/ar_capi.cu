@@ -929,8 +929,7 @@ int run_windowed_render(int M, int TS, RenderLaunch rl, const CallConst &cc, con
     const uint32_t kWindow[3] = {w0, two ? w0 : (w0 < 8192u ? 8192u : 0xffffffffu), 0xffffffffu};
     const uint32_t *round1_order = nullptr;
     uint32_t *act[2] = {act0, act1};
-    CK(cudaMemsetAsync(state, 0, sizeof(uint32_t) * n_pairs, st));
-    launch_init_rounds(words, (uint32_t)n_seg, seg_state, seg_swept, st);
+    launch_init_rounds(words, (uint32_t)n_seg, seg_state, seg_swept, state, n_pairs, st);
     rl.seg_state = seg_state;
     rl.seg_swept = seg_swept;
     ++*launches;

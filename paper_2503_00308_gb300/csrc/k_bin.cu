@@ -3,9 +3,9 @@
 // "AbstractSplat on GPUs").
 //
 // Pipeline (all on the render stream):
-//   1. flags/scan   : compact the (cell, Gaussian) pairs that reach the image;
-//   2. events       : two per pair (lower / upper depth-key endpoint), keyed by
-//                     the order-preserving bits of the FP64 key;
+//   1-2. events     : two per (cell, Gaussian) pair that reaches the image (lower /
+//                     upper depth-key endpoint), keyed by the order-preserving
+//                     bits of the FP64 key;
 //   3. sort         : stable LSD radix sort by key, then stably by cell;
 //   4. entries      : each event is copied to every tile its pixel box meets,
 //                     in sorted-event order (cell-major), keyed by tile and cell;
@@ -134,8 +134,8 @@ size_t scan_temp_words(uint64_t n)
 // exclusive scan of n words (in may equal out); tmp from scan_temp_words.
 // dl: the length on the device (n its bound); the words past it are neither
 // read nor written.
-static void exclusive_scan_dl(const uint32_t *in, uint32_t *out, uint64_t n, uint32_t *tmp, cudaStream_t st,
-                              int *launches, DevLen dl)
+static void exclusive_scan(const uint32_t *in, uint32_t *out, uint64_t n, uint32_t *tmp, cudaStream_t st,
+                           int *launches, DevLen dl = DevLen{})
 {
     if (n == 0) return;
     const uint64_t nb = (n + SC_TILE - 1) / SC_TILE;
@@ -153,14 +153,9 @@ static void exclusive_scan_dl(const uint32_t *in, uint32_t *out, uint64_t n, uin
     uint32_t *sums = tmp, *offs = tmp + nb;
     scan_sums_kernel<<<(unsigned)nb, SC_THREADS, 0, st>>>(in, (uint32_t)n, sums, dl);
     ++*launches;
-    exclusive_scan_dl(sums, offs, nb, tmp + 2 * nb, st, launches, DevLen{});
+    exclusive_scan(sums, offs, nb, tmp + 2 * nb, st, launches);
     scan_apply_kernel<false><<<(unsigned)nb, SC_THREADS, 0, st>>>(in, (uint32_t)n, offs, out, dl);
     ++*launches;
-}
-
-void exclusive_scan(const uint32_t *in, uint32_t *out, uint64_t n, uint32_t *tmp, cudaStream_t st, int *launches)
-{
-    exclusive_scan_dl(in, out, n, tmp, st, launches, DevLen{});
 }
 
 // ------------------------------------------------------------ radix sort
@@ -633,23 +628,96 @@ static int radix_sort(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, 
 }
 
 // -------------------------------------------------------------- binning
-__global__ void valid_flags_kernel(const PixBox *__restrict__ boxes, uint64_t n, uint32_t *__restrict__ flags)
+// Events.  Counting the present pairs of each block and writing their events, with
+// the positions found anew, are two launches where flags, their scan, the
+// writing and the cells' ranges were five of 3 us each in a small call.
+constexpr int EV_ROUNDS = 8, EV_TILE = SC_THREADS * EV_ROUNDS;
+
+__global__ void __launch_bounds__(SC_THREADS) event_count_kernel(const PixBox *__restrict__ boxes, uint64_t n,
+                                                                 uint32_t *__restrict__ sums)
 {
-    const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    if (i < n) flags[i] = boxes[i].x0 >= 0 ? 1u : 0u;
+    __shared__ uint32_t s_warp[SC_THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t i0 = (uint64_t)blockIdx.x * EV_TILE + (uint64_t)warp * (32 * EV_ROUNDS) + lane;
+    uint32_t cnt = 0;
+#pragma unroll
+    for (int r = 0; r < EV_ROUNDS; ++r) {
+        const uint64_t i = i0 + r * 32;
+        cnt += __popc(__ballot_sync(0xffffffffu, i < n && boxes[i].x0 >= 0));
+    }
+    if (lane == 0) s_warp[warp] = cnt;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t t = 0;
+        for (int w = 0; w < SC_THREADS / 32; ++w) t += s_warp[w];
+        sums[blockIdx.x] = t;
+    }
 }
 
-__global__ void emit_events_kernel(const PixBox *__restrict__ boxes, const double *__restrict__ keys,
-                                   const uint32_t *__restrict__ pos, uint64_t n, uint64_t *__restrict__ ev_key,
-                                   uint32_t *__restrict__ ev_val)
+// Items of the blocks before this one: the sum of their counts (SUMS), or the
+// scanned count.
+template <bool SUMS>
+__device__ __forceinline__ uint32_t items_before(const uint32_t *__restrict__ offs, uint32_t *s_warp)
 {
-    const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    if (i >= n || boxes[i].x0 < 0) return;
-    const uint32_t p = pos[i];
-    ev_key[2 * p] = key_bits(keys[2 * i]);
-    ev_key[2 * p + 1] = key_bits(keys[2 * i + 1]);
-    ev_val[2 * p] = (uint32_t)(2 * i);
-    ev_val[2 * p + 1] = (uint32_t)(2 * i + 1);
+    if (!SUMS) return offs[blockIdx.x];
+    uint32_t part = 0, before;
+    for (uint32_t b = threadIdx.x; b < blockIdx.x; b += SC_THREADS) part += offs[b];
+    block_exclusive_scan(part, s_warp, before);
+    return before;
+}
+
+// offs: the blocks' counts, added up here (SUMS), or their scan.  Also the
+// first sorted event of every cell (cell c holds [cell_ev[c], cell_ev[c + 1])):
+// cell c's events start at twice the position of pair c n_gauss.
+template <bool SUMS>
+__global__ void __launch_bounds__(SC_THREADS) event_emit_kernel(const PixBox *__restrict__ boxes,
+                                                                const double *__restrict__ keys, uint64_t n,
+                                                                uint64_t n_gauss, int n_cells, uint32_t ne,
+                                                                const uint32_t *__restrict__ offs,
+                                                                uint64_t *__restrict__ ev_key,
+                                                                uint32_t *__restrict__ ev_val,
+                                                                uint32_t *__restrict__ cell_ev)
+{
+    __shared__ uint32_t s_warp[32], s_cnt[SC_THREADS / 32], s_bal[EV_TILE / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t blk0 = (uint64_t)blockIdx.x * EV_TILE;
+    const uint64_t i0 = blk0 + (uint64_t)warp * (32 * EV_ROUNDS) + lane;
+    uint32_t bal[EV_ROUNDS], cnt = 0;
+#pragma unroll
+    for (int r = 0; r < EV_ROUNDS; ++r) {
+        const uint64_t i = i0 + r * 32;
+        bal[r] = __ballot_sync(0xffffffffu, i < n && boxes[i].x0 >= 0);
+        cnt += __popc(bal[r]);
+    }
+    const uint32_t before = items_before<SUMS>(offs, s_warp);
+    if (lane == 0) {
+        s_cnt[warp] = cnt;
+#pragma unroll
+        for (int r = 0; r < EV_ROUNDS; ++r) s_bal[warp * EV_ROUNDS + r] = bal[r];
+    }
+    __syncthreads();
+    uint32_t run = before;
+    for (int w = 0; w < warp; ++w) run += s_cnt[w];
+#pragma unroll
+    for (int r = 0; r < EV_ROUNDS; ++r) {
+        const uint64_t i = i0 + r * 32;
+        if ((bal[r] >> lane) & 1u) {
+            const uint32_t p = run + __popc(bal[r] & ((1u << lane) - 1u));
+            const double2 k = reinterpret_cast<const double2 *>(keys)[i];
+            reinterpret_cast<ulonglong2 *>(ev_key)[p] = make_ulonglong2(key_bits(k.x), key_bits(k.y));
+            reinterpret_cast<uint2 *>(ev_val)[p] = make_uint2((uint32_t)(2 * i), (uint32_t)(2 * i + 1));
+        }
+        run += __popc(bal[r]);
+    }
+    if (!cell_ev) return;
+    const uint64_t end = blk0 + EV_TILE < n ? blk0 + EV_TILE : n;
+    for (uint64_t c = (blk0 + n_gauss - 1) / n_gauss + threadIdx.x; c * n_gauss < end; c += SC_THREADS) {
+        const uint32_t at = (uint32_t)(c * n_gauss - blk0);
+        uint32_t p = before + __popc(s_bal[at / 32] & ((1u << at % 32) - 1u));
+        for (uint32_t w = 0; w < at / 32; ++w) p += __popc(s_bal[w]);
+        cell_ev[c] = 2u * p;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) cell_ev[n_cells] = ne;
 }
 
 __device__ __forceinline__ void tile_rect(const PixBox &b, int TS, int &tx0, int &tx1, int &ty0, int &ty1)
@@ -657,38 +725,27 @@ __device__ __forceinline__ void tile_rect(const PixBox &b, int TS, int &tx0, int
     tx0 = b.x0 / TS; tx1 = b.x1 / TS; ty0 = b.y0 / TS; ty1 = b.y1 / TS;
 }
 
-// First sorted event of every cell (cell c holds [cell_ev[c], cell_ev[c + 1])):
-// from the exclusive scan pos of the pairs' presence flags, cell c's events
-// start at 2 pos[c n_gauss].
-__global__ void cell_events_kernel(const uint32_t *__restrict__ pos, uint64_t n_gauss, int n_cells, uint32_t ne,
-                                   uint32_t *__restrict__ cell_ev)
+// The tile counts of each block's 256 sorted events, summed
+__global__ void __launch_bounds__(SC_THREADS) tile_sums_kernel(const uint32_t *__restrict__ ev_val, uint64_t ne,
+                                                               const PixBox *__restrict__ boxes, int TS,
+                                                               uint32_t *__restrict__ sums)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c > n_cells) return;
-    cell_ev[c] = c < n_cells ? 2u * pos[(uint64_t)c * n_gauss] : ne;
-}
-
-// The depth prefix of a cell: its first ceil(E / 2^shift) sorted events, E
-// the cell's events (shift = 0: all of them).  Sorted event e of cell `cell`
-// lies in it when this holds.
-__device__ __forceinline__ bool in_prefix(uint64_t e, uint32_t cell, const uint32_t *__restrict__ cell_ev, int shift)
-{
-    if (!shift) return true;
-    const uint32_t c0 = cell_ev[cell], ec = cell_ev[cell + 1] - c0;
-    return e - c0 < (((uint64_t)ec + (1u << shift) - 1u) >> shift);
-}
-
-__global__ void tile_counts_kernel(const uint32_t *__restrict__ ev_val, uint64_t ne,
-                                   const PixBox *__restrict__ boxes, int TS, uint64_t n_gauss,
-                                   const uint32_t *__restrict__ cell_ev, int shift, uint32_t *__restrict__ cnt)
-{
-    const uint64_t e = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    if (e >= ne) return;
-    const uint32_t ri = ev_val[e] >> 1;
-    int tx0, tx1, ty0, ty1;
-    tile_rect(boxes[ri], TS, tx0, tx1, ty0, ty1);
-    cnt[e] = in_prefix(e, (uint32_t)(ri / n_gauss), cell_ev, shift) ? (uint32_t)((tx1 - tx0 + 1) * (ty1 - ty0 + 1))
-                                                                      : 0u;
+    __shared__ uint32_t s_warp[SC_THREADS / 32];
+    const uint64_t e = blockIdx.x * (uint64_t)SC_THREADS + threadIdx.x;
+    uint32_t cnt = 0;
+    if (e < ne) {
+        int tx0, tx1, ty0, ty1;
+        tile_rect(boxes[ev_val[e] >> 1], TS, tx0, tx1, ty0, ty1);
+        cnt = (uint32_t)((tx1 - tx0 + 1) * (ty1 - ty0 + 1));
+    }
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = cnt;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t t = 0;
+        for (int w = 0; w < SC_THREADS / 32; ++w) t += s_warp[w];
+        sums[blockIdx.x] = t;
+    }
 }
 
 // *word = cnt[n - 1] before an in-place exclusive scan of cnt, then (add)
@@ -884,11 +941,15 @@ __device__ __forceinline__ uint32_t entry_segment(uint32_t key, int cb, int n_ti
 // range of the output (off is their exclusive scan).  The lanes stride over
 // that range, so every store instruction writes 32 consecutive words; each
 // lane finds the event of its entry by a binary search over the warp's 32
-// offsets (shuffles).  Launch with a multiple of 32 threads per block.
+// offsets (shuffles).  Blocks of SC_THREADS.
+// OFFS 0: off[] holds each item's offset; 1, 2: the blocks' counts (1) or their
+// scan (2), and the items' offsets are found here (a count and this launch, where
+// the counts, their scan and this were four).
 // With evmap, the items are the first phase's prefix events in their
 // compacted index (*n_map of them, evmap: the sorted event of each), else the
 // sorted events themselves.
-__global__ void emit_entries_kernel(const uint32_t *__restrict__ ev_val, uint64_t ne,
+template <int OFFS>
+__global__ void __launch_bounds__(SC_THREADS) emit_entries_kernel(const uint32_t *__restrict__ ev_val, uint64_t ne,
                                     const PixBox *__restrict__ boxes, int TS, int ntx, int n_tiles, int cb,
                                     uint64_t n_gauss, const uint32_t *__restrict__ evmap,
                                     const uint32_t *__restrict__ n_map, const uint32_t *__restrict__ off,
@@ -898,9 +959,9 @@ __global__ void emit_entries_kernel(const uint32_t *__restrict__ ev_val, uint64_
     const int lane = threadIdx.x & 31;
     if (evmap) ne = min(ne, (uint64_t)*n_map);
     const uint64_t e0 = ((blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5) * 32u;
-    if (e0 >= ne) return;  // uniform across the warp
+    if (!OFFS && e0 >= ne) return;  // uniform across the warp
     const uint64_t item = e0 + (uint64_t)lane;
-    uint32_t myoff = 0xffffffffu, myend = 0, cell = 0, myev = 0;
+    uint32_t myoff = 0xffffffffu, myend = 0, cell = 0, myev = 0, cnt = 0;
     int tx0 = 0, ty0 = 0, tw = 1;
     if (item < ne) {
         myev = evmap ? evmap[item] : (uint32_t)item;
@@ -909,9 +970,18 @@ __global__ void emit_entries_kernel(const uint32_t *__restrict__ ev_val, uint64_
         int tx1, ty1;
         tile_rect(boxes[ri], TS, tx0, tx1, ty0, ty1);
         tw = tx1 - tx0 + 1;
-        myoff = off[item];
-        myend = myoff + (uint32_t)(tw * (ty1 - ty0 + 1));
+        cnt = (uint32_t)(tw * (ty1 - ty0 + 1));
+        if (!OFFS) myoff = off[item];
     }
+    if (OFFS) {
+        __shared__ uint32_t s_warp[32];
+        uint32_t all;
+        const uint32_t before = items_before<OFFS == 1>(off, s_warp);
+        const uint32_t at = before + block_exclusive_scan(cnt, s_warp, all);
+        if (item < ne) myoff = at;
+    }
+    if (item < ne) myend = myoff + cnt;
+    if (OFFS && e0 >= ne) return;
     const uint32_t start = __shfl_sync(full, myoff, 0);
     uint32_t end = myend;
 #pragma unroll
@@ -1003,7 +1073,8 @@ __global__ void seg_bounds_kernel(const uint32_t *__restrict__ key, uint64_t n, 
 }
 
 // Packed keys come out of the tile sort in ascending order (tile, then cell),
-// so each segment's range is found by two binary searches over the keys.
+// so each segment's range is found by two binary searches over the keys; with
+// len_key, also the items of the schedule's sort.
 __device__ __forceinline__ uint32_t lower_bound_u32(const uint32_t *__restrict__ a, uint32_t n, uint32_t v)
 {
     uint32_t lo = 0, hi = n;
@@ -1015,7 +1086,8 @@ __device__ __forceinline__ uint32_t lower_bound_u32(const uint32_t *__restrict__
 }
 __global__ void seg_bounds_search_kernel(const uint32_t *__restrict__ key, uint32_t n, int cb, int n_cells,
                                          int n_tiles, uint32_t *__restrict__ start, uint32_t *__restrict__ end,
-                                         const uint32_t *__restrict__ n_dev)
+                                         const uint32_t *__restrict__ n_dev, uint32_t *__restrict__ len_key,
+                                         uint32_t *__restrict__ len_val)
 {
     const uint64_t sg = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     if (n_dev && *n_dev < n) n = *n_dev;
@@ -1023,8 +1095,13 @@ __global__ void seg_bounds_search_kernel(const uint32_t *__restrict__ key, uint3
     const uint32_t cell = (uint32_t)(sg / (uint64_t)n_tiles), tile = (uint32_t)(sg % (uint64_t)n_tiles);
     const uint32_t k = (tile << cb) | cell;
     const uint32_t b = lower_bound_u32(key, n, k);
+    const uint32_t e = (b < n && key[b] == k) ? (k == 0xffffffffu ? n : lower_bound_u32(key, n, k + 1u)) : b;
     start[sg] = b;
-    end[sg] = (b < n && key[b] == k) ? (k == 0xffffffffu ? n : lower_bound_u32(key, n, k + 1u)) : b;
+    end[sg] = e;
+    if (len_key) {
+        len_key[sg] = length_key(e - b);
+        len_val[sg] = (uint32_t)sg;
+    }
 }
 
 __global__ void iota_kernel(uint32_t *__restrict__ p, uint64_t n)
@@ -1038,9 +1115,10 @@ static inline unsigned blocks_for(uint64_t n, int t) { return (unsigned)((n + t 
 // The entries' stable sort by tile (packed keys: the tile bits above cb) or
 // by segment, then the segment bounds; n_dev: the entries' count when it is
 // known on the device only (n_entries bounds it).  Returns the buffer
-// holding the result.
-static int sort_entries(const BinArgs &a, bool packed, int cb, int tb, const uint32_t *n_dev, cudaStream_t st,
-                        int *launches)
+// holding the result.  schedule: with the items of the schedule's sort, where the
+// bounds are searched (packed).
+static int sort_entries(const BinArgs &a, bool packed, int cb, int tb, const uint32_t *n_dev, bool schedule,
+                        cudaStream_t st, int *launches)
 {
     const int T = 256;
     int h;
@@ -1054,7 +1132,9 @@ static int sort_entries(const BinArgs &a, bool packed, int cb, int tb, const uin
     const uint32_t *keys = a.ent_seg[h];
     if (packed) {
         seg_bounds_search_kernel<<<blocks_for(a.n_segments, T), T, 0, st>>>(keys, (uint32_t)a.n_entries, cb, a.n_cells,
-                                                                            a.n_tiles, a.seg_start, a.seg_end, n_dev);
+                                                                            a.n_tiles, a.seg_start, a.seg_end, n_dev,
+                                                                            schedule ? a.seg_k[0] : nullptr,
+                                                                            a.seg_v[0]);
         ++*launches;
     } else {
         cudaMemsetAsync(a.seg_start, 0, sizeof(uint32_t) * a.n_segments, st);
@@ -1071,14 +1151,14 @@ static int sort_entries(const BinArgs &a, bool packed, int cb, int tb, const uin
 int run_binning(const BinArgs &a, BinOut &o, cudaStream_t st, int *launches)
 {
     const int T = 256;
-    // 1. compact the pairs that reach the image
-    valid_flags_kernel<<<blocks_for(a.n_pairs, T), T, 0, st>>>(a.boxes, a.n_pairs, a.u32_a);
-    ++*launches;
-    exclusive_scan(a.u32_a, a.u32_a, a.n_pairs, a.scan_tmp, st, launches);
-    // 2. events
-    emit_events_kernel<<<blocks_for(a.n_pairs, T), T, 0, st>>>(a.boxes, a.keys, a.u32_a, a.n_pairs, a.ev_key[0],
-                                                                 a.ev_val[0]);
-    ++*launches;
+    // 1-2. the events of the pairs that reach the image, and the cells' ranges
+    const uint64_t eb = (a.n_pairs + EV_TILE - 1) / EV_TILE;
+    event_count_kernel<<<(unsigned)eb, SC_THREADS, 0, st>>>(a.boxes, a.n_pairs, a.u32_a);
+    auto emit = eb <= SC_SUM_BLOCKS ? event_emit_kernel<true> : event_emit_kernel<false>;
+    if (eb > SC_SUM_BLOCKS) exclusive_scan(a.u32_a, a.u32_a, eb, a.scan_tmp, st, launches);
+    emit<<<(unsigned)eb, SC_THREADS, 0, st>>>(a.boxes, a.keys, a.n_pairs, a.n_gauss, a.n_cells, (uint32_t)a.n_events, a.u32_a,
+                                              a.ev_key[0], a.ev_val[0], a.cell_ev);
+    *launches += 2;
     const uint64_t ne = a.n_events;
     o.seg_total = nullptr;
     if (ne == 0) {
@@ -1093,15 +1173,8 @@ int run_binning(const BinArgs &a, BinOut &o, cudaStream_t st, int *launches)
         o.seg_order = a.seg_v[1];  // where a sorted one ends
         return cudaGetLastError() == cudaSuccess ? 0 : 1;
     }
-    // the first phase bins only each cell's depth prefix (see in_prefix): the
-    // cells' event ranges, while the presence scan is at hand (also wanted by
-    // the renderer's stop histogram when there is one phase)
+    // the first phase bins only each cell's depth prefix
     const bool prefix = a.prefix_shift > 0 && a.cell_ev;
-    if (a.cell_ev) {
-        cell_events_kernel<<<blocks_for((uint64_t)a.n_cells + 1, T), T, 0, st>>>(a.u32_a, a.n_gauss, a.n_cells,
-                                                                                  (uint32_t)ne, a.cell_ev);
-        ++*launches;
-    }
     // 3. sort by key bits, then stably by cell
     int f = radix_sort<uint64_t>(a.ev_key[0], a.ev_val[0], a.ev_key[1], a.ev_val[1], ne, 64, a.hist, st, launches);
     uint64_t *evk = a.ev_key[f];
@@ -1136,6 +1209,7 @@ int run_binning(const BinArgs &a, BinOut &o, cudaStream_t st, int *launches)
     // in their compacted index (words[2] of them; evmap: the sorted event of
     // each), and the count of its entries is then known on the device only.
     const uint32_t *n_dev = nullptr, *evmap = nullptr;
+    auto emit_entries = emit_entries_kernel<0>;
     if (prefix) {
         prefix_ranges_kernel<<<1, SC_THREADS, 0, st>>>(a.cell_ev, a.n_cells, a.prefix_shift, a.pref_start,
                                                        a.words + 2);
@@ -1143,15 +1217,17 @@ int run_binning(const BinArgs &a, BinOut &o, cudaStream_t st, int *launches)
                                                               a.n_cells, a.words + 2, a.u32_a, a.u32_b);
         const DevLen dl{a.words + 2, 1, 1};
         scan_last_kernel<<<1, 32, 0, st>>>(a.u32_a, ne, a.words, 0, dl);
-        exclusive_scan_dl(a.u32_a, a.u32_a, ne, a.scan_tmp, st, launches, dl);
+        exclusive_scan(a.u32_a, a.u32_a, ne, a.scan_tmp, st, launches, dl);
         scan_last_kernel<<<1, 32, 0, st>>>(a.u32_a, ne, a.words, 1, dl);
         *launches += 4;
         n_dev = a.words;
         evmap = a.u32_b;
     } else {
-        tile_counts_kernel<<<blocks_for(ne, T), T, 0, st>>>(evv, ne, a.boxes, a.TS, a.n_gauss, a.cell_ev, 0, a.u32_a);
+        const uint64_t tb256 = blocks_for(ne, SC_THREADS);
+        tile_sums_kernel<<<(unsigned)tb256, SC_THREADS, 0, st>>>(evv, ne, a.boxes, a.TS, a.u32_a);
         ++*launches;
-        exclusive_scan(a.u32_a, a.u32_a, ne, a.scan_tmp, st, launches);
+        if (tb256 > SC_SUM_BLOCKS) exclusive_scan(a.u32_a, a.u32_a, tb256, a.scan_tmp, st, launches);
+        emit_entries = tb256 > SC_SUM_BLOCKS ? emit_entries_kernel<2> : emit_entries_kernel<1>;
     }
     // entry keys: tile bits above cell bits when both fit in 32 bits
     int cb = 0, tb = 0;
@@ -1159,19 +1235,21 @@ int run_binning(const BinArgs &a, BinOut &o, cudaStream_t st, int *launches)
     while ((1ull << tb) < (uint64_t)a.n_tiles) ++tb;
     if (tb == 0) tb = 1;
     const bool packed = cb + tb <= 32;
-    emit_entries_kernel<<<blocks_for(ne, T), T, 0, st>>>(evv, ne, a.boxes, a.TS, a.ntx, a.n_tiles, packed ? cb : -1,
-                                                          a.n_gauss, evmap, prefix ? a.words + 2 : nullptr, a.u32_a,
-                                                          a.ent_seg[0],
-                                                          a.ent_ev[0]);
+    emit_entries<<<blocks_for(ne, SC_THREADS), SC_THREADS, 0, st>>>(evv, ne, a.boxes, a.TS, a.ntx, a.n_tiles,
+                                                                    packed ? cb : -1, a.n_gauss, evmap,
+                                                                    prefix ? a.words + 2 : nullptr, a.u32_a, a.ent_seg[0],
+                                                                    a.ent_ev[0]);
     ++*launches;
     // 5-6. stable sort by tile, segment bounds
-    const int h = sort_entries(a, packed, cb, tb, n_dev, st, launches);
+    const int h = sort_entries(a, packed, cb, tb, n_dev, true, st, launches);
     o.ent_seg = a.ent_seg[h];
     o.ent_ev = a.ent_ev[h];
     // 7. schedule: segments by decreasing length (load balance of the render)
-    seg_len_kernel<<<blocks_for(a.n_segments, T), T, 0, st>>>(a.seg_start, a.seg_end, a.n_segments, a.seg_k[0],
-                                                               a.seg_v[0]);
-    ++*launches;
+    if (!packed) {
+        seg_len_kernel<<<blocks_for(a.n_segments, T), T, 0, st>>>(a.seg_start, a.seg_end, a.n_segments, a.seg_k[0],
+                                                                   a.seg_v[0]);
+        ++*launches;
+    }
     int q = radix_sort<uint32_t>(a.seg_k[0], a.seg_v[0], a.seg_k[1], a.seg_v[1], a.n_segments, 8, a.hist, st, launches);
     o.seg_order = a.seg_v[q];
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
@@ -1213,7 +1291,7 @@ int run_rebin(const BinArgs &a, const BinOut &first, const uint32_t *active, con
                                                            a.sat, n_active, a.u32_a);
     scan_last_kernel<<<1, 32, 0, st>>>(a.u32_a, ne, a.words + 1, 0, dl);
     *launches += 7;
-    exclusive_scan_dl(a.u32_a, a.u32_a, ne, a.scan_tmp, st, launches, dl);
+    exclusive_scan(a.u32_a, a.u32_a, ne, a.scan_tmp, st, launches, dl);
     scan_last_kernel<<<1, 32, 0, st>>>(a.u32_a, ne, a.words + 1, 1, dl);
     int cb = 0, tb = 0;
     while ((1ull << cb) < (uint64_t)a.n_cells) ++cb;
@@ -1224,7 +1302,7 @@ int run_rebin(const BinArgs &a, const BinOut &first, const uint32_t *active, con
                                                          a.n_gauss, a.mask, a.sat, n_active, a.u32_a, a.ent_seg[0],
                                                          a.ent_ev[0]);
     *launches += 2;
-    const int h = sort_entries(a, packed, cb, tb, a.words + 1, st, launches);
+    const int h = sort_entries(a, packed, cb, tb, a.words + 1, false, st, launches);
     o.ent_seg = a.ent_seg[h];
     o.ent_ev = a.ent_ev[h];
     // the active segments, longest full list first (the first phase's order
@@ -1239,15 +1317,19 @@ int run_rebin(const BinArgs &a, const BinOut &first, const uint32_t *active, con
 
 // ------------------------------------------------------------ windowed rounds
 // every counter of the windowed rounds in one launch (they were fifteen
-// memsets, a tenth of a small render's graph), and the segments' state
-__global__ void init_rounds_kernel(uint32_t *words, uint32_t n_seg, uint32_t *seg_state, uint32_t *seg_swept)
+// memsets, a tenth of a small render's graph), and the segments' and pairs' states
+// (state: 16-byte aligned)
+__global__ void init_rounds_kernel(uint32_t *words, uint32_t n_seg, uint32_t *seg_state, uint32_t *seg_swept,
+                                   uint32_t *state, uint64_t n_pairs)
 {
-    const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    if (i < 32) words[i] = i ? 0u : n_seg;
-    if (i < n_seg) {
+    const uint64_t i0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, step = gridDim.x * (uint64_t)blockDim.x;
+    if (i0 < 32) words[i0] = i0 ? 0u : n_seg;
+    for (uint64_t i = i0; i < n_seg; i += step) {
         seg_state[i] = 0u;
         seg_swept[i] = 0u;
     }
+    for (uint64_t i = i0; i < n_pairs / 4; i += step) reinterpret_cast<uint4 *>(state)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (i0 < n_pairs % 4) state[n_pairs / 4 * 4 + i0] = 0u;
 }
 
 // For each active segment, the lower endpoints among its first `window`
@@ -1289,9 +1371,12 @@ __global__ void __launch_bounds__(256) demand_kernel(const uint32_t *__restrict_
     }
 }
 
-void launch_init_rounds(uint32_t *words, uint32_t n_seg, uint32_t *seg_state, uint32_t *seg_swept, cudaStream_t st)
+void launch_init_rounds(uint32_t *words, uint32_t n_seg, uint32_t *seg_state, uint32_t *seg_swept, uint32_t *state,
+                        uint64_t n_pairs, cudaStream_t st)
 {
-    init_rounds_kernel<<<blocks_for((uint64_t)n_seg + 32, 256), 256, 0, st>>>(words, n_seg, seg_state, seg_swept);
+    const uint64_t most = n_pairs / 4 > n_seg ? n_pairs / 4 : n_seg, want = blocks_for(most + 32, 256);
+    init_rounds_kernel<<<(unsigned)(want < kDevGrid ? want : kDevGrid), 256, 0, st>>>(words, n_seg, seg_state, seg_swept,
+                                                                                     state, n_pairs);
 }
 
 void launch_demand(const uint32_t *active, const uint32_t *n_active, uint32_t max_active, const uint32_t *seg_start,
