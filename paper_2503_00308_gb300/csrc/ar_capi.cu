@@ -67,11 +67,11 @@ int rec_scalar_offset_m1();
 int rec_scalar_offset_m4();
 int rec_scalar_offset_m6();
 int launch_call_prep_m1(const double *, const double *, const CallConst &, void *, const float *, const float *,
-                        const double *, double *, cudaStream_t);
+                        const double *, double *, cudaStream_t, ZeroWords, ZeroWords);
 int launch_call_prep_m4(const double *, const double *, const CallConst &, void *, const float *, const float *,
-                        const double *, double *, cudaStream_t);
+                        const double *, double *, cudaStream_t, ZeroWords, ZeroWords);
 int launch_call_prep_m6(const double *, const double *, const CallConst &, void *, const float *, const float *,
-                        const double *, double *, cudaStream_t);
+                        const double *, double *, cudaStream_t, ZeroWords, ZeroWords);
 int launch_record_prep_m1(const double *, const void *, const CallConst &, const void *, int, float *, PixBox *,
                           double *, unsigned long long *, cudaStream_t, uint32_t *, uint32_t *);
 int launch_record_prep_m4(const double *, const void *, const CallConst &, const void *, int, float *, PixBox *,
@@ -124,11 +124,11 @@ static int rec_scalar_offset(int M)
     return M == 1 ? rec_scalar_offset_m1() : (M == 4 ? rec_scalar_offset_m4() : rec_scalar_offset_m6());
 }
 int launch_call_prep(int M, const double *lo, const double *hi, const CallConst &cc, void *cells, const float *uw_lo,
-                     const float *uw_hi, const double *Mw, double *vN, cudaStream_t st)
+                     const float *uw_hi, const double *Mw, double *vN, cudaStream_t st, ZeroWords za, ZeroWords zb)
 {
-    if (M == 1) return launch_call_prep_m1(lo, hi, cc, cells, uw_lo, uw_hi, Mw, vN, st);
-    if (M == 4) return launch_call_prep_m4(lo, hi, cc, cells, uw_lo, uw_hi, Mw, vN, st);
-    return launch_call_prep_m6(lo, hi, cc, cells, uw_lo, uw_hi, Mw, vN, st);
+    if (M == 1) return launch_call_prep_m1(lo, hi, cc, cells, uw_lo, uw_hi, Mw, vN, st, za, zb);
+    if (M == 4) return launch_call_prep_m4(lo, hi, cc, cells, uw_lo, uw_hi, Mw, vN, st, za, zb);
+    return launch_call_prep_m6(lo, hi, cc, cells, uw_lo, uw_hi, Mw, vN, st, za, zb);
 }
 int launch_record_prep(int M, const double *vN, const void *gp,
                        const CallConst &cc, const void *cells, int TS, float *recs, PixBox *boxes, double *keys,
@@ -255,6 +255,8 @@ void Workspace::release()
     whist_pending = false;
     if (h_counters) cudaFreeHost(h_counters);
     h_counters = nullptr;
+    if (h_cells) cudaFreeHost(h_cells);
+    h_cells = nullptr;
     for (cudaEvent_t e : evs) cudaEventDestroy(e);
     evs.clear();
 }
@@ -662,7 +664,7 @@ static int enqueue_rest(ar_scene *s, Workspace &ws, const CallConst &cc, int M, 
 // plain: FP64 records and the plain FP64 renderer instead of the FP32 ones.
 static int render_batch(ar_scene *s, Workspace &ws, const CallConst &cc, int M, int TS, int CH, const double *d_lo,
                         const double *d_hi, float *out_lo, float *out_hi, cudaStream_t st, bool profiling,
-                        int batch, ar_render_stats &rs, int &launches, bool plain)
+                        int batch, int max_batches, ar_render_stats &rs, int &launches, bool plain)
 {
     const int W = cc.W, H = cc.H, n_cells = cc.n_cells;
     const uint64_t n_pairs = (uint64_t)n_cells * (uint64_t)s->n;
@@ -676,13 +678,16 @@ static int render_batch(ar_scene *s, Workspace &ws, const CallConst &cc, int M, 
     cudaEvent_t *ev = &ws.evs[kEventsPerBatch * batch];
     NvtxRange batch_range("ar.cell_batch");
     if (profiling) CK(cudaEventRecord(ev[0], st));
-    CK(cudaMemsetAsync(ws.counters.p, 0, sizeof(unsigned long long) * 8, st));
     // the certain drops culled first where the last render found many
     const bool cull = !plain && (s->cull_force >= 0 ? s->cull_force == 1 : ws.cull_on);
     if (cull) RK(ws.clist.ensure(sizeof(uint32_t) * (n_pairs + 1)));
     NvtxRange prep_range("ar.prep: cells and (Gaussian, cell) decisions");
+    // counters start from 0: the record prep's eight for each batch, every
+    // batch's and the histograms with the first
+    const ZeroWords zc{ws.counters.as<uint32_t>(), 2u * (batch ? 8u : 8u + (uint32_t)kCountersPerBatch * (uint32_t)max_batches)};
+    const ZeroWords zh{ws.whist.as<uint32_t>(), batch ? 0u : (uint32_t)kHistWords};
     if (launch_call_prep(M, d_lo, d_hi, cc, ws.cells.p, s->uw_lo, s->uw_hi, s->Mw,
-                         batch == 0 ? ws.vN.as<double>() : nullptr, st))
+                         batch == 0 ? ws.vN.as<double>() : nullptr, st, zc, zh))
         return fail(AR_EDEVICE, "call_prep launch");
     const int rp = plain ? launch_record_prep64(M, ws.vN.as<double>(), s->gp, cc, ws.cells.p, TS,
                                                 ws.recs.as<double>(), ws.boxes.as<PixBox>(), ws.keys.as<double>(),
@@ -1119,24 +1124,39 @@ int render_core(ar_scene *s, Workspace &ws, const ar_intrinsics *in, const ar_no
         CK(cudaEventCreate(&e));
         ws.evs.push_back(e);
     }
-    RK(ws.cells_lohi.ensure(sizeof(double) * 12 * n_cells));
     RK(ws.vN.ensure(sizeof(double) * VN_STRIDE * s->n));
     RK(ws.counters.ensure(sizeof(unsigned long long) * (8 + kCountersPerBatch * max_batches)));
-    {
-        std::vector<double> lohi((size_t)12 * n_cells);
-        for (int c = 0; c < n_cells; ++c)
-            for (int k = 0; k < MAXV; ++k) {
-                lohi[(size_t)MAXV * c + k] = cells[c].lo[k];
-                lohi[(size_t)MAXV * n_cells + (size_t)MAXV * c + k] = cells[c].hi[k];
-            }
-        CK(cudaMemcpyAsync(ws.cells_lohi.p, lohi.data(), sizeof(double) * lohi.size(), cudaMemcpyHostToDevice, st));
-        CK(cudaStreamSynchronize(st));  // the host vector is released on return
-    }
-    const double *d_lo = ws.cells_lohi.as<double>(), *d_hi = d_lo + (size_t)MAXV * n_cells;
     RK(ws.whist.ensure(sizeof(uint32_t) * kHistWords));
     if (!ws.h_whist) CK(cudaMallocHost(&ws.h_whist, sizeof(uint32_t) * kHistWords));
-    CK(cudaMemsetAsync(ws.whist.p, 0, sizeof(uint32_t) * kHistWords, st));
-    CK(cudaMemsetAsync(ws.counters.as<unsigned long long>() + 8, 0, sizeof(unsigned long long) * kCountersPerBatch * max_batches, st));
+    // The cells' bounds.  Up to kPageLockedCells are read by the kernel from
+    // page-locked memory: no copy, and no wait for one before the host's array
+    // may go (every batch waits for its record prep, so the last reader has ended
+    // when a call returns).  With the counters zeroed by the call prep, a render
+    // of 64 Gaussians takes 210 us, 220 before (212 with a copy from page-locked
+    // memory).  More cells are copied.
+    const size_t lohi_words = (size_t)12 * n_cells;
+    std::vector<double> lohi_many;
+    double *lohi;
+    if (n_cells <= kPageLockedCells) {
+        if (!ws.h_cells) CK(cudaMallocHost(&ws.h_cells, sizeof(double) * 12 * kPageLockedCells));
+        lohi = ws.h_cells;
+    } else {
+        lohi_many.resize(lohi_words);
+        lohi = lohi_many.data();
+    }
+    for (int c = 0; c < n_cells; ++c)
+        for (int k = 0; k < MAXV; ++k) {
+            lohi[(size_t)MAXV * c + k] = cells[c].lo[k];
+            lohi[(size_t)MAXV * n_cells + (size_t)MAXV * c + k] = cells[c].hi[k];
+        }
+    const double *d_lo = lohi;
+    if (n_cells > kPageLockedCells) {
+        RK(ws.cells_lohi.ensure(sizeof(double) * lohi_words));
+        CK(cudaMemcpyAsync(ws.cells_lohi.p, lohi, sizeof(double) * lohi_words, cudaMemcpyHostToDevice, st));
+        CK(cudaStreamSynchronize(st));  // the host vector is released on return
+        d_lo = ws.cells_lohi.as<double>();
+    }
+    const double *d_hi = d_lo + (size_t)MAXV * n_cells;
     int launches = 0;
     NvtxRange call_range(plain ? "ar.render_abstract_plain_fp64" : "ar.render_abstract");
     std::vector<std::pair<int, int>> batches;  // (first cell, cells)
@@ -1148,7 +1168,7 @@ int render_core(ar_scene *s, Workspace &ws, const ar_intrinsics *in, const ar_no
         cb.n_cells = nb;
         const size_t off = (size_t)c0 * W * H * 3;
         const int r = render_batch(s, ws, cb, M, TS, CH, d_lo + (size_t)MAXV * c0, d_hi + (size_t)MAXV * c0,
-                                   out_lo + off, out_hi + off, st, profiling, (int)b, rs, launches, plain);
+                                   out_lo + off, out_hi + off, st, profiling, (int)b, max_batches, rs, launches, plain);
         if (r == kSplitBatch) {
             // more tile entries than 32-bit indices reach (its record prep ran,
             // nothing else was enqueued): the batch goes again as two halves

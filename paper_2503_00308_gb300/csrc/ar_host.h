@@ -33,6 +33,7 @@ constexpr size_t kMaxGraphs = 32;  // cached graphs per workspace (least recentl
 // Everything one render needs besides the scene itself.  A scene owns one
 // workspace; a server owns one per slot so that concurrent requests never
 // share buffers.
+constexpr int kPageLockedCells = 4096;  // 400 KB
 struct Workspace {
     DevBuf cells_lohi, cells, vN, recs, boxes, keys, counters;
     DevBuf evk0, evk1, evv0, evv1, ents0, ents1, ente0, ente1;
@@ -55,6 +56,7 @@ struct Workspace {
     DevBuf lvl_lo, lvl_hi;      // one refinement round's union (ar_render_abstract_refined)
     DevBuf wpart;               // partial width sums of the refinement's pieces
     unsigned long long *h_counters = nullptr;  // page-locked
+    double *h_cells = nullptr;                 // page-locked: the bounds of a call's cells, up to kPageLockedCells
     std::vector<cudaEvent_t> evs;              // 9 per cell batch (stage timing)
     int n_batches = 0;                         // cell batches of the last render
     int64_t fallback_prep = 0;                 // MatrixInv fallbacks counted by the record kernel

@@ -62,9 +62,14 @@ struct RenderLaunch {
 
 size_t cell_data_bytes(int M);
 int rec_width(int M);
-// the cells' forms, and (vN non-null) the Gaussians' v and N
+struct ZeroWords {  // n words to be set to 0
+    uint32_t *p = nullptr;
+    uint32_t n = 0;
+};
+// the cells' forms, and (vN non-null) the Gaussians' v and N; za and zb are zeroed
 int launch_call_prep(int M, const double *lo, const double *hi, const CallConst &cc, void *cells, const float *uw_lo,
-                     const float *uw_hi, const double *Mw, double *vN, cudaStream_t st);
+                     const float *uw_hi, const double *Mw, double *vN, cudaStream_t st, ZeroWords za = {},
+                     ZeroWords zb = {});
 // list, count (optional): cull the certain drops first and run the FP64
 // decision chain over the list of the other pairs (cull_kernel)
 int launch_record_prep(int M, const double *vN, const void *gp,

@@ -164,9 +164,9 @@ int ar_render_abstract_noalloc(ar_scene *s, const ar_intrinsics *in, const ar_no
                             n_cells, cudaMemcpyHostToDevice, st));
     NA_CK(cudaMemcpy2DAsync(d_hi, MAXV * sizeof(double), cells[0].hi, sizeof(ar_pose_box), MAXV * sizeof(double),
                             n_cells, cudaMemcpyHostToDevice, st));
-    // the counters keep the previous call's values: clear them
-    NA_CK(cudaMemsetAsync(counters, 0, 8 * sizeof(unsigned long long), st));
-    if (launch_call_prep(M, d_lo, d_hi, cc, cellbuf, s->uw_lo, s->uw_hi, s->Mw, vN, st) ||
+    // the counters keep the previous call's values: cleared with the cells' forms
+    if (launch_call_prep(M, d_lo, d_hi, cc, cellbuf, s->uw_lo, s->uw_hi, s->Mw, vN, st,
+                         ZeroWords{reinterpret_cast<uint32_t *>(counters), 16u}) ||
         launch_record_prep(M, vN, s->gp, cc, cellbuf, TS, recs, boxes, keys, counters, st))
         return set_last_error(AR_EDEVICE, cudaGetErrorString(cudaGetLastError()));
     unsigned long long hc[4] = {0, 0, 0, 0};

@@ -15,11 +15,12 @@ int AR_CAT(rec_scalar_offset_m, AR_M)() { return Rec<AR_M>::SC; }
 
 int AR_CAT(launch_call_prep_m, AR_M)(const double *lo, const double *hi, const CallConst &cc, void *cells,
                                      const float *uw_lo, const float *uw_hi, const double *Mw, double *vN,
-                                     cudaStream_t st)
+                                     cudaStream_t st, ZeroWords za, ZeroWords zb)
 {
     const unsigned cb = (unsigned)((cc.n_cells + CALL_PREP_T / 32 - 1) / (CALL_PREP_T / 32));
     const unsigned gb = vN ? (unsigned)((cc.n_gauss + CALL_PREP_T - 1) / CALL_PREP_T) : 0u;
-    call_prep_kernel<AR_M><<<cb + gb, CALL_PREP_T, 0, st>>>(lo, hi, cc, (CellData<AR_M> *)cells, cb, uw_lo, uw_hi, Mw, vN);
+    call_prep_kernel<AR_M><<<cb + gb, CALL_PREP_T, 0, st>>>(lo, hi, cc, (CellData<AR_M> *)cells, cb, uw_lo, uw_hi, Mw, vN,
+                                                            za, zb);
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
 

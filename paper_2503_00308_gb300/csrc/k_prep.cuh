@@ -265,8 +265,12 @@ template <int M>
 __global__ void __launch_bounds__(CALL_PREP_T) call_prep_kernel(
     const double *__restrict__ cells_lo, const double *__restrict__ cells_hi, CallConst cc,
     CellData<M> *__restrict__ cells, unsigned cell_blocks, const float *__restrict__ uw_lo,
-    const float *__restrict__ uw_hi, const double *__restrict__ Mw, double *__restrict__ vN)
+    const float *__restrict__ uw_hi, const double *__restrict__ Mw, double *__restrict__ vN, ZeroWords za, ZeroWords zb)
 {
+    // the call's counters (they were three memsets, some 2 us each)
+    const uint32_t t0 = blockIdx.x * CALL_PREP_T + threadIdx.x, step = gridDim.x * CALL_PREP_T;
+    for (uint32_t i = t0; i < za.n; i += step) za.p[i] = 0u;
+    for (uint32_t i = t0; i < zb.n; i += step) zb.p[i] = 0u;
     constexpr int ROW = VN_STRIDE + 1;
     __shared__ union {
         CellScratch<M> cell[CALL_PREP_T / 32];
