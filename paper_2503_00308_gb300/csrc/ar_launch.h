@@ -30,6 +30,7 @@ struct RenderLaunch {
     const uint64_t *ev_key;
     int W, H, ntx, n_tiles, n_cells;
     uint64_t n_entries = 0;           // of the segments' full lists
+    uint64_t n_events = 0;            // of all cells
     int64_t n_gauss;
     float k_open;                     // 1 / (1 - largest opacity), rounded up
     float fp64_dev = 3.0e38f;         // opacity evaluations whose FP32 deviation estimate exceeds this

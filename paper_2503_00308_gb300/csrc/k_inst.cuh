@@ -167,7 +167,8 @@ int AR_CAT(launch_record_build_m, AR_M)(const double *vN, const CallConst &cc, c
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const CellData<AR_M> *cd = (const CellData<AR_M> *)cells;
     // the list's length is on the device: a short list is the group builder's,
-    // a long one the one-thread builder's
+    // a long one the one-thread builder's (not launched where the pairs are too few
+    // for one)
     auto coop = record_build_coop_kernel<AR_M>;
     const int coop_smem = (int)sizeof(double) * (COOP_T / 4) * Coop<AR_M>::STRIDE;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, coop, COOP_T, coop_smem) != cudaSuccess || per_sm < 1)
@@ -176,11 +177,13 @@ int AR_CAT(launch_record_build_m, AR_M)(const double *vN, const CallConst &cc, c
     coop<<<sms * per_sm < coop_most ? sms * per_sm : coop_most, COOP_T, coop_smem, st>>>(
         vN, cc.fx, cc.fy, cc.cx, cc.cy, cd, n_gauss, work, count, recs, counters, split_list, split_count);
     if (cudaGetLastError() != cudaSuccess) return 1;
-    auto kern = record_build_kernel<AR_M>;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 128, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
-    kern<<<sms * per_sm, 128, 0, st>>>(vN, cc.fx, cc.fy, cc.cx, cc.cy, cd, n_gauss, work, count, recs, counters,
-                                       split_list, split_count, list_cap, khigh_count);
-    if (cudaGetLastError() != cudaSuccess) return 1;
+    if (list_cap > COOP_MAX) {
+        auto kern = record_build_kernel<AR_M>;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 128, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
+        kern<<<sms * per_sm, 128, 0, st>>>(vN, cc.fx, cc.fy, cc.cx, cc.cy, cd, n_gauss, work, count, recs, counters,
+                                           split_list, split_count, list_cap, khigh_count);
+        if (cudaGetLastError() != cudaSuccess) return 1;
+    }
     // the deferred pairs (the counts stay on the device)
     auto fin = finish_build_kernel<AR_M>;
     const int fin_smem = (int)sizeof(double) * FINISH_GROUPS * Coop<AR_M>::STRIDE;
