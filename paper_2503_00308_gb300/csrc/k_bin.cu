@@ -85,8 +85,7 @@ __global__ void __launch_bounds__(SC_THREADS) scan_sums_kernel(const uint32_t *_
 
 // offs: the block's offset (scanned sums), or (SUMS) the blocks' sums, of which
 // each block adds up those before it: for SC_SUM_BLOCKS blocks at most, that
-// costs less than the launches of a scan of the sums (a small render has ten
-// scans, each some 3 us per launch).
+// costs less than the launches of a scan of the sums (some 3 us each).
 constexpr uint32_t SC_SUM_BLOCKS = 2048;
 template <bool SUMS>
 __global__ void __launch_bounds__(SC_THREADS) scan_apply_kernel(const uint32_t *__restrict__ in, uint32_t n,
