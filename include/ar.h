@@ -368,6 +368,13 @@ int ar_debug_set_prefix(ar_scene *scene, int32_t shift);
  * or another mode. */
 int ar_debug_set_cull(ar_scene *scene, int32_t mode);
 
+/* Test hook: with on = 1, ar_debug_alpha takes every record of its pairs through
+ * the last kernel of the record build as one whose Taylor order exceeds the
+ * default, whatever its order and whether or not MatrixInv holds on the whole
+ * cell (0, the default: as the renderer builds it).  The outputs are the same.
+ * AR_EINVAL for a null scene or on not 0/1. */
+int ar_debug_set_high_order(ar_scene *scene, int32_t on);
+
 /* Test hooks, host only (no CUDA call): the two sizes a scene's next render
  * learns from the sweep statistics of its previous one.
  * ar_debug_learned_prefix: the depth prefix of the first binning phase (each

@@ -82,6 +82,7 @@ def lib():
             "ar_debug_set_entry_cap": ([P, c_int64], ctypes.c_int),
             "ar_debug_set_prefix": ([P, c_int32], ctypes.c_int),
             "ar_debug_set_cull": ([P, c_int32], ctypes.c_int),
+            "ar_debug_set_high_order": ([P, c_int32], ctypes.c_int),
             "ar_debug_learned_prefix": ([P, P, ctypes.c_uint64, ctypes.c_uint64, P], ctypes.c_int),
             "ar_debug_learned_window": ([P, P], ctypes.c_int),
             "ar_bounds_union": ([P, P, ctypes.c_int32, ctypes.c_int32, ctypes.c_int32, P, P, P], ctypes.c_int),
@@ -293,6 +294,10 @@ def ar_debug_set_prefix(scene, shift: int):
 
 def ar_debug_set_cull(scene, mode: int):
     return check(lib().ar_debug_set_cull(scene, int(mode)))
+
+
+def ar_debug_set_high_order(scene, on: bool):
+    return check(lib().ar_debug_set_high_order(scene, 1 if on else 0))
 
 
 def ar_debug_learned_prefix(weights, counts, n_entries: int, n_events: int) -> int:

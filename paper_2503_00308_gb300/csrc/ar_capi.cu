@@ -96,6 +96,20 @@ int launch_record_build_m4(const double *, const CallConst &, const void *, int6
 int launch_record_build_m6(const double *, const CallConst &, const void *, int64_t, const uint32_t *,
                            const uint32_t *, float *, unsigned long long *, uint32_t *, uint32_t *, uint32_t, uint32_t *,
                            cudaStream_t);
+int launch_finish_build_m1(const double *, const CallConst &, const void *, int64_t, const uint32_t *, const uint32_t *,
+                           uint32_t, const uint32_t *, float *, unsigned long long *, cudaStream_t);
+int launch_finish_build_m4(const double *, const CallConst &, const void *, int64_t, const uint32_t *, const uint32_t *,
+                           uint32_t, const uint32_t *, float *, unsigned long long *, cudaStream_t);
+int launch_finish_build_m6(const double *, const CallConst &, const void *, int64_t, const uint32_t *, const uint32_t *,
+                           uint32_t, const uint32_t *, float *, unsigned long long *, cudaStream_t);
+// (the last kernel of launch_record_build, for ar_debug_set_high_order)
+static int launch_finish_build(int M, const double *vN, const CallConst &cc, const void *cells, int64_t n_gauss,
+                               const uint32_t *split_list, const uint32_t *split_count, uint32_t list_cap,
+                               const uint32_t *khigh_count, float *recs, cudaStream_t st)
+{
+    auto f = M == 1 ? launch_finish_build_m1 : (M == 4 ? launch_finish_build_m4 : launch_finish_build_m6);
+    return f(vN, cc, cells, n_gauss, split_list, split_count, list_cap, khigh_count, recs, nullptr, st);
+}
 int launch_debug_alpha_m1(const float *, int, const int64_t *, const int32_t *, const int32_t *, int, float, double *,
                           cudaStream_t);
 int launch_debug_alpha_m4(const float *, int, const int64_t *, const int32_t *, const int32_t *, int, float, double *,
@@ -456,6 +470,14 @@ int ar_debug_set_cull(ar_scene *s, int32_t mode)
     if (!s) return fail(AR_EINVAL, "scene is null");
     if (mode < -1 || mode > 1) return fail(AR_EINVAL, "mode must be -1, 0 or 1");
     s->cull_force = mode;
+    return AR_OK;
+}
+
+int ar_debug_set_high_order(ar_scene *s, int32_t on)
+{
+    if (!s) return fail(AR_EINVAL, "scene is null");
+    if (on != 0 && on != 1) return fail(AR_EINVAL, "on must be 0 or 1");
+    s->debug_high_order = on != 0;
     return AR_OK;
 }
 
@@ -1659,6 +1681,12 @@ int ar_debug_alpha(ar_scene *s, const ar_intrinsics *in, const ar_nominal_pose *
     Workspace &ws = s->ws;
     CallConst cc;
     const int M = call_const(s, in, pose, cell, 1, cc);
+    if (s->debug_high_order) {
+        // every byte 0xff (a NaN) before the decisions are written again, so that a
+        // value part left unwritten shows
+        CK(cudaMemset(ws.recs.p, 0xff, sizeof(float) * rec_width(M) * s->n));
+        RK(ar_debug_records(s, in, pose, cell, nullptr));
+    }
     // the value parts of the listed pairs (cell 0: pair index = Gaussian index);
     // pairs that reach no pixel keep their decision part only
     std::vector<PixBox> boxes((size_t)s->n);
@@ -1689,16 +1717,25 @@ int ar_debug_alpha(ar_scene *s, const ar_intrinsics *in, const ar_nominal_pose *
         return fail(AR_ENOMEM, "debug buffers");
     }
     uint32_t words[8] = {nw, 0, 0, 0, 0, 0, 0, 0};
+    std::vector<uint32_t> high(work.rbegin(), work.rend());  // (that list runs from its back)
+    if (s->debug_high_order &&
+        cudaMemcpy(d_list, high.data(), sizeof(uint32_t) * nw, cudaMemcpyHostToDevice) != cudaSuccess)
+        rc = fail(AR_EDEVICE, "debug copies: %s", cudaGetErrorString(cudaGetLastError()));
     if (cudaMemcpy(d_work, work.data(), sizeof(uint32_t) * nw, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(d_words, words, sizeof words, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(d_gi, gi, sizeof(int64_t) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(d_px, px, sizeof(int32_t) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(d_py, py, sizeof(int32_t) * n, cudaMemcpyHostToDevice) != cudaSuccess)
         rc = fail(AR_EDEVICE, "debug copies: %s", cudaGetErrorString(cudaGetLastError()));
-    if (rc == AR_OK && nw > 0 &&
-        launch_record_build(M, ws.vN.as<double>(), cc, ws.cells.p, s->n, d_work, d_words, ws.recs.as<float>(), nullptr,
-                            d_list, d_words + 3, nw, d_words + 4, 0))
-        rc = fail(AR_EDEVICE, "record build launch: %s", cudaGetErrorString(cudaGetLastError()));
+    if (rc == AR_OK && nw > 0 && s->debug_high_order) {
+        if (launch_finish_build(M, ws.vN.as<double>(), cc, ws.cells.p, s->n, d_list, d_words + 3, nw, d_words,
+                                ws.recs.as<float>(), 0))
+            rc = fail(AR_EDEVICE, "record build launch: %s", cudaGetErrorString(cudaGetLastError()));
+    } else if (rc == AR_OK && nw > 0) {
+        if (launch_record_build(M, ws.vN.as<double>(), cc, ws.cells.p, s->n, d_work, d_words, ws.recs.as<float>(),
+                                nullptr, d_list, d_words + 3, nw, d_words + 4, 0))
+            rc = fail(AR_EDEVICE, "record build launch: %s", cudaGetErrorString(cudaGetLastError()));
+    }
     if (rc == AR_OK &&
         launch_debug_alpha(M, ws.recs.as<float>(), n, d_gi, d_px, d_py, precision, s->fp64_dev, d_out, 0))
         rc = fail(AR_EDEVICE, "debug launch: %s", cudaGetErrorString(cudaGetLastError()));

@@ -92,7 +92,7 @@ constexpr uint32_t F_FALLBACK = 1u;  // MatrixInv failed, even on split pieces: 
 constexpr uint32_t F_STRADDLE = 2u;  // depth may cross the near plane: lower alpha is 0
 constexpr uint32_t F_OPEN = 4u;      // depth-key interval has positive width
 constexpr uint32_t F_SPLIT = 8u;     // MatrixInv held only after splitting the cell (constant Conic)
-constexpr uint32_t F_SPLIT_PENDING = 16u;  // returned by a deferred record build, never stored
+constexpr uint32_t F_SPLIT_PENDING = 16u;  // returned by a deferred record build, never left in a record
 constexpr uint32_t F_KHIGH_PENDING = 32u;  // likewise, for a Taylor order above the default
 
 // doubles per Gaussian of the per-call array vN: v = R_wc (uw - t) as an

@@ -150,6 +150,7 @@ struct ar_scene {
     // culling of the certain drops before the FP64 decision chain: -1 chosen
     // per workspace, 0 off, 1 on; set by ar_debug_set_cull for tests
     int cull_force = -1;
+    bool debug_high_order = false;  // ar_debug_set_high_order
     float fp64_dev = AR_FP64_ALPHA_DEFAULT;  // FP64 re-evaluation threshold (ar_scene_set_fp64_alpha)
     ar_render_stats stats;
     cudaStream_t stats_stream = nullptr;

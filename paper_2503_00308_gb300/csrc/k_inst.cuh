@@ -157,6 +157,25 @@ static int launch_render_fp64_ts(const RenderLaunch &a, cudaStream_t st)
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
 
+// the deferred pairs (the counts stay on the device)
+int AR_CAT(launch_finish_build_m, AR_M)(const double *vN, const CallConst &cc, const void *cells, int64_t n_gauss,
+                                        const uint32_t *split_list, const uint32_t *split_count, uint32_t list_cap,
+                                        const uint32_t *khigh_count, float *recs, unsigned long long *counters,
+                                        cudaStream_t st)
+{
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    auto fin = finish_build_kernel<AR_M>;
+    const int fin_smem = (int)sizeof(double) * FINISH_GROUPS * Coop<AR_M>::STRIDE;
+    if (cudaFuncSetAttribute(fin, cudaFuncAttributeMaxDynamicSharedMemorySize, fin_smem) != cudaSuccess) return 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fin, FINISH_T, fin_smem) != cudaSuccess || per_sm < 1)
+        per_sm = 1;
+    fin<<<sms * per_sm, FINISH_T, fin_smem, st>>>(vN, cc.fx, cc.fy, cc.cx, cc.cy, (const CellData<AR_M> *)cells, n_gauss,
+                                                  split_list, split_count, list_cap, khigh_count, recs, counters);
+    return cudaGetLastError() == cudaSuccess ? 0 : 1;
+}
+
 int AR_CAT(launch_record_build_m, AR_M)(const double *vN, const CallConst &cc, const void *cells, int64_t n_gauss,
                                         const uint32_t *work, const uint32_t *count, float *recs,
                                         unsigned long long *counters, uint32_t *split_list, uint32_t *split_count,
@@ -184,15 +203,8 @@ int AR_CAT(launch_record_build_m, AR_M)(const double *vN, const CallConst &cc, c
                                            split_list, split_count, list_cap, khigh_count);
         if (cudaGetLastError() != cudaSuccess) return 1;
     }
-    // the deferred pairs (the counts stay on the device)
-    auto fin = finish_build_kernel<AR_M>;
-    const int fin_smem = (int)sizeof(double) * FINISH_GROUPS * Coop<AR_M>::STRIDE;
-    if (cudaFuncSetAttribute(fin, cudaFuncAttributeMaxDynamicSharedMemorySize, fin_smem) != cudaSuccess) return 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fin, FINISH_T, fin_smem) != cudaSuccess || per_sm < 1)
-        per_sm = 1;
-    fin<<<sms * per_sm, FINISH_T, fin_smem, st>>>(vN, cc.fx, cc.fy, cc.cx, cc.cy, cd, n_gauss, split_list, split_count,
-                                                  list_cap, khigh_count, recs, counters);
-    return cudaGetLastError() == cudaSuccess ? 0 : 1;
+    return AR_CAT(launch_finish_build_m, AR_M)(vN, cc, cells, n_gauss, split_list, split_count, list_cap, khigh_count,
+                                               recs, counters, st);
 }
 
 int AR_CAT(launch_debug_alpha_m, AR_M)(const float *recs, int n, const int64_t *gi, const int32_t *px,

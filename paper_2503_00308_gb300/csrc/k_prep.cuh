@@ -1639,7 +1639,11 @@ __global__ void __launch_bounds__(128) record_build_kernel(
 // the chain took 192 us for the three pairs of a 10k-Gaussian cell.
 //
 // The pairs whose Taylor order exceeds the default (the back of split_list,
-// khigh_count of them): eight records per warp.
+// khigh_count of them): eight records per warp.  Their cells passed the
+// assertion of Algorithm 3 in record_build_kernel, but coop_matinv evaluates it
+// anew, and two evaluations need not round alike next to RHO_MAX: a pair that it
+// refuses is split by the block that took it, so that no record is left
+// without its W and flags.
 //
 // counters as in record_build_kernel ([0] fallbacks, [2] splits; the pairs were
 // counted as built there).
@@ -1655,11 +1659,13 @@ __global__ void __launch_bounds__(FINISH_T) finish_build_kernel(
     extern __shared__ double s_forms[];
     __shared__ uint64_t s_piece[2][64];
     __shared__ double s_hull[FINISH_T / 32][4][2];
-    __shared__ int s_next, s_failed, s_ok;
+    __shared__ int s_next, s_failed, s_ok, s_pending;
     constexpr unsigned FULL = 0xffffffffu;
     const int tid = threadIdx.x, ln = tid & 31, wp = tid >> 5, q = ln & 3, grp = tid >> 2;
     double *s = s_forms + grp * G::STRIDE;
     uint32_t fb = 0, sp = 0;
+    if (tid == 0) s_pending = 0;
+    __syncthreads();
     // high orders: groups of the last blocks first (the splits take the first)
     const uint32_t nk = *khigh_count, rb = gridDim.x - 1u - blockIdx.x;
     for (uint32_t i0 = (wp * gridDim.x + rb) * 8u; i0 < nk; i0 += gridDim.x * FINISH_GROUPS) {
@@ -1668,14 +1674,35 @@ __global__ void __launch_bounds__(FINISH_T) finish_build_kernel(
         const uint32_t p = list[list_cap - 1u - (act ? i : nk - 1u)];
         const int cell = (int)(p / (uint64_t)n_gauss);
         const int64_t g = (int64_t)p - (int64_t)cell * n_gauss;
-        const uint32_t f = coop_record<M>(s, q, vN + VN_STRIDE * g, fx, fy, cx, cy, cells[cell],
-                                          recs + (size_t)p * RL::WIDTH, act);
-        if (act && q == 0 && (f & F_FALLBACK)) ++fb;
+        float *rec = recs + (size_t)p * RL::WIDTH;
+        const uint32_t f = coop_record<M>(s, q, vN + VN_STRIDE * g, fx, fy, cx, cy, cells[cell], rec, act);
+        if (act && q == 0) {
+            if (f & F_SPLIT_PENDING) {
+                // (its cell was accepted by another evaluation of the assertion)
+                rec_put_flags(rec + RL::FLAGS, f);
+                s_pending = 1;
+            } else if (f & F_FALLBACK) {
+                ++fb;
+            }
+        }
     }
     __syncthreads();
-    const uint32_t ns = *split_count;
-    for (uint32_t i = blockIdx.x; i < ns; i += gridDim.x) {
-        const uint32_t p = list[i];
+    // the splits: this block's high-order pairs that are left with
+    // F_SPLIT_PENDING, if there are any, then its pairs of the split list
+    const uint32_t ns = *split_count, step = gridDim.x * FINISH_GROUPS;
+    const uint32_t own = s_pending ? (nk + step - 1u) / step * FINISH_GROUPS : 0u;
+    for (uint32_t t = 0;; ++t) {
+        uint32_t i, p;
+        if (t < own) {
+            i = (t % FINISH_GROUPS / 8u * gridDim.x + rb) * 8u + t % 8u + t / FINISH_GROUPS * step;
+            if (i >= nk) continue;
+            p = list[list_cap - 1u - i];
+            if (!(__float_as_uint(recs[(size_t)p * RL::WIDTH + RL::FLAGS]) & F_SPLIT_PENDING)) continue;
+        } else {
+            i = blockIdx.x + (t - own) * gridDim.x;
+            if (i >= ns) break;
+            p = list[i];
+        }
         const int cell = (int)(p / (uint64_t)n_gauss);
         const int64_t g = (int64_t)p - (int64_t)cell * n_gauss;
         float *rec = recs + (size_t)p * RL::WIDTH;
@@ -1755,7 +1782,7 @@ __global__ void __launch_bounds__(FINISH_T) finish_build_kernel(
             __syncwarp();
             const bool w_ok = group_all(coop_w<M>(s, q, rec, grp == 0 && whole && conic_ok));
             if (tid == 0) {
-                uint32_t flags = __float_as_uint(rec[RL::FLAGS]);
+                uint32_t flags = __float_as_uint(rec[RL::FLAGS]) & ~F_SPLIT_PENDING;
                 if (whole) flags |= F_SPLIT;
                 if (!whole || !s_ok || !conic_ok || !w_ok) flags |= F_FALLBACK;
                 rec_put_flags(rec + RL::FLAGS, flags);
