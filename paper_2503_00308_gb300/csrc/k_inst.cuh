@@ -1,5 +1,6 @@
 // k_inst.cuh -- instantiation of the per-M kernels; included once per M by
 // k_m1.cu, k_m4.cu, k_m6.cu with AR_M defined.
+#include "ar.h"
 #include "ar_launch.h"
 #include "k_prep.cuh"
 #include "k_render.cuh"
@@ -133,13 +134,14 @@ static int launch_render_ts(const RenderLaunch &a, cudaStream_t st)
 }
 
 // the FP64-capable sweep of the segments listed in a.precise (it stages 16
-// entries at a time whatever the FP32 sweep's chunk is)
-template <int TS, bool REL>
-static int launch_render_fp64_ts(const RenderLaunch &a, cudaStream_t st)
+// entries at a time whatever the FP32 sweep's chunk is), in the form that its
+// items ask for
+template <int TS, bool REL, bool FULL>
+static int launch_render_fp64_form(const RenderLaunch &a, uint32_t full_from, cudaStream_t st)
 {
     constexpr int CH = 16, RING = 4;
-    typedef PreciseSmem<AR_M, CH, RING> SM;
-    auto kern = render_fp64_kernel<AR_M, TS, CH, RING, REL>;
+    typedef PreciseSmem<AR_M, CH, RING, FULL> SM;
+    auto kern = render_fp64_kernel<AR_M, TS, CH, RING, REL, FULL>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SM)) != cudaSuccess) return 1;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
@@ -153,8 +155,20 @@ static int launch_render_fp64_ts(const RenderLaunch &a, cudaStream_t st)
                                        a.precise_first, a.n_precise, a.seg_state, render_parts(TS, a), a.window,
                                        a.round_no, a.next_active, a.n_next, a.precise_mask, a.ent_ev, a.ev_val, a.ev_key,
                                        a.W, a.H, a.ntx, a.n_tiles, a.n_gauss, a.k_open, a.fp64_dev, a.out_lo, a.out_hi,
-                                       a.counters, a.work_fp64);
+                                       a.counters, a.work_fp64, full_from);
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
+}
+
+template <int TS, bool REL>
+static int launch_render_fp64_ts(const RenderLaunch &a, cudaStream_t st)
+{
+    if (!(a.fp64_dev < AR_FP64_ALPHA_DEFAULT)) return launch_render_fp64_form<TS, REL, false>(a, 0u, st);
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const uint32_t full_from = FULL_ITEMS * (uint32_t)sms * PRECISE_CTAS;
+    if (launch_render_fp64_form<TS, REL, false>(a, full_from, st)) return 1;
+    return launch_render_fp64_form<TS, REL, true>(a, full_from, st);
 }
 
 // the deferred pairs (the counts stay on the device)

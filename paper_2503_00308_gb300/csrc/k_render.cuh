@@ -671,6 +671,10 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 
 // pixels per work item of the FP64 sweep
 constexpr int PRECISE_PX = 8;
+// work items per resident CTA, and per listed segment, from which the other form
+// of the FP64 sweep takes them (see render_fp64_kernel)
+constexpr uint32_t FULL_ITEMS = 2, FULL_PER_SEGMENT = 4;
+constexpr int PRECISE_CTAS = 11, FULL_CTAS = 12;  // per SM
 // words per segment of the FP64 sweep's pixel mask
 template <int TS> struct PreciseMask {
     static constexpr int WORDS = TS * TS / 32;
@@ -1094,23 +1098,34 @@ template <int M> __device__ __noinline__ AlphaOut<M> pixel_alpha_again(const flo
 }
 
 // The FP64-capable sweep: the segments and pixels that render_kernel listed,
-// from their start.  A segment lists one pixel or a few, so a warp takes up to
-// PX of them and puts its lanes to their evaluations, which do not
-// depend on one another, instead of to pixels: per chunk of entries,
+// from their start, a warp per CTA, in one of two forms.
+//
+// FULL = false, for segments that list one pixel or a few: a work item is up to PX
+// listed pixels of a segment, and the warp puts its lanes to their evaluations,
+// which do not depend on one another, instead of to pixels: per chunk of entries,
 //   - the (entry, pixel) pairs of the lower endpoints that a pixel's box test
 //     passes are listed, and the records of the entries that any passes staged;
 //   - the pairs are evaluated in FP32, one per lane, into shared memory;
 //   - lane k blends pixel k's entries in order, taking an evaluation in FP64
 //     where the pixel's state asks for it.
-// With a lane per pixel the warp's one or two busy lanes made every evaluation
-// in turn, about a thousand instructions each.  The render stage (both sweeps):
-// 16 cells of 10k Gaussians 0.797 -> 0.731 ms, 32 cells at 400 x 300 3.37 ->
-// 3.14, 64 cells of 300k 48.94 -> 48.34.
-// One warp per CTA; a work item is a listed segment and up to PX of its listed
-// pixels.
-template <int M, int CH, int RING> struct PreciseSmem {
-    static constexpr int PX = PRECISE_PX;
-    static constexpr int PAIRS = CH * PX;
+// FULL = true, where most pixels of most segments are listed: an item is 32 listed
+// pixels, and a lane blends its own and makes their evaluations, FP32 and FP64, itself.
+//
+// Either is bound by its evaluations' FP64 pipe and latency, so by the lanes that make
+// them.  The render stage (both sweeps), FULL form against the other: at the default
+// threshold 16 cells of 10k Gaussians 0.797 / 0.731 ms, 32 cells at 400 x 300 3.37 /
+// 3.14, 64 cells of 300k 48.94 / 48.34; at 1e-5, which lists every pixel, 8 cells of 10k at
+// 400 x 300 5.2 / 9.7 ms, a cell of 300k at 1280 x 720 1.5 / 3.0; at 1e-6, a narrow cell of
+// 300k at 800 x 800 19 / 51.
+// The line, read on the device: full_from items of PX pixels (FULL_ITEMS per resident
+// CTA) and FULL_PER_SEGMENT per segment.  At the default threshold the calls measured
+// (2k to 300k Gaussians, cells of all widths) list up to 7400 segments with three
+// evaluations each or 64 with 24, far from it, so below that threshold only the
+// host launches both forms, one of which takes the items (full_from 0: FULL is not
+// launched).  FULL_CTAS of 14 and 16 (128 registers) took 23 ms on the last.
+template <int M, int CH, int RING, bool FULL> struct PreciseSmem {
+    static constexpr int PX = FULL ? 32 : PRECISE_PX;
+    static constexpr int PAIRS = FULL ? 1 : CH * PX;
     static constexpr int RES = (2 * M + 7 + 3) / 4;  // L.c, U.c, L.k, U.k, rL, rU, alo, ahi, dev as 16-byte vectors
     float rec[CH][Rec<M>::WIDTH];
     float4 res[PAIRS][RES];
@@ -1118,13 +1133,13 @@ template <int M, int CH, int RING> struct PreciseSmem {
     PixBox box[CH];
     EvInfo ev[CH];
     uint32_t rid[RING][PX];
-    float ux[PX], uy[PX];
+    float ux[FULL ? 1 : PX], uy[FULL ? 1 : PX];
     uint32_t redo;                                   // the parts of the tile to sweep again, should the item be abandoned
     uint8_t pair[PAIRS], slot[PAIRS];                // pair i's (entry, pixel) and the inverse
 };
 
-template <int M, int TS, int CH, int RING, bool REL>
-__global__ void __launch_bounds__(32, 11) render_fp64_kernel(
+template <int M, int TS, int CH, int RING, bool REL, bool FULL>
+__global__ void __launch_bounds__(32, FULL ? FULL_CTAS : PRECISE_CTAS) render_fp64_kernel(
     const float *__restrict__ recs, const PixBox *__restrict__ boxes, const uint32_t *__restrict__ seg_start,
     const uint32_t *__restrict__ seg_end, const uint32_t *__restrict__ seg_total,
     const uint32_t *__restrict__ listed, const uint32_t *__restrict__ first_item,
@@ -1133,32 +1148,43 @@ __global__ void __launch_bounds__(32, 11) render_fp64_kernel(
     const uint32_t *__restrict__ precise_mask, const uint32_t *__restrict__ entry_ev, const uint32_t *__restrict__ ev_val,
     const uint64_t *__restrict__ ev_key, int W, int H, int ntx, int n_tiles, int64_t n_gauss,
     float k_open, float fp64_dev, float *__restrict__ out_lo, float *__restrict__ out_hi,
-    unsigned long long *__restrict__ counters, unsigned int *__restrict__ work)
+    unsigned long long *__restrict__ counters, unsigned int *__restrict__ work, uint32_t full_from)
 {
     using RL = Rec<M>;
-    using SM = PreciseSmem<M, CH, RING>;
-    constexpr unsigned FULL = 0xffffffffu;
+    using SM = PreciseSmem<M, CH, RING, FULL>;
+    constexpr unsigned ALL = 0xffffffffu;
     constexpr int PX = SM::PX, NPIX = TS * TS, ROW4 = RL::WIDTH / 4, SC4 = RL::SCW / 4;
     constexpr int PER = SM::PAIRS / 32;  // (entry, pixel) pairs per lane
-    static_assert(CH <= 32 && ROW4 <= 32 && PX == 8, "lane l tests pixel l mod 8");
+    static_assert(CH <= 32 && ROW4 <= 32 && (PX == 8 || FULL), "lane l tests pixel l mod 8");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SM &sm = *reinterpret_cast<SM *>(smem_raw);
     const int ln = threadIdx.x;
     const uint32_t below = (1u << ln) - 1u;
     uint32_t evals = 0, recomp = 0, wide = 0;
-    const uint32_t n_work = (uint32_t)*n_listed, n_seg = (uint32_t)(*n_listed >> 32);
+    uint32_t n_work = (uint32_t)*n_listed;
+    const uint32_t n_seg = (uint32_t)(*n_listed >> 32);
+    if (full_from) {
+        // (both forms are launched: one of them takes the items)
+        if (FULL != (n_work >= full_from && n_work / FULL_PER_SEGMENT >= n_seg)) return;
+        if (FULL) n_work = n_seg * (NPIX / 32);
+    }
     for (;;) {
         uint32_t at = 0;
         if (ln == 0) at = atomicAdd(work, 1u);
-        at = __shfl_sync(FULL, at, 0);
+        at = __shfl_sync(ALL, at, 0);
         if (at >= n_work) break;
-        // the listed segment wk that holds the item: first_item[wk] <= at
-        uint32_t wk = 0;
-        for (uint32_t end = n_seg; end - wk > 1u;) {
-            const uint32_t mid = wk + (end - wk) / 2u;
-            if (first_item[mid] <= at) wk = mid; else end = mid;
+        uint32_t wk = 0, part;
+        if (FULL) {
+            wk = at / (NPIX / 32);
+            part = at % (NPIX / 32);
+        } else {
+            // the listed segment wk that holds the item: first_item[wk] <= at
+            for (uint32_t end = n_seg; end - wk > 1u;) {
+                const uint32_t mid = wk + (end - wk) / 2u;
+                if (first_item[mid] <= at) wk = mid; else end = mid;
+            }
+            part = at - first_item[wk];
         }
-        const uint32_t part = at - first_item[wk];
         const uint32_t seg = listed[wk];
         const uint32_t *pm = precise_mask + (size_t)seg * PreciseMask<TS>::WORDS;
         const int cell = (int)(seg / (uint32_t)n_tiles);
@@ -1176,8 +1202,9 @@ __global__ void __launch_bounds__(32, 11) render_fp64_kernel(
                 rem -= c;
             }
         }
+        if (FULL && !__any_sync(ALL, pid >= 0)) continue;  // past the segment's listed pixels
         // (the warps of a tile are numbered by rows: its first half is the first part)
-        const uint32_t redo = __reduce_or_sync(FULL, pid < 0 ? 0u : 1u << (SEG_DONE + (pid >> 5) * parts / (NPIX / 32)));
+        const uint32_t redo = __reduce_or_sync(ALL, pid < 0 ? 0u : 1u << (SEG_DONE + (pid >> 5) * parts / (NPIX / 32)));
         __syncwarp();
         if (ln == 0) sm.redo = redo;
         const uint32_t b0 = seg_start[seg], b1 = seg_end[seg];
@@ -1209,8 +1236,10 @@ __global__ void __launch_bounds__(32, 11) render_fp64_kernel(
             if (ln < PX) {
 #pragma unroll
                 for (int k = 0; k < RING; ++k) sm.rid[k][ln] = 0xffffffffu;
-                sm.ux[ln] = px + 0.5f;
-                sm.uy[ln] = py + 0.5f;
+                if (!FULL) {
+                    sm.ux[ln] = px + 0.5f;
+                    sm.uy[ln] = py + 0.5f;
+                }
             }
             for (uint32_t base = b0; base < b1 || incomplete; base += CH) {
                 if (!done) {
@@ -1233,7 +1262,7 @@ __global__ void __launch_bounds__(32, 11) render_fp64_kernel(
                         hi_adj = hi_one ? -1.f : ehi2;
                     }
                 }
-                const uint32_t alive = __ballot_sync(FULL, !done);
+                const uint32_t alive = __ballot_sync(ALL, !done);
                 if (alive == 0u) break;
                 const int cnt = base < b1 ? (int)min((uint32_t)CH, b1 - base) : 0;
                 if ((incomplete && base + CH > b1) || base + (uint32_t)cnt - b0 > window) {
@@ -1254,42 +1283,50 @@ __global__ void __launch_bounds__(32, 11) render_fp64_kernel(
                     sm.ev[ln] = EvInfo{rec, bits};
                     sm.box[ln] = box_cell[rec];
                 }
-                const uint32_t uppers = __ballot_sync(FULL, up);
+                const uint32_t uppers = __ballot_sync(ALL, up);
                 __syncwarp();
-                // lane l tests entries (l / 8) + 4 j against pixel l mod 8
                 int n_pairs = 0;
                 uint32_t hits = 0;  // the entries that meet a pixel
-#pragma unroll
-                for (int j = 0; j < PER; ++j) {
-                    const int e = (ln >> 3) + 4 * j;
-                    bool in = false;
-                    if (e < cnt && ((alive >> (ln & 7)) & 1u)) {
+                if constexpr (FULL) {
+                    for (int e = 0; e < cnt; ++e) {
                         const PixBox bx = sm.box[e];
-                        in = px >= bx.x0 && px <= bx.x1 && py >= bx.y0 && py <= bx.y1;
+                        const bool in = !done && px >= bx.x0 && px <= bx.x1 && py >= bx.y0 && py <= bx.y1;
+                        hits |= (__any_sync(ALL, in) ? 1u : 0u) << e;
                     }
-                    const uint32_t m = __ballot_sync(FULL, in);
+                } else {
+                    // lane l tests entries (l / 8) + 4 j against pixel l mod 8
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) hits |= ((m >> (8 * q)) & 255u ? 1u : 0u) << (4 * j + q);
-                    const bool ev = in && !((uppers >> e) & 1u);
-                    const uint32_t mp = __ballot_sync(FULL, ev);
-                    if (ev) {
-                        const int i = n_pairs + __popc(mp & below);
-                        sm.pair[i] = (uint8_t)(e * PX + (ln & 7));
-                        sm.slot[e * PX + (ln & 7)] = (uint8_t)i;
+                    for (int j = 0; j < PER; ++j) {
+                        const int e = (ln >> 3) + 4 * j;
+                        bool in = false;
+                        if (e < cnt && ((alive >> (ln & 7)) & 1u)) {
+                            const PixBox bx = sm.box[e];
+                            in = px >= bx.x0 && px <= bx.x1 && py >= bx.y0 && py <= bx.y1;
+                        }
+                        const uint32_t m = __ballot_sync(ALL, in);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) hits |= ((m >> (8 * q)) & 255u ? 1u : 0u) << (4 * j + q);
+                        const bool ev = in && !((uppers >> e) & 1u);
+                        const uint32_t mp = __ballot_sync(ALL, ev);
+                        if (ev) {
+                            const int i = n_pairs + __popc(mp & below);
+                            sm.pair[i] = (uint8_t)(e * PX + (ln & 7));
+                            sm.slot[e * PX + (ln & 7)] = (uint8_t)i;
+                        }
+                        n_pairs += __popc(mp);
                     }
-                    n_pairs += __popc(mp);
                 }
                 // the whole row for a lower endpoint, its scalars for an upper one
                 for (uint32_t h = hits; h; h &= h - 1u) {
                     const int e = __ffs(h) - 1;
-                    const uint32_t rk = __shfl_sync(FULL, rec, e);
+                    const uint32_t rk = __shfl_sync(ALL, rec, e);
                     const bool upk = (uppers >> e) & 1u;
                     const int at = (upk ? RL::SC : 0) + 4 * ln;
                     if (ln < (upk ? SC4 : ROW4)) cp_async16(&sm.rec[e][at], rec_cell + (size_t)rk * RL::WIDTH + at);
                 }
                 cp_async_wait_all();
                 __syncwarp();
-                for (int i = ln; i < n_pairs; i += 32) {
+                for (int i = ln; !FULL && i < n_pairs; i += 32) {
                     const int c = sm.pair[i];
                     AlphaOut<M> o;
                     pixel_alpha<M>(sm.rec[c / PX], sm.ux[c % PX], sm.uy[c % PX], o);
@@ -1330,7 +1367,9 @@ __global__ void __launch_bounds__(32, 11) render_fp64_kernel(
                     n_open += lower ? 1 : -1;
                     AlphaOut<M> cache;
                     bool have = lower;
-                    if (lower) {
+                    if (FULL && lower) {
+                        pixel_alpha<M>(r, ux, uy, cache);
+                    } else if (lower) {
                         float4 v[SM::RES];
                         const int i = sm.slot[e * PX + ln];
 #pragma unroll
@@ -1458,9 +1497,9 @@ __global__ void __launch_bounds__(32, 11) render_fp64_kernel(
         __syncwarp();
     }
     if (counters) {
-        const uint32_t a = __reduce_add_sync(FULL, evals);
-        const uint32_t b = __reduce_add_sync(FULL, recomp);
-        const uint32_t c = __reduce_add_sync(FULL, wide);
+        const uint32_t a = __reduce_add_sync(ALL, evals);
+        const uint32_t b = __reduce_add_sync(ALL, recomp);
+        const uint32_t c = __reduce_add_sync(ALL, wide);
         if (ln == 0) {
             if (a) atomicAdd(&counters[0], (unsigned long long)a);
             if (b) atomicAdd(&counters[1], (unsigned long long)b);
