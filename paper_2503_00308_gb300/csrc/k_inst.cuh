@@ -83,7 +83,7 @@ int AR_CAT(launch_render_plain_m, AR_M)(int TS, const RenderLaunch &a, cudaStrea
     return TS == 16 ? launch_render_plain_ts<16>(a, st) : launch_render_plain_ts<8>(a, st);
 }
 
-template <int TS, bool REL, int CH, int PARTS>
+template <int TS, bool REL, int CH, int PARTS, int CTAS>
 static int launch_render_parts(const RenderLaunch &a, cudaStream_t st)
 {
     // double-buffered chunks of CH events (16 unless the autotuner picks 8 or
@@ -93,7 +93,7 @@ static int launch_render_parts(const RenderLaunch &a, cudaStream_t st)
     // shared memory small)
     constexpr int RING = 4, NT = Part<TS, PARTS>::NT;
     typedef RenderSmem<AR_M, NT, CH, RING> SM;
-    auto kern = render_kernel<AR_M, TS, CH, RING, REL, PARTS>;
+    auto kern = render_kernel<AR_M, TS, CH, RING, REL, PARTS, CTAS>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::BYTES) != cudaSuccess)
         return 1;
     int dev = 0, sms = 0, per_sm = 0;
@@ -129,8 +129,11 @@ template <int TS, bool REL, int CH = 16>
 static int launch_render_ts(const RenderLaunch &a, cudaStream_t st)
 {
     if constexpr (TS == 16)
-        if (render_parts(TS, a) == 2) return launch_render_parts<TS, REL, CH, 2>(a, st);
-    return launch_render_parts<TS, REL, CH, 1>(a, st);
+        return render_parts(TS, a) == 2 ? launch_render_parts<TS, REL, CH, 2, 4>(a, st)
+                                        : launch_render_parts<TS, REL, CH, 1, 2>(a, st);
+    else
+        return (uint64_t)a.n_cells * (uint64_t)a.n_tiles >= SIX_SEGMENTS ? launch_render_parts<TS, REL, CH, 1, 6>(a, st)
+                                                                         : launch_render_parts<TS, REL, CH, 1, 4>(a, st);
 }
 
 // the FP64-capable sweep of the segments listed in a.precise (it stages 16

@@ -617,20 +617,28 @@ __device__ __forceinline__ float open_ratio_up(float a)
 // themselves, and short lists.  The render stage, whole / halves: 16 narrow
 // cells of the 300k scene 85.6 / 82.6 ms, 64 cells of it 48.3 / 47.0, 32 cells of
 // 10k at 400 x 300 3.14 / 2.99; 36 segments of 200k Gaussians 15.7 / 16.5 ms,
-// 2650 segments of 350 Gaussians 60 / 67 us.
+// 2650 segments of 350 Gaussians 60 / 67 us.  Over scenes of 300 to 60k Gaussians halves
+// take 0.82 to 1.01 of a whole tile's time from 152 segments and 64 entries each on, 1.0 to
+// 1.28 below 32 entries; between 80 and 152 segments of 64 entries 0.83 to 0.96, which
+// the line leaves.
 // (16 warps per SM at 128 registers, a few spills: halves at 168 registers and
 // 12 warps took 88.2 ms on the first.  8 x 8 parts took 86.4, and warps alone,
 // without a barrier but each staging its own records, 88.6.)
-// At tile 8, six CTAs of two warps: unlimited, 225 registers let four fit, and
-// the render stage of 16 cells of 10k Gaussians took 0.73 ms against 0.61.
+// At tile 8, four or six CTAs (of two warps) per SM: at four, 225 registers hold the
+// sweep's state without spills and a segment's chain is faster; at six, the device
+// sweeps more of them at a time.  The render stage, four / six: 1152 segments of 20k
+// Gaussians 4.23 / 4.82 ms, 2500 of 20k 0.83 / 0.95, 2592 of 10k at six variables 1.38 /
+// 1.52, 3888 of 10k 1.01 / 1.04; 4608 of 10k 0.86 / 0.78, 10000 of 10k (4 variables)
+// 0.72 / 0.61, 24000 of 3k 0.57 / 0.45.
 template <int TS, int PARTS> struct Part {
     static constexpr int H = TS / PARTS;  // its rows
     static constexpr int NT = TS * H;     // threads
-    static constexpr int CTAS = TS == 16 ? 2 * PARTS : 6;  // per SM
 };
 // a render takes halves with at least this many segments, and this many entries
 // per segment on average
 constexpr uint64_t HALVES_SEGMENTS = 152, HALVES_ENTRIES = 64;
+// and six CTAs per SM at tile 8 with at least this many
+constexpr uint64_t SIX_SEGMENTS = 4256;
 // Shared-memory layout (dynamic; about 70 KB at six pose variables, 256 threads,
 // chunks of 16 and a ring of 4, so two CTAs fit on an SM):
 //   two buffers, each with the records staged for
@@ -709,8 +717,8 @@ constexpr int SEG_DONE = 8, SEG_LISTED = 16;
 // the masked pixels alone.
 // The decision is per pixel, taken from the pixel's own sweep, so every pixel
 // gets the bounds one FP64-capable sweep would give it.
-template <int M, int TS, int CH, int RING, bool REL, int PARTS>
-__global__ void __launch_bounds__(Part<TS, PARTS>::NT, Part<TS, PARTS>::CTAS) render_kernel(
+template <int M, int TS, int CH, int RING, bool REL, int PARTS, int CTAS>
+__global__ void __launch_bounds__(Part<TS, PARTS>::NT, CTAS) render_kernel(
     const float *__restrict__ recs, const PixBox *__restrict__ boxes, const uint32_t *__restrict__ seg_start,
     const uint32_t *__restrict__ seg_end, const uint32_t *__restrict__ seg_total,
     const uint32_t *__restrict__ cell_ev, const uint32_t *__restrict__ active, const uint32_t *__restrict__ n_active,
