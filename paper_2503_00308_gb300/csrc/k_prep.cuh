@@ -1636,7 +1636,10 @@ __global__ void __launch_bounds__(128) record_build_kernel(
 // matinv_split: each failing piece bisected along its own split_var, down to
 // SPLIT_DEPTH; the hull and the outcome do not depend on the order), and the
 // first group finishes the record.  A warp per pair with every lane repeating
-// the chain took 192 us for the three pairs of a 10k-Gaussian cell.
+// the chain took 192 us for the three pairs of a 10k-Gaussian cell.  Many pairs are
+// bound by the FP64 pipe, so a warp without a piece at a level stays out of it: the build
+// stage with 4292 such pairs among 114684 records takes 4.9 ms, 6.1 where all four
+// warps went through every level (5.8 with a warp per pair).
 //
 // The pairs whose Taylor order exceeds the default (the back of split_list,
 // khigh_count of them): eight records per warp.  Their cells passed the
@@ -1726,7 +1729,8 @@ __global__ void __launch_bounds__(FINISH_T) finish_build_kernel(
         for (int depth = 1; depth <= SPLIT_DEPTH && cnt > 0; ++depth) {
             if (tid == 0) s_next = 0;
             __syncthreads();
-            for (int base = 0; base < cnt; base += FINISH_GROUPS) {
+            // (a warp without a piece leaves the FP64 pipe to the others)
+            for (int base = 0; base + wp * 8 < cnt; base += FINISH_GROUPS) {
                 const bool act = base + grp < cnt;
                 const uint64_t pc = s_piece[cur][act ? base + grp : 0];
                 double ctr[M], h[M];
