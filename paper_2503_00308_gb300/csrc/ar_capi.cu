@@ -78,9 +78,9 @@ int launch_record_prep_m4(const double *, const void *, const CallConst &, const
                           double *, unsigned long long *, cudaStream_t, uint32_t *, uint32_t *);
 int launch_record_prep_m6(const double *, const void *, const CallConst &, const void *, int, float *, PixBox *,
                           double *, unsigned long long *, cudaStream_t, uint32_t *, uint32_t *);
-int launch_render_m1(int, const RenderLaunch &, cudaStream_t);
-int launch_render_m4(int, const RenderLaunch &, cudaStream_t);
-int launch_render_m6(int, const RenderLaunch &, cudaStream_t);
+int launch_render_m1(int, const RenderLaunch &, cudaStream_t, int *);
+int launch_render_m4(int, const RenderLaunch &, cudaStream_t, int *);
+int launch_render_m6(int, const RenderLaunch &, cudaStream_t, int *);
 int launch_record_prep64_m1(const double *, const void *, const CallConst &,
                             const void *, int, double *, PixBox *, double *, unsigned long long *, cudaStream_t);
 int launch_record_prep64_m4(const double *, const void *, const CallConst &,
@@ -89,13 +89,13 @@ int launch_record_prep64_m6(const double *, const void *, const CallConst &,
                             const void *, int, double *, PixBox *, double *, unsigned long long *, cudaStream_t);
 int launch_record_build_m1(const double *, const CallConst &, const void *, int64_t, const uint32_t *,
                            const uint32_t *, float *, unsigned long long *, uint32_t *, uint32_t *, uint32_t, uint32_t *,
-                           cudaStream_t);
+                           cudaStream_t, int *);
 int launch_record_build_m4(const double *, const CallConst &, const void *, int64_t, const uint32_t *,
                            const uint32_t *, float *, unsigned long long *, uint32_t *, uint32_t *, uint32_t, uint32_t *,
-                           cudaStream_t);
+                           cudaStream_t, int *);
 int launch_record_build_m6(const double *, const CallConst &, const void *, int64_t, const uint32_t *,
                            const uint32_t *, float *, unsigned long long *, uint32_t *, uint32_t *, uint32_t, uint32_t *,
-                           cudaStream_t);
+                           cudaStream_t, int *);
 int launch_finish_build_m1(const double *, const CallConst &, const void *, int64_t, const uint32_t *, const uint32_t *,
                            uint32_t, const uint32_t *, float *, unsigned long long *, cudaStream_t);
 int launch_finish_build_m4(const double *, const CallConst &, const void *, int64_t, const uint32_t *, const uint32_t *,
@@ -152,9 +152,10 @@ int launch_record_prep(int M, const double *vN, const void *gp,
     if (M == 4) return launch_record_prep_m4(vN, gp, cc, cells, TS, recs, boxes, keys, counters, st, list, count);
     return launch_record_prep_m6(vN, gp, cc, cells, TS, recs, boxes, keys, counters, st, list, count);
 }
-int launch_render(int M, int TS, const RenderLaunch &a, cudaStream_t st)
+int launch_render(int M, int TS, const RenderLaunch &a, cudaStream_t st, int *launches)
 {
-    return M == 1 ? launch_render_m1(TS, a, st) : (M == 4 ? launch_render_m4(TS, a, st) : launch_render_m6(TS, a, st));
+    auto f = M == 1 ? launch_render_m1 : (M == 4 ? launch_render_m4 : launch_render_m6);
+    return f(TS, a, st, launches);
 }
 int launch_record_prep64(int M, const double *vN, const void *gp,
                          const CallConst &cc, const void *cells, int TS, double *recs, PixBox *boxes, double *keys,
@@ -167,16 +168,16 @@ int launch_record_prep64(int M, const double *vN, const void *gp,
 int launch_record_build(int M, const double *vN, const CallConst &cc, const void *cells, int64_t n_gauss,
                         const uint32_t *work, const uint32_t *count, float *recs, unsigned long long *counters,
                         uint32_t *split_list, uint32_t *split_count, uint32_t list_cap, uint32_t *khigh_count,
-                        cudaStream_t st)
+                        cudaStream_t st, int *launches)
 {
     if (M == 1)
         return launch_record_build_m1(vN, cc, cells, n_gauss, work, count, recs, counters, split_list, split_count,
-                                      list_cap, khigh_count, st);
+                                      list_cap, khigh_count, st, launches);
     if (M == 4)
         return launch_record_build_m4(vN, cc, cells, n_gauss, work, count, recs, counters, split_list, split_count,
-                                      list_cap, khigh_count, st);
+                                      list_cap, khigh_count, st, launches);
     return launch_record_build_m6(vN, cc, cells, n_gauss, work, count, recs, counters, split_list, split_count,
-                                  list_cap, khigh_count, st);
+                                  list_cap, khigh_count, st, launches);
 }
 int launch_render_plain(int M, int TS, const RenderLaunch &a, cudaStream_t st)
 {
@@ -720,7 +721,7 @@ static int render_batch(ar_scene *s, Workspace &ws, const CallConst &cc, int M, 
                                               cull ? ws.clist.as<uint32_t>() : nullptr,
                                               cull ? ws.clist.as<uint32_t>() + n_pairs : nullptr);
     if (rp) return fail(AR_EDEVICE, "record_prep launch: %s", cudaGetErrorString(cudaGetLastError()));
-    launches += 2;
+    launches += cull ? 3 : 2;
     if (profiling) CK(cudaEventRecord(ev[1], st));
     CK(cudaMemcpyAsync(ws.h_counters, ws.counters.p, sizeof(unsigned long long) * 5, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -988,10 +989,10 @@ int run_windowed_render(int M, int TS, RenderLaunch rl, const CallConst &cc, con
         const uint32_t *cur = r == 0 ? rl.seg_order : (r == 1 && round1_order ? round1_order : act[(r - 1) & 1]);
         launch_demand(cur, cur_n, (uint32_t)n_seg, rl.seg_start, rl.seg_end, rl.ent_ev, rl.ev_val, kWindow[r], state,
                       wlist, cnt, st);
+        ++*launches;
         if (launch_record_build(M, vN, cc, cells, rl.n_gauss, wlist, cnt, rl.recs, build_counters, split_list,
-                                cnt + 1, (uint32_t)n_pairs, cnt + 2, st))
+                                cnt + 1, (uint32_t)n_pairs, cnt + 2, st, launches))
             return fail(AR_EDEVICE, "record build launch: %s", cudaGetErrorString(cudaGetLastError()));
-        *launches += 2;
         if (ev) CK(record_stage(ev[2 * r], st));
         rl.active = cur;
         rl.n_active = cur_n;
@@ -1006,10 +1007,9 @@ int run_windowed_render(int M, int TS, RenderLaunch rl, const CallConst &cc, con
         rl.work_fp64 = cnt + 5;
         rl.round_no = r;
         rl.direct = rl.interleave && r == 0;
-        if (launch_render(M, TS, rl, st))
+        if (launch_render(M, TS, rl, st, launches))
             return fail(AR_EDEVICE, "render launch: %s", cudaGetErrorString(cudaGetLastError()));
         if (ev) CK(record_stage(ev[2 * r + 1], st));
-        *launches += 6;
         if (r == 0) {
             // the second binning phase: full lists for the segments that
             // left the first round (a window or their depth prefix ran out)
@@ -1733,7 +1733,7 @@ int ar_debug_alpha(ar_scene *s, const ar_intrinsics *in, const ar_nominal_pose *
             rc = fail(AR_EDEVICE, "record build launch: %s", cudaGetErrorString(cudaGetLastError()));
     } else if (rc == AR_OK && nw > 0) {
         if (launch_record_build(M, ws.vN.as<double>(), cc, ws.cells.p, s->n, d_work, d_words, ws.recs.as<float>(),
-                                nullptr, d_list, d_words + 3, nw, d_words + 4, 0))
+                                nullptr, d_list, d_words + 3, nw, d_words + 4, 0, nullptr))
             rc = fail(AR_EDEVICE, "record build launch: %s", cudaGetErrorString(cudaGetLastError()));
     }
     if (rc == AR_OK &&

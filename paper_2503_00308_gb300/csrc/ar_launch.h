@@ -77,7 +77,7 @@ int launch_record_prep(int M, const double *vN, const void *gp,
                        const CallConst &cc, const void *cells, int TS, float *recs, PixBox *boxes, double *keys,
                        unsigned long long *counters, cudaStream_t st, uint32_t *list = nullptr,
                        uint32_t *count = nullptr);
-int launch_render(int M, int TS, const RenderLaunch &a, cudaStream_t st);
+int launch_render(int M, int TS, const RenderLaunch &a, cudaStream_t st, int *launches);
 int launch_record_prep64(int M, const double *vN, const void *gp,
                          const CallConst &cc, const void *cells, int TS, double *recs, PixBox *boxes, double *keys,
                          unsigned long long *counters, cudaStream_t st);
@@ -95,11 +95,11 @@ int launch_width_partials(const float *lo, const float *hi, int n_cells, size_t 
 // value parts of the records listed in work[0, *count); counters: [0] fallbacks, [1] built, [2] split.
 // split_list (list_cap >= *count entries), split_count and khigh_count (zeroed by the caller): pairs whose
 // MatrixInv fails on the cell, and from the back pairs whose Taylor order exceeds the default, which a last
-// kernel finishes.
+// kernel finishes.  launches (optional) is advanced by the kernels launched.
 int launch_record_build(int M, const double *vN, const CallConst &cc, const void *cells, int64_t n_gauss,
                         const uint32_t *work, const uint32_t *count, float *recs, unsigned long long *counters,
                         uint32_t *split_list, uint32_t *split_count, uint32_t list_cap, uint32_t *khigh_count,
-                        cudaStream_t st);
+                        cudaStream_t st, int *launches);
 // concrete render (k_concrete.cu)
 size_t concrete_pose_bytes();
 int concrete_rec_width();

@@ -140,7 +140,7 @@ static int launch_render_ts(const RenderLaunch &a, cudaStream_t st)
 // entries at a time whatever the FP32 sweep's chunk is), in the form that its
 // items ask for
 template <int TS, bool REL, bool FULL>
-static int launch_render_fp64_form(const RenderLaunch &a, uint32_t full_from, cudaStream_t st)
+static int launch_render_fp64_form(const RenderLaunch &a, uint32_t full_from, cudaStream_t st, int *launches)
 {
     constexpr int CH = 16, RING = 4;
     typedef PreciseSmem<AR_M, CH, RING, FULL> SM;
@@ -159,19 +159,20 @@ static int launch_render_fp64_form(const RenderLaunch &a, uint32_t full_from, cu
                                        a.round_no, a.next_active, a.n_next, a.precise_mask, a.ent_ev, a.ev_val, a.ev_key,
                                        a.W, a.H, a.ntx, a.n_tiles, a.n_gauss, a.k_open, a.fp64_dev, a.out_lo, a.out_hi,
                                        a.counters, a.work_fp64, full_from);
+    ++*launches;
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
 
 template <int TS, bool REL>
-static int launch_render_fp64_ts(const RenderLaunch &a, cudaStream_t st)
+static int launch_render_fp64_ts(const RenderLaunch &a, cudaStream_t st, int *launches)
 {
-    if (!(a.fp64_dev < AR_FP64_ALPHA_DEFAULT)) return launch_render_fp64_form<TS, REL, false>(a, 0u, st);
+    if (!(a.fp64_dev < AR_FP64_ALPHA_DEFAULT)) return launch_render_fp64_form<TS, REL, false>(a, 0u, st, launches);
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const uint32_t full_from = FULL_ITEMS * (uint32_t)sms * PRECISE_CTAS;
-    if (launch_render_fp64_form<TS, REL, false>(a, full_from, st)) return 1;
-    return launch_render_fp64_form<TS, REL, true>(a, full_from, st);
+    if (launch_render_fp64_form<TS, REL, false>(a, full_from, st, launches)) return 1;
+    return launch_render_fp64_form<TS, REL, true>(a, full_from, st, launches);
 }
 
 // the deferred pairs (the counts stay on the device)
@@ -196,7 +197,7 @@ int AR_CAT(launch_finish_build_m, AR_M)(const double *vN, const CallConst &cc, c
 int AR_CAT(launch_record_build_m, AR_M)(const double *vN, const CallConst &cc, const void *cells, int64_t n_gauss,
                                         const uint32_t *work, const uint32_t *count, float *recs,
                                         unsigned long long *counters, uint32_t *split_list, uint32_t *split_count,
-                                        uint32_t list_cap, uint32_t *khigh_count, cudaStream_t st)
+                                        uint32_t list_cap, uint32_t *khigh_count, cudaStream_t st, int *launches)
 {
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
@@ -213,13 +214,16 @@ int AR_CAT(launch_record_build_m, AR_M)(const double *vN, const CallConst &cc, c
     coop<<<sms * per_sm < coop_most ? sms * per_sm : coop_most, COOP_T, coop_smem, st>>>(
         vN, cc.fx, cc.fy, cc.cx, cc.cy, cd, n_gauss, work, count, recs, counters, split_list, split_count);
     if (cudaGetLastError() != cudaSuccess) return 1;
+    int n = 2;
     if (list_cap > COOP_MAX) {
+        ++n;
         auto kern = record_build_kernel<AR_M>;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 128, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
         kern<<<sms * per_sm, 128, 0, st>>>(vN, cc.fx, cc.fy, cc.cx, cc.cy, cd, n_gauss, work, count, recs, counters,
                                            split_list, split_count, list_cap, khigh_count);
         if (cudaGetLastError() != cudaSuccess) return 1;
     }
+    if (launches) *launches += n;
     return AR_CAT(launch_finish_build_m, AR_M)(vN, cc, cells, n_gauss, split_list, split_count, list_cap, khigh_count,
                                                recs, counters, st);
 }
@@ -232,7 +236,7 @@ int AR_CAT(launch_debug_alpha_m, AR_M)(const float *recs, int n, const int64_t *
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
 
-int AR_CAT(launch_render_m, AR_M)(int TS, const RenderLaunch &a, cudaStream_t st)
+int AR_CAT(launch_render_m, AR_M)(int TS, const RenderLaunch &a, cudaStream_t st, int *launches)
 {
     int r;
     if (TS == 8) r = a.rel ? launch_render_ts<8, true>(a, st) : launch_render_ts<8, false>(a, st);
@@ -240,10 +244,12 @@ int AR_CAT(launch_render_m, AR_M)(int TS, const RenderLaunch &a, cudaStream_t st
     else if (a.ch == 32) r = a.rel ? launch_render_ts<16, true, 32>(a, st) : launch_render_ts<16, false, 32>(a, st);
     else r = a.rel ? launch_render_ts<16, true>(a, st) : launch_render_ts<16, false>(a, st);
     if (r) return r;
+    ++*launches;
     // the segments where some pixel met an evaluation needing FP64 (window
     // abandons go to the same next list)
-    if (TS == 8) return a.rel ? launch_render_fp64_ts<8, true>(a, st) : launch_render_fp64_ts<8, false>(a, st);
-    return a.rel ? launch_render_fp64_ts<16, true>(a, st) : launch_render_fp64_ts<16, false>(a, st);
+    if (TS == 8)
+        return a.rel ? launch_render_fp64_ts<8, true>(a, st, launches) : launch_render_fp64_ts<8, false>(a, st, launches);
+    return a.rel ? launch_render_fp64_ts<16, true>(a, st, launches) : launch_render_fp64_ts<16, false>(a, st, launches);
 }
 
 }  // namespace ar
