@@ -455,7 +455,7 @@ int ar_scene_set_fp64_alpha(ar_scene *scene, float threshold);
  * one host synchronisation of a cell batch (which reads how many pairs and
  * tile entries it has, to size its buffers), everything else the batch
  * enqueues -- the binning and the windowed rounds of record build and render,
- * some forty kernels and memsets -- depends on the host only through those
+ * two dozen to a hundred kernels -- depends on the host only through those
  * sizes, the workspace's buffers and the call's parameters.  With graphs on,
  * that phase is captured once per such key (on a private stream, then
  * launched on cuda_stream) and later batches with the same key replay the

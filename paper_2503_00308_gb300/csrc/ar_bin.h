@@ -44,7 +44,7 @@ struct BinOut {
     const uint32_t *ev_val;  // sorted event values: 2 * pair + (upper endpoint)
     const uint32_t *ent_seg; // entries sorted by segment
     const uint32_t *ent_ev;  // entry -> sorted event index
-    const uint32_t *seg_order;  // segments, longest first
+    const uint32_t *seg_order;  // segments, longest first to within an eighth (length_key)
     const uint32_t *seg_total;  // full-list lengths, or null: the lists are complete (seg_end - seg_start)
 };
 
@@ -54,7 +54,7 @@ int run_binning(const BinArgs &a, BinOut &o, cudaStream_t st, int *launches);
 // The second phase: complete lists for the segments active[0, *n_active)
 // (a device count), sorted as run_binning sorts them, in place of the first
 // phase's lists (the other segments' bounds become empty); o.seg_order lists
-// the active segments again, longest first.
+// the active segments again, in the schedule's order.
 int run_rebin(const BinArgs &a, const BinOut &first, const uint32_t *active, const uint32_t *n_active, BinOut &o,
               cudaStream_t st, int *launches);
 

@@ -765,7 +765,7 @@ static int render_batch(ar_scene *s, Workspace &ws, const CallConst &cc, int M, 
     // render) depends on the host only through the sizes read above, so with
     // graphs on it is captured once per sizes, buffers and parameters and
     // replayed as one CUDA graph: a repeated render of the same shape
-    // launches one graph instead of some forty kernels and memsets.
+    // launches one graph instead of two dozen to a hundred kernels.
     std::vector<uint64_t> key;
     if (s->graphs && !plain) {
         const uint64_t head[] = {(uint64_t)M, (uint64_t)TS, (uint64_t)CH, (uint64_t)n_cells, n_pairs, ne, nent, (uint64_t)n_tiles,

@@ -105,7 +105,7 @@ constexpr int VN_STRIDE = VN_ENC + VN_ENC_DOUBLES;
 // Per-Gaussian scene parameters of the abstract render as boxes (Sec. 4.5):
 // opacity o in [o_lo, o_hi], the cutoff exponent tau = 2 ln(255 o) at both
 // ends (-inf below 1/255), and each colour channel in [c_lo, c_hi]; lo = hi
-// without boxes.  (The mean's box enters through v; see pose_prep_kernel.)
+// without boxes.  (The mean's box enters through v; see pose_prep_one.)
 struct GParam {
     double tau_lo, tau_hi;
     float o_lo, o_hi;

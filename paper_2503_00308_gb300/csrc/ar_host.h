@@ -82,7 +82,9 @@ struct TunedTile {
     int W, H, M, TS, CH;  // key (image size, pose variables) -> tile edge, events per staged chunk
 };
 // The FP32 render of one batch in windowed rounds (see render_kernel):
-// demand -> build -> render per round, windows w0, 8192, then unlimited.
+// demand -> build -> render per round, at most three: windows w0, 8192 (w0 again after a
+// two-phase binning), then unlimited; one round where no list is longer than w0, two
+// where the events are few, the second unlimited.
 // state [n_pairs] (zeroed here), wlist [n_pairs], act0/act1 [n_seg], words
 // [kRoundWords] (the rounds' counters, set here by one launch);
 // build_counters: [0] fallbacks, [1] records built, [2] splits (optional);

@@ -55,18 +55,12 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t *s
     return excl;
 }
 
-// The length of a scanned array known on the device only: mul ceil(*p /
-// div) words, at most the host's bound (p null: the host's length).
+// The length of a scanned array known on the device only: *p words, at most the
+// host's bound (p null: the host's length).
 struct DevLen {
     const uint32_t *p = nullptr;
-    uint32_t mul = 1, div = 1;
 };
-__device__ __forceinline__ uint32_t dev_len(DevLen d, uint32_t n)
-{
-    if (!d.p) return n;
-    const uint64_t w = (uint64_t)d.mul * (((uint64_t)*d.p + d.div - 1) / d.div);
-    return w < n ? (uint32_t)w : n;
-}
+__device__ __forceinline__ uint32_t dev_len(DevLen d, uint32_t n) { return d.p && *d.p < n ? *d.p : n; }
 
 __global__ void __launch_bounds__(SC_THREADS) scan_sums_kernel(const uint32_t *__restrict__ in, uint32_t n,
                                                                uint32_t *__restrict__ sums, DevLen dl)
@@ -1220,7 +1214,7 @@ int run_binning(const BinArgs &a, BinOut &o, cudaStream_t st, int *launches)
                                                        a.words + 2);
         prefix_counts_kernel<<<blocks_for(ne, T), T, 0, st>>>(evv, ne, a.boxes, a.TS, a.cell_ev, a.pref_start,
                                                               a.n_cells, a.words + 2, a.u32_a, a.u32_b);
-        const DevLen dl{a.words + 2, 1, 1};
+        const DevLen dl{a.words + 2};
         scan_last_kernel<<<1, 32, 0, st>>>(a.u32_a, ne, a.words, 0, dl);
         exclusive_scan(a.u32_a, a.u32_a, ne, a.scan_tmp, st, launches, dl);
         scan_last_kernel<<<1, 32, 0, st>>>(a.u32_a, ne, a.words, 1, dl);
@@ -1291,7 +1285,7 @@ int run_rebin(const BinArgs &a, const BinOut &first, const uint32_t *active, con
                                                                                       nty + 1, 1);
     // the events' count, or 0 when no segment is active (nothing is then read)
     events_if_active_kernel<<<1, 32, 0, st>>>(n_active, (uint32_t)ne, a.words + 3);
-    const DevLen dl{a.words + 3, 1, 1};
+    const DevLen dl{a.words + 3};
     masked_counts_kernel<<<blocks_for(ne, T), T, 0, st>>>(first.ev_val, ne, a.boxes, a.TS, a.ntx, nty, a.n_gauss,
                                                            a.sat, n_active, a.u32_a);
     scan_last_kernel<<<1, 32, 0, st>>>(a.u32_a, ne, a.words + 1, 0, dl);
@@ -1321,8 +1315,8 @@ int run_rebin(const BinArgs &a, const BinOut &first, const uint32_t *active, con
 }
 
 // ------------------------------------------------------------ windowed rounds
-// every counter of the windowed rounds in one launch (they were fifteen
-// memsets, a tenth of a small render's graph), and the segments' and pairs' states
+// every counter of the windowed rounds in one launch (fifteen memsets are a
+// tenth of a small render's graph), and the segments' and pairs' states
 // (state: 16-byte aligned)
 __global__ void init_rounds_kernel(uint32_t *words, uint32_t n_seg, uint32_t *seg_state, uint32_t *seg_swept,
                                    uint32_t *state, uint64_t n_pairs)

@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(CALL_PREP_T) call_prep_kernel(
     CellData<M> *__restrict__ cells, unsigned cell_blocks, const float *__restrict__ uw_lo,
     const float *__restrict__ uw_hi, const double *__restrict__ Mw, double *__restrict__ vN, ZeroWords za, ZeroWords zb)
 {
-    // the call's counters (they were three memsets, some 2 us each)
+    // the call's counters (a memset each would cost some 2 us)
     const uint32_t t0 = blockIdx.x * CALL_PREP_T + threadIdx.x, step = gridDim.x * CALL_PREP_T;
     for (uint32_t i = t0; i < za.n; i += step) za.p[i] = 0u;
     for (uint32_t i = t0; i < zb.n; i += step) zb.p[i] = 0u;
@@ -448,7 +448,7 @@ static __device__ __noinline__ int screen_fp64(const double (*rd_int)[2], const 
 }
 
 // The enclosures screen_fp32 starts from: the concretised R_delta entries
-// and v - s (enc: the enclosures of v_lo, v_hi, N that pose_prep_kernel
+// and v - s (enc: the enclosures of v_lo, v_hi, N that call_prep_kernel
 // stored)
 template <int M>
 __device__ __forceinline__ void screen_inputs_fp32(const CellData<M> &cd, const float *enc, EI *Ri, EI *vs, bool &ok)

@@ -1,7 +1,7 @@
 // k_render.cuh -- per-pixel effective-opacity relaxation and BlendInd blend.
 //
-// One CTA per (cell, tile), one thread per pixel.  The tile's bin holds the
-// two depth-key endpoints of every (Gaussian, cell) pair whose pixel box meets
+// A CTA takes a (cell, tile) segment or half of one, a thread a pixel (the FP64 sweep: a
+// warp and some of its pixels).  The segment's bin holds the two depth-key endpoints of every (Gaussian, cell) pair whose pixel box meets
 // the tile, sorted by key.  Each pixel sweeps that list once:
 //
 //   lower endpoint of i : effective-opacity bounds of i at this pixel
@@ -694,7 +694,7 @@ template <int TS> struct PreciseMask {
 constexpr int SEG_DONE = 8, SEG_LISTED = 16;
 
 // Persistent grid: each CTA takes work items, (segment, part), from the active
-// list of (cell, tile) segments (longest first in the first round) through an
+// list of (cell, tile) segments (longest first, to within an eighth) through an
 // atomic counter until none are left.
 //
 // Windowed rounds: only the records of the pairs whose lower endpoints lie in
