@@ -51,18 +51,18 @@ def flops_per_triple(M: int) -> int:
 BOOKKEEPING_FLOPS_PER_TRIPLE = 156
 
 
-# DRAM bytes of the render kernel per opacity evaluation, from an ncu capture
+# DRAM bytes of the render kernels per opacity evaluation, from an ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum) of round 0 of the first 4
-# cells of the 300k-Gaussian workload, both instances (FP32 sweep 35.6 MB, FP64
-# re-sweep 15.0 MB), over the render's 73.2M evaluations.  Valid only for the
+# cells of the 300k-Gaussian workload, both sweeps (FP32 36.2 MB, FP64
+# 10.1 MB), over the render's 73.2M evaluations.  Valid only for the
 # kernel sources it was taken from (their SHA-256 below); otherwise the
 # roofline's traffic is reported as null.
-RENDER_TRAFFIC = {"bytes_per_evaluation": (27421952 + 8210688 + 14208256 + 770304) / 73160149,
+RENDER_TRAFFIC = {"bytes_per_evaluation": (28003072 + 8234240 + 10014976 + 48384) / 73160149,
                   # the same capture's smsp__issue_active of the FP32 sweep (the bound of
                   # this issue-limited kernel: one warp instruction per scheduler per cycle)
-                  "issue_active_fp32_sweep": 0.6353,
+                  "issue_active_fp32_sweep": 0.6602,
                   "sources": ["k_render.cuh", "ar_num.cuh", "ar_common.cuh", "k_inst.cuh"],
-                  "sha256": "8c9745917e963b6bda2abd316fbede1feb72bca27086a702d94f1fa9fdf3beea"}
+                  "sha256": "a78d751000028fcd953395acfd3b21c511bdfe8a3c45f65196fb03bd17077264"}
 
 
 def render_capture_valid() -> bool:
