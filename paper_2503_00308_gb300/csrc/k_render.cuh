@@ -620,7 +620,9 @@ __device__ __forceinline__ float open_ratio_up(float a)
 // 2650 segments of 350 Gaussians 60 / 67 us.  Over scenes of 300 to 60k Gaussians halves
 // take 0.82 to 1.01 of a whole tile's time from 152 segments and 64 entries each on, 1.0 to
 // 1.28 below 32 entries; between 80 and 152 segments of 64 entries 0.83 to 0.96, which
-// the line leaves.
+// the line leaves.  In images of less than three tiles a side the middle of the view
+// lies near a corner of four tiles, one half of each of which has most of its work: many cells
+// of an object at 20 x 20 to 40 x 36 take 1.0 to 1.14 by halves, at 48 x 16 to 70 x 38 0.82 to 1.05.
 // (16 warps per SM at 128 registers, a few spills: halves at 168 registers and
 // 12 warps took 88.2 ms on the first.  8 x 8 parts took 86.4, and warps alone,
 // without a barrier but each staging its own records, 88.6.)
@@ -634,9 +636,10 @@ template <int TS, int PARTS> struct Part {
     static constexpr int H = TS / PARTS;  // its rows
     static constexpr int NT = TS * H;     // threads
 };
-// a render takes halves with at least this many segments, and this many entries
-// per segment on average
+// a render takes halves with at least this many segments, this many entries
+// per segment on average and this long a side of the image
 constexpr uint64_t HALVES_SEGMENTS = 152, HALVES_ENTRIES = 64;
+constexpr int HALVES_SIDE = 48;
 // and six CTAs per SM at tile 8 with at least this many
 constexpr uint64_t SIX_SEGMENTS = 4256;
 // Shared-memory layout (dynamic; about 70 KB at six pose variables, 256 threads,
