@@ -680,7 +680,8 @@ static cudaError_t record_stage(cudaEvent_t e, cudaStream_t q)
 
 static int enqueue_rest(ar_scene *s, Workspace &ws, const CallConst &cc, int M, int TS, int CH, float *out_lo, float *out_hi,
                         cudaStream_t q, bool profiling, int batch, cudaEvent_t *ev, uint64_t n_pairs, uint64_t n_seg,
-                        uint64_t ne, uint64_t nent, int ntx, int n_tiles, bool plain, int shift, int &launches);
+                        uint64_t ne, uint64_t nent, bool dense, int ntx, int n_tiles, bool plain, int shift,
+                        int &launches);
 
 // One batch of cells through the whole pipeline.  cc describes the batch
 // (n_cells = cells in the batch, slots shared by every batch of the call).
@@ -745,6 +746,7 @@ static int render_batch(ar_scene *s, Workspace &ws, const CallConst &cc, int M, 
     rs.n_fallback += (int64_t)ws.h_counters[1];
     rs.n_split += (int64_t)ws.h_counters[4];
     rs.n_entries += (int64_t)(nent / 2);
+    const bool dense = dense_boxes(ws.h_counters[0], nent);
     // every buffer of the rest of the batch, sized before any of it is enqueued
     BinOut bo;
     BinArgs sized;
@@ -772,7 +774,7 @@ static int render_batch(ar_scene *s, Workspace &ws, const CallConst &cc, int M, 
                                  (uint64_t)ntx, (uint64_t)W, (uint64_t)H, (uint64_t)s->n, ws.w0,
                                  (uint64_t)s->blend, (uint64_t)float_bits(s->fp64_dev), (uint64_t)float_bits(s->k_open),
                                  (uint64_t)profiling, (uint64_t)ws.interleave, (uint64_t)batch, (uint64_t)(uintptr_t)out_lo,
-                                 (uint64_t)(uintptr_t)out_hi, (uint64_t)(uintptr_t)d_lo, (uint64_t)shift};
+                                 (uint64_t)(uintptr_t)out_hi, (uint64_t)(uintptr_t)d_lo, (uint64_t)shift, (uint64_t)dense};
         key.assign(head, head + sizeof head / sizeof head[0]);
         ws.append_pointers(key);
         for (int k = 0; k < kEventsPerBatch; ++k) key.push_back((uint64_t)(uintptr_t)ev[k]);
@@ -806,7 +808,7 @@ static int render_batch(ar_scene *s, Workspace &ws, const CallConst &cc, int M, 
     }
     const int launches0 = launches;
     const int rc = enqueue_rest(s, ws, cc, M, TS, CH, out_lo, out_hi, q, profiling, batch, ev, n_pairs, n_seg, ne, nent,
-                                ntx, n_tiles, plain, shift, launches);
+                                dense, ntx, n_tiles, plain, shift, launches);
     if (capturing) {
         cudaGraph_t graph = nullptr;
         const cudaError_t e = cudaStreamEndCapture(ws.cap_stream, &graph);
@@ -831,8 +833,8 @@ static int render_batch(ar_scene *s, Workspace &ws, const CallConst &cc, int M, 
         s->graphs = false;
         RK(rc);
         launches = launches0;
-        return enqueue_rest(s, ws, cc, M, TS, CH, out_lo, out_hi, st, profiling, batch, ev, n_pairs, n_seg, ne, nent, ntx,
-                            n_tiles, plain, shift, launches);
+        return enqueue_rest(s, ws, cc, M, TS, CH, out_lo, out_hi, st, profiling, batch, ev, n_pairs, n_seg, ne, nent, dense,
+                            ntx, n_tiles, plain, shift, launches);
     }
     return rc;
 }
@@ -841,7 +843,8 @@ static int render_batch(ar_scene *s, Workspace &ws, const CallConst &cc, int M, 
 // render (windowed rounds, or the plain FP64 renderer), enqueued on q.
 static int enqueue_rest(ar_scene *s, Workspace &ws, const CallConst &cc, int M, int TS, int CH, float *out_lo, float *out_hi,
                         cudaStream_t q, bool profiling, int batch, cudaEvent_t *ev, uint64_t n_pairs, uint64_t n_seg,
-                        uint64_t ne, uint64_t nent, int ntx, int n_tiles, bool plain, int shift, int &launches)
+                        uint64_t ne, uint64_t nent, bool dense, int ntx, int n_tiles, bool plain, int shift,
+                        int &launches)
 {
     const int W = cc.W, H = cc.H, n_cells = cc.n_cells;
     BinOut bo;
@@ -867,6 +870,7 @@ static int enqueue_rest(ar_scene *s, Workspace &ws, const CallConst &cc, int M, 
     rl.W = W; rl.H = H; rl.ntx = ntx; rl.n_tiles = n_tiles; rl.n_cells = n_cells;
     rl.n_entries = nent;
     rl.n_events = ne;
+    rl.dense = dense;
     rl.n_gauss = s->n;
     rl.k_open = s->k_open;
     rl.rel = s->blend == AR_BLEND_RELATIONAL;

@@ -31,6 +31,7 @@ struct RenderLaunch {
     int W, H, ntx, n_tiles, n_cells;
     uint64_t n_entries = 0;           // of the segments' full lists
     uint64_t n_events = 0;            // of all cells
+    bool dense = false;               // (see dense_boxes)
     int64_t n_gauss;
     float k_open;                     // 1 / (1 - largest opacity), rounded up
     float fp64_dev = 3.0e38f;         // opacity evaluations whose FP32 deviation estimate exceeds this
@@ -60,6 +61,13 @@ struct RenderLaunch {
     unsigned long long *n_precise = nullptr;
     unsigned int *work_fp64 = nullptr;
 };
+
+// Whether a screen box holds many pixels of each tile that it meets: DENSE_PX or more
+// on average (triples: pixels in boxes; a box has two entries per tile).  The
+// relational sweep of few segments at six pose variables takes halves of tiles only
+// then (see Part).
+constexpr uint64_t DENSE_PX = 32;
+inline bool dense_boxes(uint64_t n_triples, uint64_t n_entries) { return 2 * n_triples >= DENSE_PX * n_entries; }
 
 size_t cell_data_bytes(int M);
 int rec_width(int M);

@@ -122,10 +122,9 @@ static int launch_render_parts(const RenderLaunch &a, cudaStream_t st)
 static int render_parts(int TS, const RenderLaunch &a)
 {
     const uint64_t n_seg = (uint64_t)a.n_cells * (uint64_t)a.n_tiles;
-    return TS == 16 && n_seg >= HALVES_SEGMENTS && n_seg < (1ull << 30) && a.n_entries >= HALVES_ENTRIES * n_seg &&
-                   (a.W >= HALVES_SIDE || a.H >= HALVES_SIDE)
-               ? 2
-               : 1;
+    if (TS != 16 || n_seg < HALVES_SEGMENTS || n_seg >= (1ull << 30) || a.n_entries < HALVES_ENTRIES * n_seg) return 1;
+    const bool small_rel = a.rel && AR_M > 4 && !a.dense;
+    return (middle_on_edge(a.H) && n_seg < EDGE_SEGMENTS) || (small_rel && n_seg < SMALL_REL_SEGMENTS) ? 1 : 2;
 }
 
 template <int TS, bool REL, int CH = 16>

@@ -620,9 +620,15 @@ __device__ __forceinline__ float open_ratio_up(float a)
 // 2650 segments of 350 Gaussians 60 / 67 us.  Over scenes of 300 to 60k Gaussians halves
 // take 0.82 to 1.01 of a whole tile's time from 152 segments and 64 entries each on, 1.0 to
 // 1.28 below 32 entries; between 80 and 152 segments of 64 entries 0.83 to 0.96, which
-// the line leaves.  In images of less than three tiles a side the middle of the view
-// lies near a corner of four tiles, one half of each of which has most of its work: many cells
-// of an object at 20 x 20 to 40 x 36 take 1.0 to 1.14 by halves, at 48 x 16 to 70 x 38 0.82 to 1.05.
+// the line leaves.  With few segments the halves that have most of the work do not even out.
+// In a low image whose middle row lies near the edge of tiles, one half of each tile there is
+// such: 240 to 660 segments of an object at 32 x 32, 36 x 36, 40 x 30, 48 x 30 and 64 x 64 take
+// 0.9 to 1.14 by halves (640 at 32 x 32, a third wave of whole tiles, 0.77; 96 x 96 0.94 to 1.04),
+// 1024 at 64 x 64 0.95 to 1.05, 1280 to 2690 at 36 x 36, 64 x 64, 83 x 66, 180 x 92 and 104 x 92
+// 0.87 to 1.02; at 39 x 25, 48 x 48, 60 x 50 and 64 x 48 0.82 to 0.97 already 192 to 480.  Relational
+// sweeps at six variables take 1.0 to 1.2 at 240 to 1400 segments of small boxes (less than 14
+// pixels in a tile), 1.01 to 1.08 at 2048, 0.93 to 1.0 at 2376 to 16320; 0.93 to 1.06 with boxes of 14
+// to 45 pixels, 0.89 to 1.02 with larger ones (DENSE_PX).
 // (16 warps per SM at 128 registers, a few spills: halves at 168 registers and
 // 12 warps took 88.2 ms on the first.  8 x 8 parts took 86.4, and warps alone,
 // without a barrier but each staging its own records, 88.6.)
@@ -636,10 +642,14 @@ template <int TS, int PARTS> struct Part {
     static constexpr int H = TS / PARTS;  // its rows
     static constexpr int NT = TS * H;     // threads
 };
-// a render takes halves with at least this many segments, this many entries
-// per segment on average and this long a side of the image
-constexpr uint64_t HALVES_SEGMENTS = 152, HALVES_ENTRIES = 64;
-constexpr int HALVES_SIDE = 48;
+// a render takes halves with at least this many segments and this many entries
+// per segment on average; not with fewer segments than EDGE_SEGMENTS where the image
+// has fewer rows than HALVES_ROWS and its middle lies within three of the edge of a
+// tile, nor with fewer than SMALL_REL_SEGMENTS in the relational sweep at six
+// variables with small boxes
+constexpr uint64_t HALVES_SEGMENTS = 152, HALVES_ENTRIES = 64, EDGE_SEGMENTS = 1216, SMALL_REL_SEGMENTS = 2280;
+constexpr int HALVES_ROWS = 96;
+inline bool middle_on_edge(int H) { return H < HALVES_ROWS && (H % 32 < 6 || H % 32 > 26); }
 // and six CTAs per SM at tile 8 with at least this many
 constexpr uint64_t SIX_SEGMENTS = 4256;
 // Shared-memory layout (dynamic; about 70 KB at six pose variables, 256 threads,
