@@ -57,12 +57,12 @@ BOOKKEEPING_FLOPS_PER_TRIPLE = 156
 # 10.1 MB), over the render's 73.2M evaluations.  Valid only for the
 # kernel sources it was taken from (their SHA-256 below); otherwise the
 # roofline's traffic is reported as null.
-RENDER_TRAFFIC = {"bytes_per_evaluation": (28003072 + 8234240 + 10014976 + 48384) / 73160149,
+RENDER_TRAFFIC = {"bytes_per_evaluation": (27966976 + 7767552 + 10016256 + 47104) / 73160149,
                   # the same capture's smsp__issue_active of the FP32 sweep (the bound of
                   # this issue-limited kernel: one warp instruction per scheduler per cycle)
-                  "issue_active_fp32_sweep": 0.6602,
+                  "issue_active_fp32_sweep": 0.6600,
                   "sources": ["k_render.cuh", "ar_num.cuh", "ar_common.cuh", "k_inst.cuh"],
-                  "sha256": "a78d751000028fcd953395acfd3b21c511bdfe8a3c45f65196fb03bd17077264"}
+                  "sha256": "db2edfb2e8ddf22f7954884673f16f41b9424bd04ad584ca9249d7fb3acb537a"}
 
 
 def render_capture_valid() -> bool:
